@@ -273,16 +273,20 @@ cudaError_t launch_pool_release(const PoolDev& p, const int32_t* ids, int32_t n,
 constexpr uint32_t kMmUnit = 2048;  // bytes of each pair per warp iteration
 
 struct MmPair {
-  const uint8_t* a;
-  const uint8_t* b;
-  uint64_t bytes;       // bytes compared: min of the two lengths
-  uint32_t vec;         // both 16-byte aligned: 16-byte loads
-  uint32_t pad;
+  const uint8_t* a;     // the first 16-byte vector (16-byte aligned)
+  const uint8_t* b;     // the same byte of the second buffer
+  uint64_t n_vec;       // 16-byte vectors from there
+  uint16_t head, tail;  // single bytes before the first vector and after the last
+  uint32_t shift;       // offset of b from a 16-byte boundary
 };
 
-// Pair i owns units [unit_begin[i], unit_begin[i+1]); counts[i] += mismatches.
+// Pair i owns units [unit_begin[i], unit_begin[i+1]) (units of kMmUnit bytes
+// after its head; at least one if it compares any byte).  sums[i] starts at
+// the count to add the mismatches to; counts[i] = the total.  `ticket`: a
+// device word, zero on entry and on exit.
 cudaError_t launch_mismatch(const MmPair* pairs, const uint64_t* unit_begin, int32_t n,
-                            uint64_t units, uint64_t* counts, int sm_count, cudaStream_t stream);
+                            uint64_t units, uint64_t* sums, uint64_t* counts, uint32_t* ticket,
+                            int sm_count, cudaStream_t stream);
 
 // ---- Reads against buffers (pcs_classify_reads) ---------------------------
 // Buffers sorted by start; maxend[i] = max(end[0..i]).

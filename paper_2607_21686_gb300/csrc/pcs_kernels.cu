@@ -229,6 +229,19 @@ __device__ __forceinline__ void st_small(uint8_t* p, uint4 v, int n, bool a4) {
   }
 }
 
+// Bytes [s, s + 16) of the 32 bytes lo : hi (s in [0, 16)): two word selects
+// and four funnel shifts, no branch on s.
+__device__ __forceinline__ uint4 align_bytes(uint4 lo, uint4 hi, uint32_t s) {
+  const bool w2 = s & 8u, w1 = s & 4u;
+  const uint32_t bits = (s & 3u) * 8u;
+  const uint32_t u0 = w2 ? lo.z : lo.x, u1 = w2 ? lo.w : lo.y, u2 = w2 ? hi.x : lo.z,
+                 u3 = w2 ? hi.y : lo.w, u4 = w2 ? hi.z : hi.x, u5 = w2 ? hi.w : hi.y;
+  const uint32_t t0 = w1 ? u1 : u0, t1 = w1 ? u2 : u1, t2 = w1 ? u3 : u2, t3 = w1 ? u4 : u3,
+                 t4 = w1 ? u5 : u4;
+  return make_uint4(__funnelshift_r(t0, t1, bits), __funnelshift_r(t1, t2, bits),
+                    __funnelshift_r(t2, t3, bits), __funnelshift_r(t3, t4, bits));
+}
+
 // Zero the bytes of a segment at or past `n` (n in [1, 16)).
 __device__ __forceinline__ uint4 mask_tail(uint4 v, int n) {
   uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -2704,83 +2717,147 @@ __global__ void __launch_bounds__(kThreads)
 
 // ---------------------------------------------------------------------------
 // Byte-mismatch distance: the count of differing bytes of buffer pairs (the
-// distance D of the discovery procedure at the byte level).  Every block
-// takes 16 KiB tiles of the pairs in turn; 16-byte loads where both buffers
-// are 16-byte aligned, byte loads otherwise.
+// distance D of the discovery procedure at the byte level).
+//
+// Bound by HBM: two reads and no write per byte pair.  A pair is cut along
+// the 16-byte boundaries of its first buffer: `head` single bytes up to the
+// first boundary, then 16-byte vectors in units of 2 KiB, then up to 15 single
+// bytes.  Where the second buffer sits at the same offset from a boundary
+// (buffers carved out of two arenas the same way, or both aligned) its vectors
+// are whole loads too; otherwise each is put together from the two aligned
+// vectors it straddles (the second of which the neighbouring lane also reads,
+// so it comes from L1).  No load reaches outside a buffer: the first and last
+// vectors, whose aligned neighbours would, are compared byte by byte.
+// Measured (calls back to back; the byte loops of a pair off a boundary ->
+// this): 64 pairs of 4 MiB at the same odd offset 455 -> 87 us (6.2 TB/s), at
+// two different ones 455 -> 90 us, aligned 90 -> 87 us; 8 pairs of 256 MiB 3,546
+// -> 601 us (7.1 TB/s) and 618 us; one pair of 100 kB 73 -> 9 us.
 // ---------------------------------------------------------------------------
 
 __device__ __forceinline__ uint32_t bytes_ne(uint32_t x, uint32_t y) {
   return __popc(__vcmpne4(x, y)) >> 3;
 }
+__device__ __forceinline__ uint32_t bytes_ne(uint4 x, uint4 y) {
+  return bytes_ne(x.x, y.x) + bytes_ne(x.y, y.y) + bytes_ne(x.z, y.z) + bytes_ne(x.w, y.w);
+}
 
-// Every warp takes a contiguous range of 2 KiB units of the concatenated
-// pairs, finds the pair of its first unit once and walks forward; its count
-// is reduced across the warp and added to the pair when the pair changes.
+// Vectors [0, left) of a unit (left <= 128), this lane's at a + 512 k, b + 512 k:
+// both sides whole loads.
+__device__ __forceinline__ uint32_t mm_unit(const uint8_t* a, const uint8_t* b, uint32_t left,
+                                            int lane) {
+  uint32_t c = 0;
+  uint4 va[4], vb[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    va[k] = vb[k] = make_uint4(0, 0, 0, 0);
+    if (lane + 32u * k < left) {
+      va[k] = __ldcs(reinterpret_cast<const uint4*>(a + 512 * k));
+      vb[k] = __ldcs(reinterpret_cast<const uint4*>(b + 512 * k));
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) c += bytes_ne(va[k], vb[k]);
+  return c;
+}
+
+// Vectors [from, to) of a unit whose second buffer lies `shift` bytes past a
+// 16-byte boundary: its vector straddles two aligned ones.
+__device__ __forceinline__ uint32_t mm_unit_shift(const uint8_t* a, const uint8_t* b,
+                                                  uint32_t shift, uint32_t from, uint32_t to,
+                                                  int lane) {
+  uint32_t c = 0;
+  uint4 va[4], vb[4], vc[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint32_t x = lane + 32u * k;
+    va[k] = vb[k] = vc[k] = make_uint4(0, 0, 0, 0);
+    if (x >= from && x < to) {
+      va[k] = __ldcs(reinterpret_cast<const uint4*>(a + 512 * k));
+      vb[k] = __ldg(reinterpret_cast<const uint4*>(b - shift + 512 * k));
+      vc[k] = __ldg(reinterpret_cast<const uint4*>(b - shift + 512 * k + 16));
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) c += bytes_ne(va[k], align_bytes(vb[k], vc[k], shift));
+  return c;
+}
+
+// Every warp takes a contiguous range of units of the concatenated pairs,
+// finds the pair of its first unit once and walks forward; its count of each
+// pair is reduced across the warp and added to the pair's sum.  `sums`
+// (scratch) starts at the bytes only one buffer of each pair has; the last
+// block to finish (atomic ticket, zero on entry and on exit) copies it to the
+// caller's counts, which saves a copy between the plan and this launch.
 __global__ void __launch_bounds__(kThreads, 4)
     k_mismatch(const MmPair* __restrict__ pairs, const uint64_t* __restrict__ unit_begin,
-               int32_t n, uint64_t units, uint64_t* counts) {
+               int32_t n, uint64_t units, unsigned long long* sums, uint64_t* counts,
+               uint32_t* ticket) {
+  __shared__ bool s_last;
   const int lane = threadIdx.x & 31;
   const uint64_t warps = static_cast<uint64_t>(gridDim.x) * kWarps;
   const uint64_t w = static_cast<uint64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
-  const uint64_t per = (units + warps - 1) / warps;
-  const uint64_t u0 = w * per;
-  const uint64_t u1 = u0 + per < units ? u0 + per : units;
-  if (u0 >= u1) return;
-  int lo = 0, hi = n - 1;  // the last pair whose first unit is <= u0
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(unit_begin + mid) <= u0) lo = mid;
-    else hi = mid - 1;
-  }
-  int pi = lo;
-  MmPair P = pairs[pi];
-  uint64_t pbeg = __ldg(unit_begin + pi), pend = __ldg(unit_begin + pi + 1);
-  uint32_t c = 0;
-  for (uint64_t u = u0; u < u1; ++u) {
-    if (u >= pend) {
-      const uint32_t tot = __reduce_add_sync(kFull, c);
-      if (lane == 0 && tot)
-        atomicAdd(reinterpret_cast<unsigned long long*>(counts + pi),
-                  static_cast<unsigned long long>(tot));
-      c = 0;
-      do {
-        ++pi;
-        pend = __ldg(unit_begin + pi + 1);
-      } while (u >= pend);
-      P = pairs[pi];
-      pbeg = __ldg(unit_begin + pi);
+  uint64_t u = units * w / warps;
+  const uint64_t u1 = units * (w + 1) / warps;
+  int pi = 0;
+  if (u < u1) {
+    // The last pair whose first unit is <= u (32 probes a round, as in
+    // find_item).
+    for (int span = n; span > 1;) {
+      const int step = (span + 31) >> 5;
+      const int i = pi + lane * step;
+      const bool le = i < pi + span && __ldg(unit_begin + i) <= u;
+      const int last = 31 - __clz(__ballot_sync(kFull, le));  // lane 0 probes pi: never empty
+      pi += last * step;
+      span = min(step, span - last * step);
     }
-    const uint64_t off = (u - pbeg) * kMmUnit;
-    const uint32_t len = static_cast<uint32_t>(P.bytes - off < kMmUnit ? P.bytes - off : kMmUnit);
-    if (P.vec) {
-      const uint4* a = reinterpret_cast<const uint4*>(P.a + off);
-      const uint4* b = reinterpret_cast<const uint4*>(P.b + off);
-      const uint32_t words = len >> 4;
-      uint4 va[4], vb[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t x = lane + 32u * k;
-        if (x < words) {
-          va[k] = __ldcs(a + x);
-          vb[k] = __ldcs(b + x);
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t x = lane + 32u * k;
-        if (x < words)
-          c += bytes_ne(va[k].x, vb[k].x) + bytes_ne(va[k].y, vb[k].y) +
-               bytes_ne(va[k].z, vb[k].z) + bytes_ne(va[k].w, vb[k].w);
-      }
-      for (uint32_t x = (words << 4) + lane; x < len; x += 32) c += P.a[off + x] != P.b[off + x];
+  }
+  for (; u < u1; ++pi) {
+    const uint64_t pbeg = __ldg(unit_begin + pi), pend = __ldg(unit_begin + pi + 1);
+    if (pend <= u) continue;  // nothing of this pair
+    const MmPair P = pairs[pi];
+    const uint64_t x0 = (u - pbeg) * (kMmUnit / 16);  // the first vector here
+    const bool first = u == pbeg, last = u1 >= pend;  // the pair's first / last unit is ours
+    uint32_t whole = static_cast<uint32_t>((last ? pend - 1 : u1) - u);
+    uint32_t left = last ? static_cast<uint32_t>(P.n_vec - (pend - 1 - pbeg) * (kMmUnit / 16)) : 0;
+    const uint8_t* a = P.a + 16 * (x0 + lane);
+    const uint8_t* b = P.b + 16 * (x0 + lane);
+    uint32_t c = 0;
+    if (P.shift == 0) {
+#pragma unroll 1
+      for (; whole; --whole, a += kMmUnit, b += kMmUnit) c += mm_unit(a, b, kMmUnit / 16, lane);
+      if (left) c += mm_unit(a, b, left, lane);
     } else {
-      for (uint32_t x = lane; x < len; x += 32) c += P.a[off + x] != P.b[off + x];
+      // The aligned neighbours of the pair's first and last vectors may lie
+      // outside the buffer: those two are compared byte by byte.
+      uint32_t from = first ? 1 : 0;
+#pragma unroll 1
+      for (; whole; --whole, a += kMmUnit, b += kMmUnit) {
+        c += mm_unit_shift(a, b, P.shift, from, kMmUnit / 16, lane);
+        from = 0;
+      }
+      if (left) c += mm_unit_shift(a, b, P.shift, from, left - 1, lane);
+      if (lane < 16 ? (first && P.n_vec > 0) : (last && P.n_vec > 1)) {
+        const uint64_t at = (lane < 16 ? 0 : 16 * (P.n_vec - 1)) + (lane & 15);
+        c += P.a[at] != P.b[at];
+      }
     }
+    // The single bytes before the first vector and after the last.
+    if (first && lane < static_cast<int>(P.head))
+      c += (P.a - P.head)[lane] != (P.b - P.head)[lane];
+    if (last && lane < static_cast<int>(P.tail))
+      c += P.a[16 * P.n_vec + lane] != P.b[16 * P.n_vec + lane];
+    const uint32_t tot = __reduce_add_sync(kFull, c);
+    if (lane == 0 && tot) atomicAdd(sums + pi, static_cast<unsigned long long>(tot));
+    u = last ? pend : u1;
   }
-  const uint32_t tot = __reduce_add_sync(kFull, c);
-  if (lane == 0 && tot)
-    atomicAdd(reinterpret_cast<unsigned long long*>(counts + pi),
-              static_cast<unsigned long long>(tot));
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int i = threadIdx.x; i < n; i += kThreads) counts[i] = __ldcg(sums + i);
+  if (threadIdx.x == 0) *ticket = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -3180,13 +3257,18 @@ cudaError_t launch_pool_cow(const PoolDev& p, int32_t* table, int64_t n_table,
 }
 
 cudaError_t launch_mismatch(const MmPair* pairs, const uint64_t* unit_begin, int32_t n,
-                            uint64_t units, uint64_t* counts, int sm_count, cudaStream_t stream) {
-  if (units == 0 || n <= 0) return cudaSuccess;
-  // One resident wave (four blocks per SM), at least eight units per warp.
-  const uint64_t want = (units + 8 * kWarps - 1) / (8 * kWarps);
-  const uint64_t cap = static_cast<uint64_t>(sm_count) * 4;
+                            uint64_t units, uint64_t* sums, uint64_t* counts, uint32_t* ticket,
+                            int sm_count, cudaStream_t stream) {
+  if (units == 0 || n <= 0) return cudaErrorInvalidValue;
+  // One resident wave; a unit per warp until that wave is full, as each
+  // further unit of a warp adds a memory round trip to a small call (18 pairs
+  // of 64 KiB: 15.4 us with at least eight units a warp and the counts copied
+  // by a launch of their own, 10.1 us so).
+  const uint64_t want = (units + kWarps - 1) / kWarps;
+  const uint64_t cap = static_cast<uint64_t>(sm_count) *
+                       resident_blocks(reinterpret_cast<const void*>(k_mismatch));
   k_mismatch<<<static_cast<unsigned>(want < cap ? want : cap), kThreads, 0, stream>>>(
-      pairs, unit_begin, n, units, counts);
+      pairs, unit_begin, n, units, reinterpret_cast<unsigned long long*>(sums), counts, ticket);
   return cudaGetLastError();
 }
 

@@ -2870,13 +2870,18 @@ pcs_status pcs_mismatch(pcs_ctx* c, const pcs_buf* a, const pcs_buf* b, int32_t 
   for (int i = 0; i < n; ++i) {
     const uint64_t m = std::min(a[i].bytes, b[i].bytes);
     if (m > 0 && (!a[i].ptr || !b[i].ptr)) return fail(PCS_E_INVAL, "pair %d: null buffer", i);
-    pairs[i].a = static_cast<const uint8_t*>(a[i].ptr);
-    pairs[i].b = static_cast<const uint8_t*>(b[i].ptr);
-    pairs[i].bytes = m;
-    pairs[i].vec = aligned16(a[i].ptr) && aligned16(b[i].ptr);
+    const uint64_t head =
+        std::min<uint64_t>((16 - (reinterpret_cast<uintptr_t>(a[i].ptr) & 15)) & 15, m);
+    MmPair& p = pairs[i];
+    p.a = static_cast<const uint8_t*>(a[i].ptr) + head;
+    p.b = static_cast<const uint8_t*>(b[i].ptr) + head;
+    p.n_vec = (m - head) / 16;
+    p.head = static_cast<uint16_t>(head);
+    p.tail = static_cast<uint16_t>((m - head) % 16);
+    p.shift = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.b) & 15);
     extra[i] = std::max(a[i].bytes, b[i].bytes) - m;
     tb[i] = tiles;
-    tiles += (m + kMmUnit - 1) / kMmUnit;
+    if (m > 0) tiles += std::max<uint64_t>((16 * p.n_vec + kMmUnit - 1) / kMmUnit, 1);
   }
   tb[n] = tiles;
   std::lock_guard<std::mutex> lk(c->mu);
@@ -2894,11 +2899,13 @@ pcs_status pcs_mismatch(pcs_ctx* c, const pcs_buf* a, const pcs_buf* b, int32_t 
   put(c->plan, o_ex, extra);
   PCS_CUDA(plan_copy(c, ws, total, stream));
   // Counts start at the bytes only one buffer has.
-  PCS_CUDA(cudaMemcpyAsync(counts, ws + o_ex, 8ull * n, cudaMemcpyDeviceToDevice, stream));
-  {
+  if (tiles == 0) {
+    PCS_CUDA(cudaMemcpyAsync(counts, ws + o_ex, 8ull * n, cudaMemcpyDeviceToDevice, stream));
+  } else {
     LaunchScope ls(c, kKMismatch, stream);
     PCS_CUDA(launch_mismatch(reinterpret_cast<const MmPair*>(ws),
-                             reinterpret_cast<const uint64_t*>(ws + o_tb), n, tiles, counts,
+                             reinterpret_cast<const uint64_t*>(ws + o_tb), n, tiles,
+                             reinterpret_cast<uint64_t*>(ws + o_ex), counts, c->call_words,
                              c->sm_count, stream));
   }
   return ws_release(c, stream);
