@@ -289,16 +289,22 @@ cudaError_t launch_mismatch(const MmPair* pairs, const uint64_t* unit_begin, int
                             int sm_count, cudaStream_t stream);
 
 // ---- Reads against buffers (pcs_classify_reads) ---------------------------
-// Buffers sorted by start; maxend[i] = max(end[0..i]).
+// The non-empty buffers sorted by start; maxend[i] = max(end[0..i]).
 struct ReadPlan {
   const uint64_t* start;
   const uint64_t* end;
   const uint64_t* maxend;
-  const uint32_t* orig;   // caller index of each sorted buffer
-  int32_t n;
-  int32_t pad;
+  const uint32_t* orig;   // [n_all] caller index of each buffer: the sorted ones, then the empty
+  uint32_t* bitmap;       // [ceil(n / 32)] device words, zero on entry
+  uint32_t* ticket;       // a device word, zero on entry and on exit
+  int32_t n;              // non-empty buffers (at least 1)
+  int32_t n_all;
+  uint64_t base, top;     // the first start and the largest end
+  int32_t slices;         // set by the launcher: slices of the address range
+  int32_t slice_shift;    // and log2 of their bytes
 };
-cudaError_t launch_classify_reads(const ReadPlan& p, const uint64_t* addr, const uint64_t* bytes,
+// flags[i] = a read overlaps buffer i; every flag is written.  m > 0.
+cudaError_t launch_classify_reads(ReadPlan p, const uint64_t* addr, const uint64_t* bytes,
                                   int64_t m, uint8_t* flags, int sm_count, cudaStream_t stream);
 
 // Occupancy of the streaming kernel (blocks per SM) for the launch shape.

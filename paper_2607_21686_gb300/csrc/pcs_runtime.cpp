@@ -2919,14 +2919,17 @@ pcs_status pcs_classify_reads(pcs_ctx* c, const pcs_buf* bufs, int32_t n, const 
   if (n == 0) return PCS_OK;
   if (n > 0x7FFFFFFF - 1) return fail(PCS_E_INVAL, "too many buffers");
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+  // The non-empty buffers by start (ties in the caller's order), then the
+  // empty ones, which no read overlaps.
   std::vector<uint32_t> ord(n);
-  for (int i = 0; i < n; ++i) ord[i] = static_cast<uint32_t>(i);
+  int nn = 0, empty = n;
+  for (int i = 0; i < n; ++i) ord[bufs[i].bytes ? nn++ : --empty] = static_cast<uint32_t>(i);
   auto start_of = [&](uint32_t i) { return reinterpret_cast<uint64_t>(bufs[i].ptr); };
-  std::stable_sort(ord.begin(), ord.end(),
+  std::stable_sort(ord.begin(), ord.begin() + nn,
                    [&](uint32_t x, uint32_t y) { return start_of(x) < start_of(y); });
-  std::vector<uint64_t> st_(n), en(n), mx(n);
+  std::vector<uint64_t> st_(nn), en(nn), mx(nn);
   uint64_t run = 0;
-  for (int k = 0; k < n; ++k) {
+  for (int k = 0; k < nn; ++k) {
     const uint64_t b0 = start_of(ord[k]);
     const uint64_t len = bufs[ord[k]].bytes;
     st_[k] = b0;
@@ -2937,8 +2940,13 @@ pcs_status pcs_classify_reads(pcs_ctx* c, const pcs_buf* bufs, int32_t n, const 
   std::lock_guard<std::mutex> lk(c->mu);
   pcs_status st = set_device(c);
   if (st) return st;
-  const uint64_t o_en = round_up(8ull * n, 256), o_mx = round_up(o_en + 8ull * n, 256);
-  const uint64_t o_or = round_up(o_mx + 8ull * n, 256), total = o_or + 4ull * n;
+  if (nn == 0 || m == 0) {  // nothing can be read
+    PCS_CUDA(cudaMemsetAsync(flags, 0, n, stream));
+    return PCS_OK;
+  }
+  const uint64_t o_en = round_up(8ull * nn, 256), o_mx = round_up(o_en + 8ull * nn, 256);
+  const uint64_t o_or = round_up(o_mx + 8ull * nn, 256), o_bm = round_up(o_or + 4ull * n, 256);
+  const uint64_t total = o_bm + 4ull * ((nn + 31) / 32);
   uint8_t* ws = nullptr;
   st = ws_acquire(c, total, stream, &ws);
   if (st) return st;
@@ -2948,14 +2956,18 @@ pcs_status pcs_classify_reads(pcs_ctx* c, const pcs_buf* bufs, int32_t n, const 
   put(c->plan, o_mx, mx);
   put(c->plan, o_or, ord);
   PCS_CUDA(plan_copy(c, ws, total, stream));
-  PCS_CUDA(cudaMemsetAsync(flags, 0, n, stream));
   ReadPlan rp{};
   rp.start = reinterpret_cast<const uint64_t*>(ws);
   rp.end = reinterpret_cast<const uint64_t*>(ws + o_en);
   rp.maxend = reinterpret_cast<const uint64_t*>(ws + o_mx);
   rp.orig = reinterpret_cast<const uint32_t*>(ws + o_or);
-  rp.n = n;
-  if (m > 0) {
+  rp.bitmap = reinterpret_cast<uint32_t*>(ws + o_bm);
+  rp.ticket = c->call_words;
+  rp.n = nn;
+  rp.n_all = n;
+  rp.base = st_[0];
+  rp.top = mx[nn - 1];
+  {
     LaunchScope ls(c, kKClassifyReads, stream);
     PCS_CUDA(launch_classify_reads(rp, addr, bytes, m, flags, c->sm_count, stream));
   }

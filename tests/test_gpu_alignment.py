@@ -40,3 +40,39 @@ def test_mismatch_of_offset_pairs(ctx, dev, oa):
             assert want[-1] == oracle.mismatch(ha[oa:oa + n].numpy(), hb.numpy())
     assert ctx.mismatch(a, b).cpu().tolist() == want
     assert ctx.mismatch(a, b).cpu().tolist() == want  # the scratch sums start over
+
+
+def _read_flags(spans, ro, rn):
+    """1 for each (start, bytes) some read [ro, ro + rn) of at least one byte overlaps."""
+    ro, rn = ro[rn > 0], rn[rn > 0]
+    return [int(n > 0 and bool(((ro < o + n) & (ro + rn > o)).any())) for o, n in spans]
+
+
+# Buffers: one; few and many staged in shared memory; the most staged and one
+# more.  Reads: below and above the line where the address table is used.
+@pytest.mark.parametrize("n,m", [(1, 40), (33, 3_000_001), (600, 2_600_000), (4096, 2_500_000),
+                                 (4096, 5000), (4097, 5000)])
+def test_classify_reads_paths(ctx, dev, n, m):
+    rnd = np.random.default_rng(n + m)
+    size = 1 << 26
+    space = torch.empty(size, dtype=torch.uint8, device=dev)
+    start = rnd.integers(0, size // 2, n)
+    length = np.minimum(np.exp(rnd.uniform(0, 16, n)).astype(np.int64), size - start)
+    length[rnd.random(n) < 0.1] = 0          # empty buffers
+    length[0] = max(length[0], 1)
+    # Reads around a few places, before the first buffer and after the last.
+    at = rnd.integers(0, size // 2, 12)
+    ro = (at[rnd.integers(0, 12, m)] + rnd.integers(-2000, 2000, m)).clip(0, size - 1)
+    ro[:: 5] = size - 1 - rnd.integers(0, 1000, len(ro[:: 5]))
+    rn = rnd.integers(0, 200, m)
+    rn[:: 1001] = 0
+    base = space.data_ptr()
+    addr = torch.from_numpy(base + ro).to(dev)
+    flags = torch.full((n,), 7, dtype=torch.uint8, device=dev)
+    bufs = [space[o:o + k] for o, k in zip(start.tolist(), length.tolist())]
+    ctx.classify_reads(bufs, addr, torch.from_numpy(rn).to(dev), flags)
+    pick = rnd.permutation(n)[:150].tolist() if m > 100000 else range(n)
+    got = flags.cpu().tolist()
+    spans = list(zip(start.tolist(), length.tolist()))
+    assert set(got) <= {0, 1}
+    assert [got[i] for i in pick] == _read_flags([spans[i] for i in pick], ro, rn)
