@@ -1,12 +1,13 @@
 // pcs_kernels.cu -- sm_103a kernels of the PCS hot path.
 //
-// k_stream<MODE>  one pass over 4 KiB chunks of many byte streams: a warp owns
-//                 a task of 2^g chunks; lane l moves the 16-byte segments
-//                 l + 32k of each chunk (every warp access is 512 contiguous
-//                 bytes), optionally gathers / scatters them through a row or
-//                 paged-ring layout, and folds them into the PCSFP64-v1 lane
-//                 chain; a shuffle tree makes the chunk hash and then the
-//                 task's aligned-group node (Sec. 4 FINGERPRINT, step 1).
+// k_stream<MODE>  one pass over 4 KiB chunks of many byte streams: a warp walks
+//                 a range of tasks of one or two chunks; lane l moves the
+//                 16-byte segments l + 32k of each chunk (every warp access is
+//                 512 contiguous bytes), puts them together from the aligned
+//                 vectors of a buffer off a 16-byte boundary or gathers /
+//                 scatters them through a row or paged-ring layout, and folds
+//                 them into the PCSFP64-v1 lane chain; a shuffle tree makes
+//                 the task's node (Sec. 4 FINGERPRINT, step 1).
 // k_bulk<MODE>    the moving passes (pack, restore) of aligned streams: per-warp
 //                 TMA pipelines of 8 KiB tiles through shared memory, the
 //                 fingerprint of each tile fused into the copy
@@ -215,20 +216,6 @@ __device__ __forceinline__ uint4 ld_small(const uint8_t* p, int n, bool a4) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-__device__ __forceinline__ void st_small(uint8_t* p, uint4 v, int n, bool a4) {
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (a4 && 4 * j + 4 <= n) {
-      *reinterpret_cast<uint32_t*>(p + 4 * j) = w[j];
-    } else {
-#pragma unroll
-      for (int b = 0; b < 4; ++b)
-        if (4 * j + b < n) p[4 * j + b] = static_cast<uint8_t>(w[j] >> (8 * b));
-    }
-  }
-}
-
 // Bytes [s, s + 16) of the 32 bytes lo : hi (s in [0, 16)): two word selects
 // and four funnel shifts, no branch on s.
 __device__ __forceinline__ uint4 align_bytes(uint4 lo, uint4 hi, uint32_t s) {
@@ -295,47 +282,221 @@ struct ModeTraits {
   static constexpr bool kStore = MODE != kModeHash;
 };
 
-// Load segment `off` of a stream from its read side.
-template <int MODE>
-__device__ __forceinline__ uint4 load_seg(const SecDesc& s, uint64_t off, uint32_t* err) {
-  const uint4 z = make_uint4(0, 0, 0, 0);
-  if (off >= s.bytes) return z;
-  if (ModeTraits<MODE>::kLoadLayout) {
-    if (s.layout == kContig) {
-      const uint64_t left = s.bytes - off;
-      if (left >= 16 && s.align == 16) return ld_stream(s.lbase + off);
-      return ld_small(s.lbase + off, left < 16 ? static_cast<int>(left) : 16, s.align >= 4);
+// Bytes of the aligned 16-byte vector at `p` that lie in logical bytes [0, L)
+// when its first byte is logical byte `off` (negative before the buffer); the
+// rest 0.  Words wholly inside are loaded as words.
+__device__ __forceinline__ uint4 ld_edge(const uint8_t* p, int64_t off, int64_t L) {
+  const int from = off < 0 ? static_cast<int>(-off) : 0;                  // bytes [from, to)
+  const int to = L - off < 16 ? static_cast<int>(L - off) : 16;
+  uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (4 * j >= from && 4 * j + 4 <= to) {
+      w[j] = *reinterpret_cast<const uint32_t*>(p + 4 * j);
+    } else if (4 * j + 4 > from && 4 * j < to) {
+#pragma unroll
+      for (int b = 4 * j; b < 4 * j + 4; ++b)
+        if (b >= from && b < to) w[j] |= static_cast<uint32_t>(p[b]) << (8 * (b & 3));
     }
-    const uint8_t* p = row_addr(s, off, err);
-    return p ? ld_stream(p) : z;
-  } else {
-    // Payload inside a record: padded to 256 bytes, so a whole segment is
-    // readable; bytes past the logical end are masked to zero.
-    uint4 v = ld_stream(s.payload + off);
-    const uint64_t left = s.bytes - off;
-    if (left < 16) v = mask_tail(v, static_cast<int>(left));
-    return v;
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Store the bytes of `v` that lie in logical bytes [0, L).
+__device__ __forceinline__ void st_edge(uint8_t* p, uint4 v, int64_t off, int64_t L) {
+  const int from = off < 0 ? static_cast<int>(-off) : 0;
+  const int to = L - off < 16 ? static_cast<int>(L - off) : 16;
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (4 * j >= from && 4 * j + 4 <= to) {
+      *reinterpret_cast<uint32_t*>(p + 4 * j) = w[j];
+    } else if (4 * j + 4 > from && 4 * j < to) {
+#pragma unroll
+      for (int b = 4 * j; b < 4 * j + 4; ++b)
+        if (b >= from && b < to) p[b] = static_cast<uint8_t>(w[j] >> (8 * (b & 3)));
+    }
   }
 }
 
-// Store segment `off` to a stream's write side.
-template <int MODE>
-__device__ __forceinline__ void store_seg(const SecDesc& s, uint64_t off, uint4 v, uint32_t* err) {
-  if (MODE == kModePack) {
-    // Record payload: write through the 256-byte padding (zeros past L).
-    const uint64_t padded = (s.bytes + kRecordAlign - 1) / kRecordAlign * kRecordAlign;
-    if (off < padded) st_stream(s.payload + off, v);
-  } else if (MODE == kModeRestore || MODE == kModeRestoreV) {
-    if (off >= s.bytes) return;
-    if (s.layout == kContig) {
-      const uint64_t left = s.bytes - off;
-      if (left >= 16 && s.align == 16) st_stream(s.lbase + off, v);
-      else st_small(s.lbase + off, v, left < 16 ? static_cast<int>(left) : 16, s.align >= 4);
-      return;
+// The value of the next (prev) lane; lane 31 (0) gets lane 0's (31's) `wrap`.
+__device__ __forceinline__ uint4 from_next_lane(uint4 v, uint4 wrap, int lane) {
+  const uint4 x = lane == 0 ? wrap : v;
+  const int src = (lane + 1) & 31;
+  return make_uint4(__shfl_sync(kFull, x.x, src), __shfl_sync(kFull, x.y, src),
+                    __shfl_sync(kFull, x.z, src), __shfl_sync(kFull, x.w, src));
+}
+__device__ __forceinline__ uint4 from_prev_lane(uint4 v, uint4 wrap, int lane) {
+  const uint4 x = lane == 31 ? wrap : v;
+  const int src = (lane + 31) & 31;
+  return make_uint4(__shfl_sync(kFull, x.x, src), __shfl_sync(kFull, x.y, src),
+                    __shfl_sync(kFull, x.z, src), __shfl_sync(kFull, x.w, src));
+}
+
+// Segments of chunks [c, c + NC) of a stream, from its read side: v[k] = bytes
+// [16 (lane + 32 k), + 16) from c * 4096, zero past the end.  A contiguous
+// buffer off a 16-byte boundary is read in the aligned vectors it touches,
+// each once: a segment straddles two of them, the second being the next
+// lane's.  INSIDE: every byte the chunks and their two neighbouring vectors
+// cover lies inside the stream; otherwise the vectors that reach outside the
+// buffer, its first and its last, are read by words and bytes.  Called by a
+// whole warp.
+template <int MODE, int NC, bool INSIDE>
+__device__ __forceinline__ void load_chunks(const SecDesc& s, uint64_t c, int lane,
+                                            uint4 (&v)[NC * kSegs], uint32_t* err) {
+  constexpr int NK = NC * kSegs;
+  const uint4 z = make_uint4(0, 0, 0, 0);
+  const uint64_t base = c * kChunkBytes;
+  if (ModeTraits<MODE>::kLoadLayout && s.layout != kContig) {
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+      const uint64_t off = base + 512u * k + 16u * lane;
+      v[k] = z;
+      if (INSIDE || off < s.bytes) {
+        const uint8_t* p = row_addr(s, off, err);
+        if (p) v[k] = ld_stream(p);
+      }
     }
-    uint8_t* p = row_addr(s, off, err);
-    if (p) st_stream(p, v);
+    return;
   }
+  // A record's payload is 256-byte aligned and padded to 256 bytes: whole
+  // segments are readable, the bytes past the end are masked below.
+  const uint8_t* src = ModeTraits<MODE>::kLoadLayout ? s.lbase : s.payload;
+  const int64_t L = static_cast<int64_t>(
+      ModeTraits<MODE>::kLoadLayout ? s.bytes : (s.bytes + 15) & ~15ull);
+  const uint32_t sh = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(src) & 15u);
+  const uint8_t* p = src - sh + base + 16u * lane;                   // this lane's vector 0
+  const int64_t off = static_cast<int64_t>(base + 16u * lane) - sh;  // and its logical byte
+  uint4 extra = z;  // lane 0: the vector after the last one (off a boundary only)
+  auto whole = [&](int k) { return INSIDE || (off + 512 * k >= 0 && off + 512 * k + 16 <= L); };
+#pragma unroll
+  for (int k = 0; k < NK; ++k) v[k] = whole(k) ? ld_stream(p + 512u * k) : z;
+  if (ModeTraits<MODE>::kLoadLayout) {
+    if (sh != 0 && lane == 0 && whole(NK)) extra = ld_stream(p + 512u * NK);
+    if (!INSIDE) {
+      // The vector the buffer's end lies in: `last`, of lane last mod 32.
+      const int64_t last = ((L + sh) >> 4) - static_cast<int64_t>(base >> 4);
+      if (((L + sh) & 15) && last >= 0 && last <= 32 * NK && lane == (last & 31)) {
+        const uint4 x = ld_edge(p + 16 * (last - lane), off + 16 * (last - lane), L);
+        const int kl = static_cast<int>(last >> 5);
+#pragma unroll
+        for (int k = 0; k < NK; ++k)
+          if (k == kl) v[k] = x;
+        if (kl == NK) extra = x;
+      }
+      if (off < 0 && off > -16) v[0] = ld_edge(p, off, L);
+    }
+    if (sh != 0) {
+      // Segments past the end are zero (the vector there may hold the
+      // buffer's last bytes, which belong to the segment before).
+      const int64_t used = INSIDE ? NK : (L - static_cast<int64_t>(base) + 511) >> 9;
+#pragma unroll
+      for (int k = 0; k < NK; ++k) {
+        if (INSIDE || k < used)
+          v[k] = align_bytes(
+              v[k], from_next_lane(v[k], k + 1 < NK ? v[k + 1 < NK ? k + 1 : k] : extra, lane), sh);
+        else
+          v[k] = z;
+      }
+    }
+  } else if (!INSIDE && (s.bytes & 15u)) {
+    // Payload bytes past the logical end read as zero.
+    const uint64_t tail = s.bytes & ~15ull;
+#pragma unroll
+    for (int k = 0; k < NK; ++k)
+      if (base + 512u * k + 16u * lane == tail)
+        v[k] = mask_tail(v[k], static_cast<int>(s.bytes & 15u));
+  }
+}
+
+// Store the segments of chunks [c, c + NC) to the stream's write side.  A
+// contiguous target off a 16-byte boundary is written in its aligned vectors:
+// each takes the end of one segment, the previous lane's, and the beginning
+// of the next; the segment before the chunks is read again from the payload.
+// INSIDE as above.  Called by a whole warp.
+template <int MODE, int NC, bool INSIDE>
+__device__ __forceinline__ void store_chunks(const SecDesc& s, uint64_t c, int lane,
+                                             const uint4 (&v)[NC * kSegs], uint32_t* err) {
+  constexpr int NK = NC * kSegs;
+  const uint64_t base = c * kChunkBytes;
+  if (MODE == kModePack) {
+    // Record payload: write through the 256-byte padding (zeros past the end).
+    const uint64_t padded = (s.bytes + kRecordAlign - 1) / kRecordAlign * kRecordAlign;
+#pragma unroll
+    for (int k = 0; k < NK; ++k)
+      if (INSIDE || base + 512u * k + 16u * lane < padded)
+        st_stream(s.payload + base + 512u * k + 16u * lane, v[k]);
+    return;
+  }
+  if (s.layout != kContig) {
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+      const uint64_t off = base + 512u * k + 16u * lane;
+      if (INSIDE || off < s.bytes) {
+        uint8_t* p = row_addr(s, off, err);
+        if (p) st_stream(p, v[k]);
+      }
+    }
+    return;
+  }
+  const uint32_t sh = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(s.lbase) & 15u);
+  const int64_t L = static_cast<int64_t>(s.bytes);
+  uint8_t* p = s.lbase - sh + base + 16u * lane;
+  const int64_t off = static_cast<int64_t>(base + 16u * lane) - sh;
+  // The target's vector that its end lies in: `last`, of lane last mod 32.
+  const int64_t last = ((L + sh) >> 4) - static_cast<int64_t>(base >> 4);
+  uint4 first_x = make_uint4(0, 0, 0, 0), last_x = first_x;
+  auto put = [&](int k, uint4 x) {
+    if (INSIDE || (off + 512 * k >= 0 && off + 512 * k + 16 <= L)) st_stream(p + 512u * k, x);
+    if (!INSIDE && k == 0) first_x = x;
+    if (!INSIDE && k == (last >> 5)) last_x = x;
+  };
+  if (sh == 0) {
+#pragma unroll
+    for (int k = 0; k < NK; ++k) put(k, v[k]);
+  } else {
+    uint4 before = make_uint4(0, 0, 0, 0);  // lane 31: the segment before the chunks
+    if (lane == 31 && c > 0) before = ld_stream(s.payload + base - 16);
+    const int64_t used = INSIDE ? NK : (L + sh - static_cast<int64_t>(base) + 511) >> 9;
+#pragma unroll
+    for (int k = 0; k < NK; ++k)
+      if (INSIDE || k < used)
+        put(k, align_bytes(from_prev_lane(v[k], k > 0 ? v[k > 0 ? k - 1 : 0] : before, lane), v[k],
+                           16 - sh));
+  }
+  if (!INSIDE && ((L + sh) & 15) && last >= 0) {
+    // The vector holding the end: one of these, or (of the last chunk only)
+    // the one after them, which takes the end of the last segment.
+    const int64_t o = 16 * (last - lane);
+    if (last < 32 * NK) {
+      if (lane == (last & 31) && off + o >= 0) st_edge(p + o, last_x, off + o, L);
+    } else if (last == 32 * NK && lane == 31 && c + NC == s.n_chunks) {
+      st_edge(p + o, align_bytes(v[NK - 1], make_uint4(0, 0, 0, 0), 16 - sh), off + o, L);
+    }
+  }
+  if (!INSIDE && off < 0) st_edge(p, first_x, off, L);
+}
+
+// Move chunks [c, c + NC) and return their node: one chunk's hash, or the
+// pair's (0 in the modes that do not hash).
+template <int MODE, int NC, bool INSIDE>
+__device__ __forceinline__ uint64_t move_chunks(const SecDesc& s, uint64_t c, int lane,
+                                                uint32_t* err) {
+  using T = ModeTraits<MODE>;
+  uint4 v[NC * kSegs];
+  load_chunks<MODE, NC, INSIDE>(s, c, lane, v, err);
+  if (T::kStore) store_chunks<MODE, NC, INSIDE>(s, c, lane, v, err);
+  if (!T::kHash) return 0;
+  uint64_t h[NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) h[q] = fmix(kSeed ^ ((c + q) * 32u + lane));
+#pragma unroll
+  for (int k = 0; k < kSegs; ++k)
+#pragma unroll
+    for (int q = 0; q < NC; ++q) h[q] = absorb(h[q], v[q * kSegs + k]);
+  const uint64_t x = NC == 2 ? tile_tree2(fmix(h[0]), fmix(h[NC - 1]), 2, lane)
+                             : warp_tree(fmix(h[0]), 32, lane);
+  return __shfl_sync(kFull, x, 0);
 }
 
 // Section of warp task `task` in a work list: the last j with begin[j] <=
@@ -359,7 +520,17 @@ __device__ __forceinline__ int find_item(const uint32_t* __restrict__ begin, int
   return lo;
 }
 
-// The warp tasks of one streaming pass (body of k_stream and k_small).
+// The warp tasks of one streaming pass (body of k_stream and k_small): each
+// warp walks a contiguous, balanced range of tasks of 2^glog2 chunks, glog2 =
+// 0 or 1, so that the item of a task is searched for once per warp.
+//
+// Buffers off a 16-byte boundary are bound by the 16 warps per SM that 128
+// registers leave (two chunks of loads each) and by issue: per segment four
+// shuffles and a funnel beside the hash.  Measured (byte and word loads of
+// each lane's own segment, interleaved tasks -> this): fingerprint of 1 GiB at
+// an odd address 1,263 -> 220 us (4.9 TB/s), at a 4-byte one 405 -> 220 us;
+// 2,000 observations of 196,613 bytes, three of four off a boundary: pack 693 ->
+// 184 us, verified restore 862 -> 211 us.
 template <int MODE>
 __device__ __forceinline__ void run_stream_tasks(const SecDesc* __restrict__ secs, const WorkList& wl,
                                                  int glog2, uint64_t* __restrict__ nodes,
@@ -367,61 +538,42 @@ __device__ __forceinline__ void run_stream_tasks(const SecDesc* __restrict__ sec
   using T = ModeTraits<MODE>;
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
-  const uint32_t nw = gridDim.x * kWarps;
-  int cur = -1;
-  for (uint32_t task = blockIdx.x * kWarps + wib; task < wl.n_tasks; task += nw) {
-    const int j = find_item(wl.begin, 0, wl.n_items, task, lane);
-    if (j != cur) {
-      __syncwarp();
-      const SecDesc* src = &secs[__ldg(wl.ids + j)];
-      if (lane < static_cast<int>(sizeof(SecDesc) / 16))
-        reinterpret_cast<uint4*>(&sdesc[wib])[lane] = __ldg(reinterpret_cast<const uint4*>(src) + lane);
-      __syncwarp();
-      cur = j;
-    }
-    const SecDesc& s = sdesc[wib];
+  const uint64_t gw = static_cast<uint64_t>(blockIdx.x) * kWarps + wib;
+  const uint64_t nw = static_cast<uint64_t>(gridDim.x) * kWarps;
+  const uint32_t t0 = static_cast<uint32_t>(wl.n_tasks * gw / nw);
+  const uint32_t t1 = static_cast<uint32_t>(wl.n_tasks * (gw + 1) / nw);
+  // The work list and the descriptors are the host's: the first task's are
+  // read before waiting for the kernel ahead.
+  const SecDesc& s = sdesc[wib];
+  auto load_desc = [&](int j) {
+    const SecDesc* src = &secs[__ldg(wl.ids + j)];
+    __syncwarp();
+    if (lane < static_cast<int>(sizeof(SecDesc) / 16))
+      reinterpret_cast<uint4*>(&sdesc[wib])[lane] = __ldg(reinterpret_cast<const uint4*>(src) + lane);
+    __syncwarp();
+  };
+  int j = 0, cur = -1;
+  if (t0 < t1) load_desc(cur = j = find_item(wl.begin, 0, wl.n_items, t0, lane));
+  grid_dependency();
+  for (uint32_t task = t0; task < t1; ++task) {
+    while (j + 1 < wl.n_items && __ldg(wl.begin + j + 1) <= task) ++j;
+    if (j != cur) load_desc(cur = j);
     const uint32_t local = task - __ldg(wl.begin + j);
     const uint64_t c0 = static_cast<uint64_t>(local) << glog2;
     const uint64_t c1 = min(c0 + (1ull << glog2), static_cast<unsigned long long>(s.n_chunks));
-    uint64_t mine = 0;  // lane j keeps the hash of chunk c0 + j
-    for (uint64_t c = c0; c < c1; c += 2) {
-      const bool two = c + 1 < c1;
-      const uint64_t base = c * kChunkBytes + 16u * lane;
-      uint4 va[kSegs], vb[kSegs];
-#pragma unroll
-      for (int k = 0; k < kSegs; ++k) va[k] = load_seg<MODE>(s, base + 512u * k, err);
-      if (two) {
-#pragma unroll
-        for (int k = 0; k < kSegs; ++k) vb[k] = load_seg<MODE>(s, base + kChunkBytes + 512u * k, err);
-      }
-      if (T::kStore) {
-#pragma unroll
-        for (int k = 0; k < kSegs; ++k) store_seg<MODE>(s, base + 512u * k, va[k], err);
-        if (two) {
-#pragma unroll
-          for (int k = 0; k < kSegs; ++k) store_seg<MODE>(s, base + kChunkBytes + 512u * k, vb[k], err);
-        }
-      }
-      if (T::kHash) {
-        uint64_t ha = fmix(kSeed ^ (c * 32u + lane));
-#pragma unroll
-        for (int k = 0; k < kSegs; ++k) ha = absorb(ha, va[k]);
-        ha = __shfl_sync(kFull, warp_tree(fmix(ha), 32, lane), 0);
-        const int jj = static_cast<int>(c - c0);
-        if (lane == jj) mine = ha;
-        if (two) {
-          uint64_t hb = fmix(kSeed ^ ((c + 1) * 32u + lane));
-#pragma unroll
-          for (int k = 0; k < kSegs; ++k) hb = absorb(hb, vb[k]);
-          hb = __shfl_sync(kFull, warp_tree(fmix(hb), 32, lane), 0);
-          if (lane == jj + 1) mine = hb;
-        }
+    // A pair whose chunks and neighbouring vectors lie inside the stream takes
+    // the unchecked path; the ends of a stream go a chunk at a time.
+    uint64_t x;
+    if (c0 + 1 < c1 && c0 > 0 && (c0 + 2) * kChunkBytes + 16 <= s.bytes) {
+      x = move_chunks<MODE, 2, true>(s, c0, lane, err);
+    } else {
+      x = move_chunks<MODE, 1, false>(s, c0, lane, err);
+      if (c0 + 1 < c1) {
+        const uint64_t y = move_chunks<MODE, 1, false>(s, c0 + 1, lane, err);
+        if (T::kHash) x = comb(x, y);
       }
     }
-    if (T::kHash) {
-      const uint64_t root = warp_tree(mine, static_cast<int>(c1 - c0), lane);
-      if (lane == 0) nodes[s.task_begin + local] = root;
-    }
+    if (T::kHash && lane == 0) nodes[s.task_begin + local] = x;
   }
 }
 
@@ -429,7 +581,6 @@ template <int MODE>
 __global__ void __launch_bounds__(kThreads, 2)
     k_stream(const SecDesc* __restrict__ secs, WorkList wl, int glog2,
              uint64_t* __restrict__ nodes, uint32_t* err) {
-  grid_dependency();
   __shared__ SecDesc sdesc[kWarps];
   run_stream_tasks<MODE>(secs, wl, glog2, nodes, err, sdesc);
 }
@@ -1328,7 +1479,6 @@ __global__ void __launch_bounds__(kThreads, 2)
             uint32_t* err, uint32_t* ticket, int n_items, const SessDesc* __restrict__ sess,
             const Entry* __restrict__ entries, uint64_t* fp_out, const uint64_t* fp_before,
             uint8_t* flags, uint32_t* bad) {
-  grid_dependency();
   __shared__ SecDesc sdesc[kWarps];
   __shared__ uint64_t smem[64];  // up to 2048 sections per session
   __shared__ uint32_t s_bad;

@@ -624,13 +624,12 @@ struct WsLayout {
   uint64_t secs = 0, sess = 0, entries = 0, banks = 0, nodes = 0, total = 0;
 };
 
-// Choose 2^g chunks per warp task: at least ~4 tasks per resident warp,
-// at most 32 chunks per task.
+// Choose 2^g chunks per task of the register kernel, which moves two chunks
+// at a time: single chunks while that gives every resident warp at most two
+// tasks, else pairs.  (Longer tasks only coarsen the warps' shares.)
 int choose_group_log2(const pcs_ctx* c, uint64_t total_chunks) {
   const uint64_t warps = static_cast<uint64_t>(c->sm_count) * c->stream_bps * 8;
-  int g = 0;
-  while (g < kMaxGroupLog2 && (total_chunks >> (g + 1)) >= 4 * warps) ++g;
-  return g;
+  return total_chunks > 2 * warps ? 1 : 0;
 }
 
 uint64_t n_chunks_of(uint64_t bytes) { return bytes == 0 ? 1 : (bytes + kChunkBytes - 1) / kChunkBytes; }

@@ -76,3 +76,41 @@ def test_classify_reads_paths(ctx, dev, n, m):
     spans = list(zip(start.tolist(), length.tolist()))
     assert set(got) <= {0, 1}
     assert [got[i] for i in pick] == _read_flags([spans[i] for i in pick], ro, rn)
+
+
+# Sections off a 16-byte boundary, pairs of chunks per task (more than 40 MB in
+# the register kernel) and single ones: lengths around chunks and tiles, restored
+# to another offset with guard bytes around every target.
+@pytest.mark.parametrize("big", [0, 24])
+def test_offset_sections_round_trip(ctx, dev, big):
+    sizes = [1, 15, 16, 17, 4095, 4096, 4097, 8191, 8192, 8193, 8192 + 4096, 3 * 8192 - 5,
+             3 * 8192 + 15, 5 * 8192, 100003]
+    sizes = [n for n in sizes for _ in OFFSETS] + [2 * 1024 * 1024 + 11 * i for i in range(big)]
+    need = sum(sizes) + 64 * len(sizes)
+    host, src = _arena(need, 5, dev)
+    dst = torch.full((need,), 0xA5, dtype=torch.uint8, device=dev)
+    at, to, secs_a, secs_b, aligned, used = 0, 0, [], [], [], torch.zeros(need, dtype=torch.bool)
+    views = []
+    for i, n in enumerate(sizes):
+        oa, ob = OFFSETS[i % len(OFFSETS)], OFFSETS[(7 * i + 3) % len(OFFSETS)]
+        at, to = (at + 15) // 16 * 16 + 16 + oa, (to + 15) // 16 * 16 + 16 + ob
+        views.append((at, to, n))
+        used[to:to + n] = True
+        secs_a.append(pcs.contig_section(9, src[at:at + n]))
+        secs_b.append(pcs.contig_section(9, dst[to:to + n]))
+        aligned.append(src[at:at + n].clone())
+        at, to = at + n, to + n
+    snap = ctx.checkpoint([pcs.Session(1, 9, secs_a, keep=[src])])[0]
+    want = u64(ctx.fingerprint(aligned))
+    assert [ctx.section(snap, i).fp for i in range(len(sizes))] == want
+    assert want[:20] == [oracle.fingerprint(host[a:a + n].numpy()) for a, _, n in views[:20]]
+    assert u64(ctx.fingerprint([src[a:a + n] for a, _, n in views])) == want
+    for verify in (False, True):
+        dst.fill_(0xA5)
+        ctx.restore([snap], [pcs.Session(1, 9, secs_b, keep=[dst])], verify=verify)
+        got = dst.cpu()
+        for a, t, n in views:
+            assert torch.equal(got[t:t + n], host[a:a + n]), (a, t, n)
+        assert bool((got[~used] == 0xA5).all())
+    ctx.delete(snap)
+    ctx.sync()
