@@ -71,8 +71,10 @@ struct alignas(16) SessDesc {
   uint32_t n_sections;
   uint32_t session_id;
   uint32_t kind;
+  uint32_t n_tasks;        // tasks of all its sections
+  uint32_t pad;
 };
-static_assert(sizeof(SessDesc) == 40 || sizeof(SessDesc) == 48, "SessDesc layout");
+static_assert(sizeof(SessDesc) == 48, "SessDesc layout");
 
 // Section entry exactly as stored in a record (64 bytes, little-endian).
 struct alignas(16) Entry {
@@ -129,14 +131,16 @@ cudaError_t launch_bulk(int mode, const SecDesc* secs, WorkList wl, uint64_t* no
                         uint32_t* dev_err, uint32_t* sched, int sm_count, cudaStream_t stream);
 
 // One launch for a small call: the register streaming pass over wl (no
-// node reduction), then the finaliser of `mode` run by the last block to
-// finish (hash: n_items buffers; pack / restore_verify: n_items sessions).
-// `ticket` must be zero; the last block resets it.
+// node reduction) and the finalisation of `mode` (hash: n_items buffers; pack
+// / restore_verify: n_items sessions of at most max_secs sections), each item
+// by the warp that completes it.  `ticket` and `done` (a word per item, at
+// most kSmallMaxItems) are zero on entry and on exit.
+constexpr int kSmallMaxItems = 64;
 cudaError_t launch_small(int mode, const SecDesc* secs, WorkList wl, int group_log2,
-                         uint64_t* nodes, uint32_t* dev_err, uint32_t* ticket, int n_items,
-                         const SessDesc* sess, const Entry* entries, uint64_t* fp_out,
-                         const uint64_t* fp_before, uint8_t* flags, uint32_t* bad, int sm_count,
-                         int blocks_per_sm, cudaStream_t stream);
+                         uint64_t* nodes, uint32_t* dev_err, uint32_t* ticket, uint32_t* done,
+                         int n_items, int max_secs, const SessDesc* sess, const Entry* entries,
+                         uint64_t* fp_out, const uint64_t* fp_before, uint8_t* flags,
+                         uint32_t* bad, int sm_count, int blocks_per_sm, cudaStream_t stream);
 
 // One level of the node reduction of stream i: count nodes at src, reduced
 // by aligned groups of 32 to ceil(count / 32) nodes at dst.

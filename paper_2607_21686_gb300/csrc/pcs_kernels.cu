@@ -70,6 +70,10 @@ __device__ __forceinline__ uint64_t comb(uint64_t a, uint64_t b) {
   return fmix(a * kP + rotl64(b, 31));
 }
 
+__device__ __forceinline__ uint64_t ld_l2(const uint64_t* p) {
+  return __ldcg(reinterpret_cast<const unsigned long long*>(p));
+}
+
 // A hint to bring the 128-byte line holding `p` into this SM's L1.
 __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
@@ -128,8 +132,9 @@ __device__ uint64_t warp_tree_inplace(uint64_t* a, uint32_t n, int lane) {
   return a[0];
 }
 
-// The same tree for n <= 1024, nothing written; called by one whole warp,
-// every lane returns the root.  Up to 32 items: one warp tree.  Beyond,
+// The same tree for n <= 1024, nothing written, read from L2 (a small call's
+// nodes are written by other blocks of the same launch); called by one whole
+// warp, every lane returns the root.  Up to 32 items: one warp tree.  Beyond,
 // in blocks of 256 items: lane l reads items 8l .. 8l+7 of the block and
 // reduces them in its registers (the tree's first three levels over that
 // aligned group of eight, an odd last item carried up), the warp then
@@ -140,7 +145,7 @@ __device__ uint64_t warp_tree_inplace(uint64_t* a, uint32_t n, int lane) {
 // level (a 256-item tree took 1,790 warp instructions that way).
 __device__ uint64_t warp_tree_regs(const uint64_t* a, uint32_t n, int lane) {
   if (n <= 32) {
-    const uint64_t v = lane < static_cast<int>(n) ? a[lane] : 0;
+    const uint64_t v = lane < static_cast<int>(n) ? ld_l2(a + lane) : 0;
     return __shfl_sync(kFull, warp_tree(v, static_cast<int>(n), lane), 0);
   }
   const uint32_t blocks = (n + 255) / 256;
@@ -151,7 +156,7 @@ __device__ uint64_t warp_tree_regs(const uint64_t* a, uint32_t n, int lane) {
     const int m = max(0, min(8, static_cast<int>(nb) - 8 * lane));  // this lane's items
     uint64_t v[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = i < m ? a[base + 8 * lane + i] : 0;
+    for (int i = 0; i < 8; ++i) v[i] = i < m ? ld_l2(a + base + 8 * lane + i) : 0;
 #pragma unroll
     for (int w = 1; w < 8; w <<= 1)
 #pragma unroll
@@ -522,7 +527,8 @@ __device__ __forceinline__ int find_item(const uint32_t* __restrict__ begin, int
 
 // The warp tasks of one streaming pass (body of k_stream and k_small): each
 // warp walks a contiguous, balanced range of tasks of 2^glog2 chunks, glog2 =
-// 0 or 1, so that the item of a task is searched for once per warp.
+// 0 or 1, so that the item of a task is searched for once per warp.  After
+// each task it calls after_task(its stream, its work list item).
 //
 // Buffers off a 16-byte boundary are bound by the 16 warps per SM that 128
 // registers leave (two chunks of loads each) and by issue: per segment four
@@ -531,10 +537,10 @@ __device__ __forceinline__ int find_item(const uint32_t* __restrict__ begin, int
 // an odd address 1,263 -> 220 us (4.9 TB/s), at a 4-byte one 405 -> 220 us;
 // 2,000 observations of 196,613 bytes, three of four off a boundary: pack 693 ->
 // 184 us, verified restore 862 -> 211 us.
-template <int MODE>
+template <int MODE, typename F>
 __device__ __forceinline__ void run_stream_tasks(const SecDesc* __restrict__ secs, const WorkList& wl,
                                                  int glog2, uint64_t* __restrict__ nodes,
-                                                 uint32_t* err, SecDesc* sdesc) {
+                                                 uint32_t* err, SecDesc* sdesc, F&& after_task) {
   using T = ModeTraits<MODE>;
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
@@ -574,6 +580,7 @@ __device__ __forceinline__ void run_stream_tasks(const SecDesc* __restrict__ sec
       }
     }
     if (T::kHash && lane == 0) nodes[s.task_begin + local] = x;
+    after_task(s, j);
   }
 }
 
@@ -582,7 +589,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     k_stream(const SecDesc* __restrict__ secs, WorkList wl, int glog2,
              uint64_t* __restrict__ nodes, uint32_t* err) {
   __shared__ SecDesc sdesc[kWarps];
-  run_stream_tasks<MODE>(secs, wl, glog2, nodes, err, sdesc);
+  run_stream_tasks<MODE>(secs, wl, glog2, nodes, err, sdesc, [](const SecDesc&, int) {});
 }
 
 // ---------------------------------------------------------------------------
@@ -1377,8 +1384,93 @@ __global__ void __launch_bounds__(512)
                                 gridDim.x, smem, &s_bad);
 }
 
-// Sessions of at most 32 sections: one warp per session (lane j keeps
-// section j's fp), the same outputs as finalize_sessions_block.
+// A session of at most 32 sections, finalised by one warp (lane j keeps
+// section j's fp): the same outputs as finalize_sessions_block.  Lane j's part
+// of the session's descriptors (the host's):
+struct SessLane {
+  uint32_t fin_begin, fin_count;  // section j's nodes
+  uint64_t bytes;                 // and its length
+};
+
+__device__ __forceinline__ SessLane session_lane(const SessDesc& S, const SecDesc* __restrict__ secs,
+                                                 int lane) {
+  SessLane l{0, 0, 0};
+  if (lane < static_cast<int>(S.n_sections)) {
+    const SecDesc* sj = secs + S.sec_begin + lane;
+    l.fin_begin = __ldg(&sj->fin_begin);
+    l.fin_count = __ldg(&sj->fin_count);
+    l.bytes = __ldg(reinterpret_cast<const unsigned long long*>(&sj->bytes));
+  }
+  return l;
+}
+
+template <int MODE>
+__device__ __forceinline__ void finalize_session_warp(const SessDesc& S, const SessLane& l, int b,
+                                                      const Entry* __restrict__ entries,
+                                                      uint64_t* nodes, uint8_t* corrupt,
+                                                      uint32_t* bad, int lane) {
+  Entry* table = reinterpret_cast<Entry*>(S.record + kHeaderBytes);
+  const int ns = static_cast<int>(S.n_sections);
+  // A restore's stored fps (lane j: section j's), read once; each section's
+  // tree then starts from its node loads, and a checkpoint's entry is read
+  // before the tree.
+  uint64_t stored = 0;
+  if (MODE != kModePack && lane < ns) stored = table[lane].fp;
+  uint64_t mine = 0;
+  bool bad_sec = false;
+  for (int j = 0; j < ns; ++j) {
+    uint4 ew = make_uint4(0, 0, 0, 0);  // pack: lanes 0..3 hold the entry, read before the tree
+    if (MODE == kModePack && lane < 4)
+      ew = reinterpret_cast<const uint4*>(&entries[S.sec_begin + j])[lane];
+    const uint32_t nb = __shfl_sync(kFull, l.fin_begin, j);
+    const uint32_t nc = __shfl_sync(kFull, l.fin_count, j);
+    const uint64_t by = __shfl_sync(kFull, l.bytes, j);
+    const uint64_t root = nc <= kFinRegNodes ? warp_tree_regs(nodes + nb, nc, lane)
+                                             : warp_tree_inplace(nodes + nb, nc, lane);
+    const uint64_t fp = fmix(root ^ (by * kP));
+    if (MODE == kModePack) {
+      // The fp (bytes 32..39 of the entry) is the first half of lane 2's word.
+      if (lane == 2) {
+        ew.x = static_cast<uint32_t>(fp);
+        ew.y = static_cast<uint32_t>(fp >> 32);
+      }
+      if (lane < 4) reinterpret_cast<uint4*>(&table[j])[lane] = ew;
+      if (lane == j) mine = fp;
+    } else {
+      if (lane == j) {
+        mine = stored;
+        bad_sec = stored != fp;
+      }
+    }
+  }
+  // Session fp = fmix(tree(fps) ^ n), the fps being the table's.
+  const uint64_t sfp = fmix(warp_tree(mine, ns, lane) ^ static_cast<uint64_t>(ns));
+  const bool any_bad = __any_sync(kFull, bad_sec);
+  if (lane == 0) {
+    if (MODE == kModePack) {
+      uint4* h = reinterpret_cast<uint4*>(S.record);
+      h[0] = make_uint4(kMagic, kVersion | (S.n_sections << 16), S.session_id, S.kind);
+      h[1] = make_uint4(static_cast<uint32_t>(S.total_bytes),
+                        static_cast<uint32_t>(S.total_bytes >> 32), static_cast<uint32_t>(sfp),
+                        static_cast<uint32_t>(sfp >> 32));
+      h[2] = make_uint4(0, 0, 0, 0);
+      h[3] = make_uint4(0, 0, 0, 0);
+    } else {
+      const uint64_t stored_sfp = *reinterpret_cast<const uint64_t*>(S.record + 24);
+      const bool broken = any_bad || stored_sfp != sfp;
+      if (corrupt) corrupt[b] = broken ? 1 : 0;
+      if (broken) atomicAdd(bad, 1u);
+    }
+  }
+  if (MODE == kModePack) {
+    // Zero the gap between the end of the table and the first payload.
+    const uint64_t from = kHeaderBytes + static_cast<uint64_t>(kEntryBytes) * S.n_sections;
+    for (uint64_t o = from + 16u * lane; o < S.payload_start; o += 16u * 32)
+      *reinterpret_cast<uint4*>(S.record + o) = make_uint4(0, 0, 0, 0);
+  }
+}
+
+// Many sessions of at most 32 sections: a warp per session.
 template <int MODE>
 __global__ void __launch_bounds__(kThreads)
     k_finalize_sessions_warp(const SecDesc* __restrict__ secs, const SessDesc* __restrict__ sess,
@@ -1386,116 +1478,89 @@ __global__ void __launch_bounds__(kThreads)
                              uint8_t* corrupt, uint32_t* bad) {
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * kWarps;
-  // Lane j reads section j's node range and length, all sections at once.
-  // These are the host's descriptors: the warp's first session reads them
-  // while the kernel ahead on the stream drains.
+  // The warp's first session's descriptors are read while the kernel ahead on
+  // the stream drains.
   SessDesc S;
-  uint32_t fin_begin = 0, fin_count = 0;
-  uint64_t sec_bytes = 0;
-  auto load_session = [&](int b) {
-    S = sess[b];
-    fin_begin = fin_count = 0;
-    sec_bytes = 0;
-    if (lane < static_cast<int>(S.n_sections)) {
-      const SecDesc* sj = secs + S.sec_begin + lane;
-      fin_begin = __ldg(&sj->fin_begin);
-      fin_count = __ldg(&sj->fin_count);
-      sec_bytes = __ldg(reinterpret_cast<const unsigned long long*>(&sj->bytes));
-    }
-  };
+  SessLane l;
   const int b_first = blockIdx.x * kWarps + (threadIdx.x >> 5);
-  if (b_first < n_sess) load_session(b_first);
+  if (b_first < n_sess) {
+    S = sess[b_first];
+    l = session_lane(S, secs, lane);
+  }
   grid_dependency();
   for (int b = b_first; b < n_sess; b += nw) {
-    if (b != b_first) load_session(b);
-    Entry* table = reinterpret_cast<Entry*>(S.record + kHeaderBytes);
-    const int ns = static_cast<int>(S.n_sections);
-    // A restore's stored fps (lane j: section j's), read once; each
-    // section's tree then starts from its node loads, and a checkpoint's
-    // entry is read before the tree.
-    uint64_t stored = 0;
-    if (MODE != kModePack && lane < ns) stored = table[lane].fp;
-    uint64_t mine = 0;
-    bool bad_sec = false;
-    for (int j = 0; j < ns; ++j) {
-      uint4 ew = make_uint4(0, 0, 0, 0);  // pack: lanes 0..3 hold the entry, read before the tree
-      if (MODE == kModePack && lane < 4)
-        ew = reinterpret_cast<const uint4*>(&entries[S.sec_begin + j])[lane];
-      const uint32_t nb = __shfl_sync(kFull, fin_begin, j);
-      const uint32_t nc = __shfl_sync(kFull, fin_count, j);
-      const uint64_t by = __shfl_sync(kFull, sec_bytes, j);
-      const uint64_t root = nc <= kFinRegNodes ? warp_tree_regs(nodes + nb, nc, lane)
-                                               : warp_tree_inplace(nodes + nb, nc, lane);
-      const uint64_t fp = fmix(root ^ (by * kP));
-      if (MODE == kModePack) {
-        // The fp (bytes 32..39 of the entry) is the first half of lane 2's word.
-        if (lane == 2) {
-          ew.x = static_cast<uint32_t>(fp);
-          ew.y = static_cast<uint32_t>(fp >> 32);
-        }
-        if (lane < 4) reinterpret_cast<uint4*>(&table[j])[lane] = ew;
-        if (lane == j) mine = fp;
-      } else {
-        if (lane == j) {
-          mine = stored;
-          bad_sec = stored != fp;
-        }
-      }
+    if (b != b_first) {
+      S = sess[b];
+      l = session_lane(S, secs, lane);
     }
-    // Session fp = fmix(tree(fps) ^ n), the fps being the table's.
-    const uint64_t sfp = fmix(warp_tree(mine, ns, lane) ^ static_cast<uint64_t>(ns));
-    const bool any_bad = __any_sync(kFull, bad_sec);
-    if (lane == 0) {
-      if (MODE == kModePack) {
-        uint4* h = reinterpret_cast<uint4*>(S.record);
-        h[0] = make_uint4(kMagic, kVersion | (S.n_sections << 16), S.session_id, S.kind);
-        h[1] = make_uint4(static_cast<uint32_t>(S.total_bytes),
-                          static_cast<uint32_t>(S.total_bytes >> 32), static_cast<uint32_t>(sfp),
-                          static_cast<uint32_t>(sfp >> 32));
-        h[2] = make_uint4(0, 0, 0, 0);
-        h[3] = make_uint4(0, 0, 0, 0);
-      } else {
-        const uint64_t stored = *reinterpret_cast<const uint64_t*>(S.record + 24);
-        const bool broken = any_bad || stored != sfp;
-        if (corrupt) corrupt[b] = broken ? 1 : 0;
-        if (broken) atomicAdd(bad, 1u);
-      }
-    }
-    if (MODE == kModePack) {
-      // Zero the gap between the end of the table and the first payload.
-      const uint64_t from = kHeaderBytes + static_cast<uint64_t>(kEntryBytes) * S.n_sections;
-      for (uint64_t o = from + 16u * lane; o < S.payload_start; o += 16u * 32)
-        *reinterpret_cast<uint4*>(S.record + o) = make_uint4(0, 0, 0, 0);
-    }
+    finalize_session_warp<MODE>(S, l, b, entries, nodes, corrupt, bad, lane);
   }
 }
 
-// Small calls in one launch: the streaming pass, then the finalisation by
-// the last block to finish (an atomic ticket; no block waits for another).
-// `ticket` is zero on entry and reset by the last block.
+// Small calls in one launch: the streaming pass, then the finalisation.  A
+// buffer, and a session of at most 32 sections, is finalised by the warp that
+// completes its last task: `done[i]` counts the tasks completed of item i
+// (zero on entry; that warp sets it back), so the items' trees run side by
+// side, on the warps that are free.  Calls with a session of more sections
+// leave all of them to the last block to finish (an atomic ticket, zero on
+// entry and reset), a warp per section.  No block or warp waits for another.
+// Bound by latency: 49 tasks of one Markov session are one chunk per warp.
+// Measured, planned calls (the last block finalising every item, a session at
+// a time -> this): 34 sessions of 14,280 bytes pack 50.6 -> 6.0 us, verified
+// restore 56.7 -> 6.8 us; 64 of 10,000 bytes 89.4 -> 5.5 and 99.8 -> 5.6 us; one
+// of 196,608 bytes 6.2 and 6.3 us either way.
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, 2)
     k_small(const SecDesc* __restrict__ secs, WorkList wl, int glog2, uint64_t* nodes,
-            uint32_t* err, uint32_t* ticket, int n_items, const SessDesc* __restrict__ sess,
-            const Entry* __restrict__ entries, uint64_t* fp_out, const uint64_t* fp_before,
-            uint8_t* flags, uint32_t* bad) {
+            uint32_t* err, uint32_t* ticket, uint32_t* done, int n_items, int max_secs,
+            const SessDesc* __restrict__ sess, const Entry* __restrict__ entries, uint64_t* fp_out,
+            const uint64_t* fp_before, uint8_t* flags, uint32_t* bad) {
   __shared__ SecDesc sdesc[kWarps];
+  const int lane = threadIdx.x & 31;
+  if (MODE == kModeHash || max_secs <= 32) {
+    run_stream_tasks<MODE>(secs, wl, glog2, nodes, err, sdesc, [&](const SecDesc& s, int j) {
+      const uint32_t i = MODE == kModeHash ? __ldg(wl.ids + j) : s.sess;
+      SessDesc S{};
+      SessLane l{};
+      if (MODE != kModeHash) {
+        S = sess[i];
+        l = session_lane(S, secs, lane);
+      }
+      const uint32_t total = MODE == kModeHash ? s.n_tasks : S.n_tasks;
+      uint32_t before = 0;
+      if (lane == 0) {
+        __threadfence();  // the task's node, before it counts as done
+        before = atomicAdd(done + i, 1u);
+      }
+      if (__shfl_sync(kFull, before, 0) + 1 != total) return;
+      __threadfence();
+      if (lane == 0) done[i] = 0;
+      if (MODE == kModeHash) {
+        const uint64_t fp = stream_fp(s, nodes, lane);
+        if (lane == 0) {
+          if (fp_out) fp_out[i] = fp;
+          if (fp_before) flags[i] = fp != fp_before[i] ? 1 : 0;
+        }
+      } else {
+        finalize_session_warp<MODE == kModeHash ? kModePack : MODE>(
+            S, l, static_cast<int>(i), entries, nodes, nullptr, bad, lane);
+      }
+    });
+    return;
+  }
   __shared__ uint64_t smem[64];  // up to 2048 sections per session
   __shared__ uint32_t s_bad;
   __shared__ bool s_last;
-  run_stream_tasks<MODE>(secs, wl, glog2, nodes, err, sdesc);
+  run_stream_tasks<MODE>(secs, wl, glog2, nodes, err, sdesc, [](const SecDesc&, int) {});
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  if (MODE == kModeHash) {
-    finalize_hash_warps(secs, n_items, nodes, fp_out, fp_before, flags, threadIdx.x >> 5, kWarps);
-  } else {
+  if (MODE != kModeHash)
     finalize_sessions_block<MODE>(secs, sess, n_items, entries, nodes, nullptr, bad, 0, 1, smem,
                                   &s_bad);
-  }
   if (threadIdx.x == 0) *ticket = 0;
 }
 
@@ -3298,29 +3363,24 @@ cudaError_t launch_bulk(int mode, const SecDesc* secs, WorkList wl, uint64_t* no
 }
 
 cudaError_t launch_small(int mode, const SecDesc* secs, WorkList wl, int group_log2,
-                         uint64_t* nodes, uint32_t* dev_err, uint32_t* ticket, int n_items,
-                         const SessDesc* sess, const Entry* entries, uint64_t* fp_out,
-                         const uint64_t* fp_before, uint8_t* flags, uint32_t* bad, int sm_count,
-                         int blocks_per_sm, cudaStream_t stream) {
+                         uint64_t* nodes, uint32_t* dev_err, uint32_t* ticket, uint32_t* done,
+                         int n_items, int max_secs, const SessDesc* sess, const Entry* entries,
+                         uint64_t* fp_out, const uint64_t* fp_before, uint8_t* flags,
+                         uint32_t* bad, int sm_count, int blocks_per_sm, cudaStream_t stream) {
   if (wl.n_tasks == 0) return cudaErrorInvalidValue;
   const uint64_t want = (static_cast<uint64_t>(wl.n_tasks) + kWarps - 1) / kWarps;
   const uint64_t cap = static_cast<uint64_t>(sm_count) * blocks_per_sm;
   const int blocks = static_cast<int>(want < cap ? want : cap);
+  auto launch = [&](auto kernel) {
+    return launch_after(kernel, blocks, kThreads, 0, stream, secs, wl, group_log2, nodes, dev_err,
+                        ticket, done, n_items, max_secs, sess, entries, fp_out, fp_before, flags,
+                        bad);
+  };
   switch (mode) {
-    case kModeHash:
-      return launch_after(k_small<kModeHash>, blocks, kThreads, 0, stream, secs, wl, group_log2,
-                          nodes, dev_err, ticket, n_items, sess, entries, fp_out, fp_before, flags,
-                          bad);
-    case kModePack:
-      return launch_after(k_small<kModePack>, blocks, kThreads, 0, stream, secs, wl, group_log2,
-                          nodes, dev_err, ticket, n_items, sess, entries, fp_out, fp_before, flags,
-                          bad);
-    case kModeRestoreV:
-      return launch_after(k_small<kModeRestoreV>, blocks, kThreads, 0, stream, secs, wl,
-                          group_log2, nodes, dev_err, ticket, n_items, sess, entries, fp_out,
-                          fp_before, flags, bad);
-    default:
-      return cudaErrorInvalidValue;
+    case kModeHash: return launch(k_small<kModeHash>);
+    case kModePack: return launch(k_small<kModePack>);
+    case kModeRestoreV: return launch(k_small<kModeRestoreV>);
+    default: return cudaErrorInvalidValue;
   }
 }
 

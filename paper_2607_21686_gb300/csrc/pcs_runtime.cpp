@@ -363,9 +363,9 @@ struct pcs_ctx {
   PtrSet<pcs_snapshot> live;
   std::vector<pcs_snapshot*> spare;  // deleted handles' objects, for the next ones
   // Workspaces, one per stream: the descriptors and tree nodes of a call,
-  // after a header of per-call device words ([0] the fused kernel's ticket,
-  // [1] failures of a verify = 1 restore, [4] and [5] the TMA kernel's work
-  // sharing).  Calls on one stream are ordered
+  // after a header of per-call device words ([0] a kernel's ticket, [1]
+  // failures of a verify = 1 restore, [4] and [5] the TMA kernel's work
+  // sharing, [64 ..] the small-call kernel's tasks done per item).  Calls on one stream are ordered
   // by the stream; calls on different streams do not share one, so they can
   // run side by side.
   struct Workspace {
@@ -485,8 +485,10 @@ Arena* arena_of(pcs_ctx* c, uint32_t placement) {
   return placement == PCS_PLACE_DEVICE ? c->dev_arena.get() : c->host_arena.get();
 }
 
-constexpr uint64_t kWsHeader = 256;  // per-call device words before the descriptors
+constexpr uint64_t kWsHeader = 512;  // per-call device words before the descriptors
 constexpr int kWordBulkSched = 4;    // header words [4], [5]: the TMA kernel's work sharing
+constexpr int kWordDone = 64;        // [64 .. 127]: the small-call kernel's tasks done per item
+static_assert(4 * (kWordDone + kSmallMaxItems) <= kWsHeader, "header words");
 
 // The header words of a call: they sit just below its descriptors, in a
 // stream's workspace and in a prepared call's buffer alike.
@@ -814,6 +816,12 @@ uint64_t total_bytes(const std::vector<SecDesc>& d) {
   return t;
 }
 
+// The tasks of each session's streams (after plan_streams).
+void count_tasks(const std::vector<SecDesc>& d, std::vector<SessDesc>& sd) {
+  for (auto& x : sd) x.n_tasks = 0;
+  for (const auto& x : d) sd[x.sess].n_tasks += x.n_tasks;
+}
+
 // Give every stream its node slots and its kernel.  bulk[i] says which.
 bool plan_streams(const pcs_ctx* c, std::vector<SecDesc>& d, const std::vector<char>& bulk,
                   StreamPlan& P, bool allow_reduce = true) {
@@ -1018,8 +1026,6 @@ std::string check_sessions(const std::vector<SecDesc>& d, const std::vector<Sess
 
 // A small call whose streams all take the register kernel runs in one
 // launch (k_small): the streaming pass and its finalisation.
-constexpr int kSmallMaxItems = 64;
-
 bool fused_ok(const std::vector<char>& bulk, bool small, int n_items) {
   if (!small || n_items > kSmallMaxItems) return false;
   for (char b : bulk)
@@ -1117,9 +1123,9 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
                 reinterpret_cast<const uint32_t*>(ws + LL.reg_begin),
                 static_cast<int>(P.reg_ids.size()), P.reg_tasks};
     LaunchScope ls(c, kKStreamHash, stream);
-    PCS_CUDA(launch_small(kModeHash, dsecs, wl, P.glog2, nodes, c->words, c->call_words, n, nullptr,
-                          nullptr, fp_out, fp_before, flags, nullptr, c->sm_count, c->stream_bps,
-                          stream));
+    PCS_CUDA(launch_small(kModeHash, dsecs, wl, P.glog2, nodes, c->words, c->call_words,
+                          c->call_words + kWordDone, n, 0, nullptr, nullptr, fp_out, fp_before,
+                          flags, nullptr, c->sm_count, c->stream_bps, stream));
     return ws_release(c, stream);
   }
   PCS_CUDA(launch_streams(c, kModeHash, dsecs, P, LL, ws, nodes, stream));
@@ -1263,9 +1269,9 @@ cudaError_t launch_prepared(pcs_ctx* c, const Prepared& pr, uint8_t* ws, uint32_
     const auto* dent = reinterpret_cast<const Entry*>(ws + pr.L.entries);
     if (pr.fused) {
       LaunchScope ls(c, kKStreamPack, stream);
-      return launch_small(kModePack, dsecs, wl, pr.P.glog2, nodes, c->words, words, pr.n,
-                          dsess, dent, nullptr, nullptr, nullptr, nullptr, c->sm_count,
-                          c->stream_bps, stream);
+      return launch_small(kModePack, dsecs, wl, pr.P.glog2, nodes, c->words, words,
+                          words + kWordDone, pr.n, pr.max_secs, dsess, dent, nullptr, nullptr,
+                          nullptr, nullptr, c->sm_count, c->stream_bps, stream);
     }
     cudaError_t e = launch_streams(c, kModePack, dsecs, pr.P, pr.LL, ws, nodes, stream);
     if (e != cudaSuccess) return e;
@@ -1276,9 +1282,9 @@ cudaError_t launch_prepared(pcs_ctx* c, const Prepared& pr, uint8_t* ws, uint32_
   uint32_t* bad = pr.verify == 1 ? words + 1 : c->words + 2;
   if (pr.fused) {
     LaunchScope ls(c, kKStreamRestoreV, stream);
-    return launch_small(kModeRestoreV, dsecs, wl, pr.P.glog2, nodes, c->words, words, pr.n,
-                        dsess, nullptr, nullptr, nullptr, nullptr, bad, c->sm_count,
-                        c->stream_bps, stream);
+    return launch_small(kModeRestoreV, dsecs, wl, pr.P.glog2, nodes, c->words, words,
+                        words + kWordDone, pr.n, pr.max_secs, dsess, nullptr, nullptr, nullptr,
+                        nullptr, bad, c->sm_count, c->stream_bps, stream);
   }
   cudaError_t e = launch_streams(c, pr.verify ? kModeRestoreV : kModeRestore, dsecs, pr.P, pr.LL,
                                  ws, pr.verify ? nodes : nullptr, stream);
@@ -1381,6 +1387,7 @@ pcs_status build_checkpoint(pcs_ctx* c, const pcs_session* sessions, int32_t n, 
     arena_of(c, placement)->free(blk);
     return fail(PCS_E_INVAL, "too much data in one call");
   }
+  if (pr->fused) count_tasks(d, sd);
   pr->P.link_bound =
       link_bound_call(d, bulk, std::vector<char>(d.size(), placement == PCS_PLACE_DEVICE), cache);
   if (c->check_plans) {
@@ -1466,6 +1473,7 @@ pcs_status build_restore(pcs_ctx* c, pcs_snapshot* const* snaps, int32_t n,
   pr->fused = verify && fused_ok(bulk, small, n) && max_secs <= 2048;
   if (!plan_streams(c, d, bulk, pr->P, !pr->fused))
     return fail(PCS_E_INVAL, "too much data in one call");
+  if (pr->fused) count_tasks(d, sd);
   pr->P.link_bound = link_bound_call(d, bulk, payload_dev, cache);
   if (c->check_plans) {
     std::vector<std::pair<const uint8_t*, const uint8_t*>> blocks(n);

@@ -114,3 +114,53 @@ def test_offset_sections_round_trip(ctx, dev, big):
         assert bool((got[~used] == 0xA5).all())
     ctx.delete(snap)
     ctx.sync()
+
+
+# Small calls, finalised by the warps that complete their items: one and many
+# sessions, one section and 32 (and 33, finalised by the last block), sections
+# of no task beyond their first chunk; the counters start over at every call.
+@pytest.mark.parametrize("n,secs", [(1, 1), (1, 32), (1, 33), (64, 2), (63, 5), (7, 40), (64, 32)])
+def test_small_calls_of_many_items(ctx, dev, n, secs):
+    rnd = np.random.default_rng(100 * n + secs)
+    size = rnd.integers(0, 2 * (1 << 20) // (3 * n * secs) + 2, (n, secs))
+    size[0, 0] = 0
+    host, src = _arena(int(size.sum()) + 16 * size.size, 9, dev)
+    dst = torch.zeros_like(src)
+    at, spans = 0, []
+    for b in size.reshape(-1).tolist():
+        at = (at + 3) // 4 * 4 if b % 3 else at
+        spans.append((at, b))
+        at += b
+    mk = lambda t: [pcs.Session(s, 9, [pcs.contig_section(1 + i, t[o:o + b]) for i, (o, b) in
+                                       enumerate(spans[s * secs:(s + 1) * secs])], keep=[t])
+                    for s in range(n)]
+    want = [oracle.fingerprint(host[o:o + b].numpy()) for o, b in spans]
+    for _ in range(2):
+        snaps = ctx.checkpoint(mk(src))
+        got = [ctx.section(s, i).fp for s in snaps for i in range(secs)]
+        assert got == want
+        dst.zero_()
+        ctx.restore(snaps, mk(dst), verify=True)
+        for o, b in spans:
+            assert torch.equal(dst[o:o + b].cpu(), host[o:o + b])
+        for s in snaps:
+            ctx.delete(s)
+        if n * secs <= 64:
+            views = [src[o:o + b] for o, b in spans]
+            assert u64(ctx.fingerprint(views)) == want
+    # A wrong byte in one record is found.
+    snap = ctx.checkpoint(mk(src))
+    victim = int(np.argmax(size.sum(1)))
+    sec = int(np.argmax(size[victim]))
+    if size[victim, sec]:
+        path = "/tmp/pcs_small_%d_%d.bin" % (n, secs)
+        ctx.write_file(snap[victim], path)
+        raw = bytearray(open(path, "rb").read())
+        raw[ctx.section(snap[victim], sec).offset] ^= 1
+        open(path, "wb").write(raw)
+        bad = ctx.read_file(path)
+        ctx.delete(snap[victim])
+        snap[victim] = bad
+        assert ctx.restore_status(snap, mk(dst)) == pcs.PCS_E_CORRUPT
+    for s in snap:
+        ctx.delete(s)
