@@ -132,9 +132,10 @@ __device__ uint64_t warp_tree_inplace(uint64_t* a, uint32_t n, int lane) {
   return a[0];
 }
 
-// The same tree for n <= 1024, nothing written, read from L2 (a small call's
-// nodes are written by other blocks of the same launch); called by one whole
-// warp, every lane returns the root.  Up to 32 items: one warp tree.  Beyond,
+// The same tree for n <= 1024, nothing written; called by one whole warp,
+// every lane returns the root.  L2: the items are read past L1 (a small call's
+// are written by other blocks of the same launch; elsewhere L1 serves seven
+// of a lane's eight loads: without it the step of 32 KV contexts lost 0.5 %).  Up to 32 items: one warp tree.  Beyond,
 // in blocks of 256 items: lane l reads items 8l .. 8l+7 of the block and
 // reduces them in its registers (the tree's first three levels over that
 // aligned group of eight, an odd last item carried up), the warp then
@@ -143,9 +144,11 @@ __device__ uint64_t warp_tree_inplace(uint64_t* a, uint32_t n, int lane) {
 // the global pairwise tree, so the root is the same; all 32 lanes combine
 // at once, where trees of 32-item groups leave half the lanes idle at each
 // level (a 256-item tree took 1,790 warp instructions that way).
+template <bool L2>
 __device__ uint64_t warp_tree_regs(const uint64_t* a, uint32_t n, int lane) {
+  auto item = [&](uint32_t i) { return L2 ? ld_l2(a + i) : a[i]; };
   if (n <= 32) {
-    const uint64_t v = lane < static_cast<int>(n) ? ld_l2(a + lane) : 0;
+    const uint64_t v = lane < static_cast<int>(n) ? item(lane) : 0;
     return __shfl_sync(kFull, warp_tree(v, static_cast<int>(n), lane), 0);
   }
   const uint32_t blocks = (n + 255) / 256;
@@ -156,7 +159,7 @@ __device__ uint64_t warp_tree_regs(const uint64_t* a, uint32_t n, int lane) {
     const int m = max(0, min(8, static_cast<int>(nb) - 8 * lane));  // this lane's items
     uint64_t v[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = i < m ? ld_l2(a + base + 8 * lane + i) : 0;
+    for (int i = 0; i < 8; ++i) v[i] = i < m ? item(base + 8 * lane + i) : 0;
 #pragma unroll
     for (int w = 1; w < 8; w <<= 1)
 #pragma unroll
@@ -1220,8 +1223,9 @@ __global__ void __launch_bounds__(kHashThreads, 1)
 // Finalisation: stream fps, record headers, verification
 // ---------------------------------------------------------------------------
 
+template <bool L2 = false>
 __device__ __forceinline__ uint64_t stream_fp(const SecDesc& s, uint64_t* nodes, int lane) {
-  const uint64_t root = s.fin_count <= kFinRegNodes ? warp_tree_regs(nodes + s.fin_begin, s.fin_count, lane)
+  const uint64_t root = s.fin_count <= kFinRegNodes ? warp_tree_regs<L2>(nodes + s.fin_begin, s.fin_count, lane)
                                              : warp_tree_inplace(nodes + s.fin_begin, s.fin_count, lane);
   return fmix(root ^ (s.bytes * kP));
 }
@@ -1404,7 +1408,7 @@ __device__ __forceinline__ SessLane session_lane(const SessDesc& S, const SecDes
   return l;
 }
 
-template <int MODE>
+template <int MODE, bool L2>
 __device__ __forceinline__ void finalize_session_warp(const SessDesc& S, const SessLane& l, int b,
                                                       const Entry* __restrict__ entries,
                                                       uint64_t* nodes, uint8_t* corrupt,
@@ -1425,7 +1429,7 @@ __device__ __forceinline__ void finalize_session_warp(const SessDesc& S, const S
     const uint32_t nb = __shfl_sync(kFull, l.fin_begin, j);
     const uint32_t nc = __shfl_sync(kFull, l.fin_count, j);
     const uint64_t by = __shfl_sync(kFull, l.bytes, j);
-    const uint64_t root = nc <= kFinRegNodes ? warp_tree_regs(nodes + nb, nc, lane)
+    const uint64_t root = nc <= kFinRegNodes ? warp_tree_regs<L2>(nodes + nb, nc, lane)
                                              : warp_tree_inplace(nodes + nb, nc, lane);
     const uint64_t fp = fmix(root ^ (by * kP));
     if (MODE == kModePack) {
@@ -1493,7 +1497,7 @@ __global__ void __launch_bounds__(kThreads)
       S = sess[b];
       l = session_lane(S, secs, lane);
     }
-    finalize_session_warp<MODE>(S, l, b, entries, nodes, corrupt, bad, lane);
+    finalize_session_warp<MODE, false>(S, l, b, entries, nodes, corrupt, bad, lane);
   }
 }
 
@@ -1536,13 +1540,13 @@ __global__ void __launch_bounds__(kThreads, 2)
       __threadfence();
       if (lane == 0) done[i] = 0;
       if (MODE == kModeHash) {
-        const uint64_t fp = stream_fp(s, nodes, lane);
+        const uint64_t fp = stream_fp<true>(s, nodes, lane);
         if (lane == 0) {
           if (fp_out) fp_out[i] = fp;
           if (fp_before) flags[i] = fp != fp_before[i] ? 1 : 0;
         }
       } else {
-        finalize_session_warp<MODE == kModeHash ? kModePack : MODE>(
+        finalize_session_warp<MODE == kModeHash ? kModePack : MODE, true>(
             S, l, static_cast<int>(i), entries, nodes, nullptr, bad, lane);
       }
     });
