@@ -58,7 +58,8 @@ struct alignas(16) SecDesc {
   uint32_t fin_count;      // nodes the finaliser trees: [fin_begin, fin_begin + fin_count)
   uint32_t fin_begin;      // (the task nodes, or their 32-to-1 reduction)
   uint32_t sess;           // checkpoint / restore: the session of this stream
-  uint32_t pad[2];
+  uint64_t row_shift;      // bytes of row 0 before the stream's first byte (a ring
+                           // walked by whole pages: see make_desc), else 0
 };
 static_assert(sizeof(SecDesc) == 112, "SecDesc layout");
 
@@ -126,8 +127,9 @@ cudaError_t launch_stream(int mode, const SecDesc* secs, WorkList wl, int group_
 // memory with cp.async.bulk; one persistent block per SM.  `sched`: two
 // device words of the call (zero on entry, left zero) that share out the
 // launch's last tiles at run time; launches using the same words must be
-// ordered.  (Hash mode runs k_hash and does not use them.)
-cudaError_t launch_bulk(int mode, const SecDesc* secs, WorkList wl, uint64_t* nodes,
+// ordered.  (Hash mode runs k_hash and does not use them.)  `shift`: some
+// stream has a row_shift.
+cudaError_t launch_bulk(int mode, bool shift, const SecDesc* secs, WorkList wl, uint64_t* nodes,
                         uint32_t* dev_err, uint32_t* sched, int sm_count, cudaStream_t stream);
 
 // One launch for a small call: the register streaming pass over wl (no

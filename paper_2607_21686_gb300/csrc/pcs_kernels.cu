@@ -253,11 +253,8 @@ __device__ __forceinline__ uint64_t div_rows(uint64_t x, uint64_t d, int shift) 
   return shift >= 0 ? (x >> shift) : (x / d);
 }
 
-// Address of logical byte `off` (a multiple of 16) on the layout side of a
-// ROWS / RING stream, or null if its row / page id is out of range.
-__device__ __forceinline__ uint8_t* row_addr(const SecDesc& s, uint64_t off, uint32_t* err) {
-  const uint64_t r = div_rows(off, s.row_bytes, s.rb_shift);
-  const uint64_t w = off - r * s.row_bytes;
+// Address of row r of a ROWS / RING stream (null if its id is out of range).
+__device__ __forceinline__ uint8_t* row_ptr(const SecDesc& s, uint64_t r, uint32_t* err) {
   uint64_t id, row;
   if (s.layout == kRows) {
     id = static_cast<uint32_t>(__ldg(s.index + r));
@@ -274,7 +271,16 @@ __device__ __forceinline__ uint8_t* row_addr(const SecDesc& s, uint64_t off, uin
     atomicOr(err, kDevErrIndex);
     return nullptr;
   }
-  return s.lbase + row * s.row_bytes + w;
+  return s.lbase + row * s.row_bytes;
+}
+
+// Address of logical byte `off` (a multiple of 16) on the layout side of a
+// ROWS / RING stream, or null if its row / page id is out of range.
+__device__ __forceinline__ uint8_t* row_addr(const SecDesc& s, uint64_t off, uint32_t* err) {
+  const uint64_t y = off + s.row_shift;
+  const uint64_t r = div_rows(y, s.row_bytes, s.rb_shift);
+  uint8_t* p = row_ptr(s, r, err);
+  return p ? p + (y - r * s.row_bytes) : nullptr;
 }
 
 // ---------------------------------------------------------------------------
@@ -646,9 +652,9 @@ constexpr uint32_t kDynMaxTilesPerWarp = 64;
 constexpr uint32_t kDynShare = 8;
 constexpr uint32_t kDynGrabsPerWarp = 8;
 constexpr uint32_t kDynChunkMax = 32;
-constexpr int kTileRows = 32;  // rows >= 512 bytes touching an 8 KiB tile: at most 17
+constexpr int kTileRows = 32;  // rows >= 512 bytes touching an 8 KiB tile: at most 17 (18 of a ring)
 constexpr long long kWaitCycles = 4000000000ll;  // give up a wait after ~2 s of SM clock
-static_assert(kTileBytes / kBulkMinRowBytes + 1 <= kTileRows, "tile rows");
+static_assert(kTileBytes / kBulkMinRowBytes + 2 <= kTileRows, "tile rows");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -727,26 +733,6 @@ struct BulkShared {
   WarpStage st[W][S];
 };
 
-// Layout-side address of row r of a ROWS / RING stream (null if out of range).
-__device__ __forceinline__ uint8_t* row_ptr(const SecDesc& s, uint64_t r, uint32_t* err) {
-  uint64_t id, row;
-  if (s.layout == kRows) {
-    id = static_cast<uint32_t>(__ldg(s.index + r));
-    row = id;
-  } else {
-    uint64_t slot = s.ring_start + r;
-    if (slot >= s.window) slot -= s.window;
-    const uint64_t pg = div_rows(slot, s.page_rows, s.pr_shift);
-    id = static_cast<uint32_t>(__ldg(s.index + pg));
-    row = id * s.page_rows + (slot - pg * s.page_rows);
-  }
-  if (id >= s.base_rows) {
-    atomicOr(err, kDevErrIndex);
-    return nullptr;
-  }
-  return s.lbase + row * s.row_bytes;
-}
-
 // End of the bytes of tile [p0, p1) that bulk copies stage: the layout side
 // up to its last whole 16-byte segment; the payload (padded to 256 bytes in
 // the record) up to its 16-byte-rounded end.
@@ -757,17 +743,30 @@ __device__ __forceinline__ uint64_t staged_end(const SecDesc& s, uint64_t p1) {
   return p1 < end ? p1 : end;
 }
 
-// Bytes of [p0, pe) that row i of a stage covers.
+// Bytes of [p0, pe) that row i of a stage covers.  SHIFT: some stream of the
+// launch begins inside its first row (row_shift), whose own first byte then
+// lies before the stream's.  Launches without any keep the unsigned form, in
+// kernels of their own: the TMA kernels' timing follows the code of their
+// staging (with the signed form for all, 32 KV contexts packed in 990 us
+// instead of 979 and came back in 979 instead of 989).
+template <bool SHIFT>
 __device__ __forceinline__ uint32_t row_share(const WarpStage& m, uint64_t rb, int i, uint64_t pe) {
-  const uint64_t lo = (m.r0 + i) * rb, hi = lo + rb;
-  const uint64_t a = lo > m.p0 ? lo : m.p0, b = hi < pe ? hi : pe;
-  return b > a ? static_cast<uint32_t>(b - a) : 0u;
+  if constexpr (SHIFT) {
+    const int64_t lo = static_cast<int64_t>((m.r0 + i) * rb) - static_cast<int64_t>(m.d.row_shift);
+    const int64_t hi = lo + static_cast<int64_t>(rb);
+    const int64_t a = max(lo, static_cast<int64_t>(m.p0)), b = min(hi, static_cast<int64_t>(pe));
+    return b > a ? static_cast<uint32_t>(b - a) : 0u;
+  } else {
+    const uint64_t lo = (m.r0 + i) * rb, hi = lo + rb;
+    const uint64_t a = lo > m.p0 ? lo : m.p0, b = hi < pe ? hi : pe;
+    return b > a ? static_cast<uint32_t>(b - a) : 0u;
+  }
 }
 
 // Bulk copies between a stage's buffer and the layout side, one per run of
 // rows contiguous in memory, covering payload bytes [m.p0, pe).  Lane i owns
 // row i (address rp; null = skipped).  Returns the bytes this lane copied.
-template <bool kLoad>
+template <bool kLoad, bool SHIFT>
 __device__ __forceinline__ uint32_t issue_runs(const WarpStage& m, uint8_t* rp, uint64_t pe,
                                                uint8_t* tile, uint64_t* bar, int lane) {
   const uint64_t rb = m.d.row_bytes;
@@ -779,15 +778,29 @@ __device__ __forceinline__ uint32_t issue_runs(const WarpStage& m, uint8_t* rp, 
   if (!start || rp == nullptr) return 0;
   const unsigned later = lane < 31 ? (starts >> (lane + 1)) : 0u;
   const int next = later ? lane + __ffs(later) : n;
-  const uint64_t row_lo = (m.r0 + lane) * rb, row_hi = (m.r0 + next) * rb;
-  const uint64_t a = row_lo > m.p0 ? row_lo : m.p0;
-  const uint64_t b = row_hi < pe ? row_hi : pe;
-  if (a >= b) return 0;
-  uint8_t* g = rp + (a - row_lo);
-  uint8_t* sp = tile + (a - m.p0);
-  if (kLoad) bulk_g2s(sp, g, static_cast<uint32_t>(b - a), bar);
-  else bulk_s2g(g, sp, static_cast<uint32_t>(b - a));
-  return static_cast<uint32_t>(b - a);
+  if constexpr (SHIFT) {
+    const int64_t sh = static_cast<int64_t>(m.d.row_shift);
+    const int64_t row_lo = static_cast<int64_t>((m.r0 + lane) * rb) - sh;
+    const int64_t row_hi = static_cast<int64_t>((m.r0 + next) * rb) - sh;
+    const int64_t a = max(row_lo, static_cast<int64_t>(m.p0));
+    const int64_t b = min(row_hi, static_cast<int64_t>(pe));
+    if (a >= b) return 0;
+    uint8_t* g = rp + (a - row_lo);
+    uint8_t* sp = tile + (a - static_cast<int64_t>(m.p0));
+    if (kLoad) bulk_g2s(sp, g, static_cast<uint32_t>(b - a), bar);
+    else bulk_s2g(g, sp, static_cast<uint32_t>(b - a));
+    return static_cast<uint32_t>(b - a);
+  } else {
+    const uint64_t row_lo = (m.r0 + lane) * rb, row_hi = (m.r0 + next) * rb;
+    const uint64_t a = row_lo > m.p0 ? row_lo : m.p0;
+    const uint64_t b = row_hi < pe ? row_hi : pe;
+    if (a >= b) return 0;
+    uint8_t* g = rp + (a - row_lo);
+    uint8_t* sp = tile + (a - m.p0);
+    if (kLoad) bulk_g2s(sp, g, static_cast<uint32_t>(b - a), bar);
+    else bulk_s2g(g, sp, static_cast<uint32_t>(b - a));
+    return static_cast<uint32_t>(b - a);
+  }
 }
 
 // Copy the descriptor of section `sec` into a stage (a whole warp; nothing
@@ -804,7 +817,7 @@ __device__ __forceinline__ void stage_desc(const SecDesc* __restrict__ secs, uin
 }
 
 // Stage tile t (of work list item `item`) into stage `st` / barrier `bar`.
-template <int MODE>
+template <int MODE, bool SHIFT>
 __device__ __forceinline__ void stage_tile(const SecDesc* __restrict__ secs, const WorkList& wl,
                                            int item, uint32_t t, WarpStage& st, uint8_t* tile,
                                            uint64_t* bar, uint32_t* err, int lane) {
@@ -822,9 +835,11 @@ __device__ __forceinline__ void stage_tile(const SecDesc* __restrict__ secs, con
   uint32_t n_rows = 0;
   uint8_t* rp = nullptr;
   if (s.layout != kContig) {
-    r0 = div_rows(p0, s.row_bytes, s.rb_shift);
+    const uint64_t sh = SHIFT ? s.row_shift : 0;  // (0: as if it were not there)
+    r0 = div_rows(p0 + sh, s.row_bytes, s.rb_shift);
     const uint64_t lim = L < p1 ? L : p1;
-    if (lim > p0) n_rows = static_cast<uint32_t>(div_rows(lim - 1, s.row_bytes, s.rb_shift) + 1 - r0);
+    if (lim > p0)
+      n_rows = static_cast<uint32_t>(div_rows(lim - 1 + sh, s.row_bytes, s.rb_shift) + 1 - r0);
     if (lane < static_cast<int>(n_rows)) rp = row_ptr(s, r0 + lane, err);
     st.rowp[lane] = rp;
   }
@@ -857,10 +872,17 @@ __device__ __forceinline__ void stage_tile(const SecDesc* __restrict__ secs, con
   // with the bytes the copies will bring, then one bulk copy per run.
   uint32_t mine = 0;
   if (lane < static_cast<int>(n_rows)) {
-    const uint32_t share = row_share(st, s.row_bytes, lane, pe);
+    const uint32_t share = row_share<SHIFT>(st, s.row_bytes, lane, pe);
     if (rp == nullptr) {
-      const uint64_t lo = (r0 + lane) * s.row_bytes;
-      const uint64_t a = lo > p0 ? lo : p0;
+      uint64_t a;
+      if constexpr (SHIFT) {
+        const int64_t lo = static_cast<int64_t>((r0 + lane) * s.row_bytes) -
+                           static_cast<int64_t>(s.row_shift);
+        a = static_cast<uint64_t>(max(lo, static_cast<int64_t>(p0)));
+      } else {
+        const uint64_t lo = (r0 + lane) * s.row_bytes;
+        a = lo > p0 ? lo : p0;
+      }
       for (uint32_t o = 0; o < share; o += 16)
         *reinterpret_cast<uint4*>(tile + (a - p0) + o) = make_uint4(0, 0, 0, 0);
       fence_async_smem();
@@ -872,13 +894,13 @@ __device__ __forceinline__ void stage_tile(const SecDesc* __restrict__ secs, con
   for (int d = 16; d > 0; d >>= 1) mine += __shfl_xor_sync(kFull, mine, d);
   if (lane == 0) mbar_arrive_expect_tx(bar, mine);
   __syncwarp();
-  issue_runs<true>(st, rp, pe, tile, bar, lane);
+  issue_runs<true, SHIFT>(st, rp, pe, tile, bar, lane);
 }
 
 // One staged tile whose loads have landed: complete it, issue its stores
 // (one bulk group), fold its chunks into the fingerprint and write its node.
 // Returns whether stores were issued.  Called by a whole warp.
-template <int MODE>
+template <int MODE, bool SHIFT>
 __device__ __forceinline__ bool bulk_tile(const WarpStage& m, uint8_t* tile,
                                           uint64_t* __restrict__ nodes, int lane) {
   using T = ModeTraits<MODE>;
@@ -926,7 +948,7 @@ __device__ __forceinline__ bool bulk_tile(const WarpStage& m, uint8_t* tile,
       for (uint64_t o = (vend > p0 ? vend : p0) + lane; o < lim; o += 32) s.lbase[o] = tile[o - p0];
     } else {
       uint8_t* rp = m.rowp[lane];
-      if (issue_runs<false>(m, rp, lim, tile, nullptr, lane)) {
+      if (issue_runs<false, SHIFT>(m, rp, lim, tile, nullptr, lane)) {
         bulk_commit();
         issued = true;
       }
@@ -965,7 +987,7 @@ __device__ __forceinline__ bool bulk_tile(const WarpStage& m, uint8_t* tile,
 
 // The TMA kernel with static work: each warp moves a contiguous, balanced
 // range of the launch's tiles, kWarpStages in flight.
-template <int MODE>
+template <int MODE, bool SHIFT>
 __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1)
     k_bulk(const SecDesc* __restrict__ secs, WorkList wl, uint64_t* __restrict__ nodes,
            uint32_t* err) {
@@ -1001,7 +1023,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1)
   };
   const int pre = static_cast<int>(t1 - t0 < static_cast<uint32_t>(kWarpStages) ? t1 - t0 : kWarpStages);
   for (int k = 0; k < pre; ++k)
-    stage_tile<MODE>(secs, wl, item_of(t0 + k), t0 + k, sh.st[warp][k], sh.buf[warp][k],
+    stage_tile<MODE, SHIFT>(secs, wl, item_of(t0 + k), t0 + k, sh.st[warp][k], sh.buf[warp][k],
                      &sh.bar[warp][k], err, lane);
   bool any_issued = false;
   for (uint32_t i = 0; t0 + i < t1; ++i) {
@@ -1017,14 +1039,14 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1)
       if (lane == 0) atomicOr(err, kDevErrTimeout);
       break;
     }
-    if (bulk_tile<MODE>(m, tile, nodes, lane)) {
+    if (bulk_tile<MODE, SHIFT>(m, tile, nodes, lane)) {
       bulk_wait_read();
       any_issued = true;
     }
     __syncwarp();
     // Reuse the stage for tile i + kWarpStages.
     const uint32_t tn = t0 + i + kWarpStages;
-    if (tn < t1) stage_tile<MODE>(secs, wl, item_of(tn), tn, m, tile, bar, err, lane);
+    if (tn < t1) stage_tile<MODE, SHIFT>(secs, wl, item_of(tn), tn, m, tile, bar, err, lane);
   }
   if (any_issued) bulk_wait_all();
 }
@@ -1036,7 +1058,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1)
 // warp asks first, so that warps that drew slower memory do not hold up the
 // end of the launch.  sched[0..1] are zero on entry; the last warp to finish
 // sets them back to zero.
-template <int MODE>
+template <int MODE, bool SHIFT>
 __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1)
     k_bulk_shared(const SecDesc* __restrict__ secs, WorkList wl, uint64_t* __restrict__ nodes,
                   uint32_t* err, uint32_t* sched) {
@@ -1109,7 +1131,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1)
   for (int k = 0; k < kWarpStages; ++k) {
     uint32_t t;
     if (!take(&t)) break;
-    stage_tile<MODE>(secs, wl, item, t, sh.st[warp][k], sh.buf[warp][k], &sh.bar[warp][k], err,
+    stage_tile<MODE, SHIFT>(secs, wl, item, t, sh.st[warp][k], sh.buf[warp][k], &sh.bar[warp][k], err,
                      lane);
     ++staged;
   }
@@ -1128,7 +1150,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1)
       if (lane == 0) atomicOr(err, kDevErrTimeout);
       break;
     }
-    if (bulk_tile<MODE>(m, tile, nodes, lane)) {
+    if (bulk_tile<MODE, SHIFT>(m, tile, nodes, lane)) {
       bulk_wait_read();
       any_issued = true;
     }
@@ -1136,7 +1158,7 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1)
     // Reuse the stage for this warp's next tile.
     uint32_t tn;
     if (take(&tn)) {
-      stage_tile<MODE>(secs, wl, item, tn, m, tile, bar, err, lane);
+      stage_tile<MODE, SHIFT>(secs, wl, item, tn, m, tile, bar, err, lane);
       ++staged;
     }
   }
@@ -3290,7 +3312,7 @@ int resident_blocks(const void* kernel) {
   return b;
 }
 
-template <int MODE>
+template <int MODE, bool SHIFT>
 cudaError_t launch_bulk_mode(const SecDesc* secs, WorkList wl, uint64_t* nodes, uint32_t* err,
                              uint32_t* sched, int sm_count, cudaStream_t stream) {
   using Shape = BulkShape<MODE>;
@@ -3303,20 +3325,21 @@ cudaError_t launch_bulk_mode(const SecDesc* secs, WorkList wl, uint64_t* nodes, 
   if (e != cudaSuccess) return e;
   const uint64_t bit = 1ull << (dev & 63);
   if (!(configured.load(std::memory_order_acquire) & bit)) {
-    e = cudaFuncSetAttribute(k_bulk<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_bulk<MODE, SHIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_bulk_shared<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(smem));
+      e = cudaFuncSetAttribute(k_bulk_shared<MODE, SHIFT>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     configured.fetch_or(bit, std::memory_order_release);
   }
   const uint64_t want = (static_cast<uint64_t>(wl.n_tasks) + Shape::kWarps - 1) / Shape::kWarps;
   const int blocks = static_cast<int>(want < static_cast<uint64_t>(sm_count) ? want : sm_count);
   if (wl.n_tasks < static_cast<uint64_t>(kDynMaxTilesPerWarp) * blocks * Shape::kWarps)
-    return launch_after(k_bulk_shared<MODE>, blocks, Shape::kThreads, smem, stream, secs, wl, nodes,
-                        err, sched);
-  return launch_after(k_bulk<MODE>, blocks, Shape::kThreads, smem, stream, secs, wl, nodes, err);
+    return launch_after(k_bulk_shared<MODE, SHIFT>, blocks, Shape::kThreads, smem, stream, secs, wl,
+                        nodes, err, sched);
+  return launch_after(k_bulk<MODE, SHIFT>, blocks, Shape::kThreads, smem, stream, secs, wl, nodes,
+                      err);
 }
 
 }  // namespace
@@ -3348,20 +3371,24 @@ cudaError_t launch_stream(int mode, const SecDesc* secs, WorkList wl, int group_
   }
 }
 
-cudaError_t launch_bulk(int mode, const SecDesc* secs, WorkList wl, uint64_t* nodes,
+cudaError_t launch_bulk(int mode, bool shift, const SecDesc* secs, WorkList wl, uint64_t* nodes,
                         uint32_t* dev_err, uint32_t* sched, int sm_count, cudaStream_t stream) {
   if (wl.n_tasks == 0) return cudaSuccess;
+  auto launch = [&](auto plain, auto shifted) {
+    return (shift ? shifted : plain)(secs, wl, nodes, dev_err, sched, sm_count, stream);
+  };
   switch (mode) {
     case kModeHash: {
       const uint64_t want = (static_cast<uint64_t>(wl.n_tasks) + kHashWarps - 1) / kHashWarps;
       const int blocks = static_cast<int>(want < static_cast<uint64_t>(sm_count) ? want : sm_count);
       return launch_after(k_hash, blocks, kHashThreads, 0, stream, secs, wl, nodes);
     }
-    case kModePack: return launch_bulk_mode<kModePack>(secs, wl, nodes, dev_err, sched, sm_count, stream);
+    case kModePack:
+      return launch(launch_bulk_mode<kModePack, false>, launch_bulk_mode<kModePack, true>);
     case kModeRestore:
-      return launch_bulk_mode<kModeRestore>(secs, wl, nodes, dev_err, sched, sm_count, stream);
+      return launch(launch_bulk_mode<kModeRestore, false>, launch_bulk_mode<kModeRestore, true>);
     case kModeRestoreV:
-      return launch_bulk_mode<kModeRestoreV>(secs, wl, nodes, dev_err, sched, sm_count, stream);
+      return launch(launch_bulk_mode<kModeRestoreV, false>, launch_bulk_mode<kModeRestoreV, true>);
     default: return cudaErrorInvalidValue;
   }
 }

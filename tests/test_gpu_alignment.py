@@ -164,3 +164,37 @@ def test_small_calls_of_many_items(ctx, dev, n, secs):
         assert ctx.restore_status(snap, mk(dst)) == pcs.PCS_E_CORRUPT
     for s in snap:
         ctx.delete(s)
+
+
+# Rings of rows below 512 bytes, walked by whole pages: pages of one row to many
+# (below and above 512 bytes, powers of two and not), first rows at and inside a
+# page, in a call large enough for the bulk-copy kernel.
+@pytest.mark.parametrize("row,page_rows", [(16, 8), (16, 100), (48, 16), (128, 3), (128, 16),
+                                           (256, 1), (256, 16), (496, 2), (496, 33)])
+def test_rings_of_short_rows(ctx, dev, row, page_rows):
+    pages = max(2, (1 << 18) // (row * page_rows))
+    window = pages * page_rows
+    starts = [0, 1, page_rows - 1, page_rows, window // 2 + 1, window - 1]
+    host, pool = _arena(len(starts) * pages * page_rows * row, 3, dev)
+    shape = (len(starts) * pages, page_rows, row)
+    pool, host = pool.view(shape), host.view(shape)
+    g = torch.Generator().manual_seed(row + page_rows)
+    tab = torch.randperm(shape[0], generator=g).to(torch.int32).view(len(starts), pages)
+    tab2 = torch.randperm(shape[0], generator=g).to(torch.int32).view(len(starts), pages)
+    dt, dt2 = tab.to(dev), tab2.to(dev)
+    out = torch.zeros_like(pool)
+
+    def sessions(p, t, from_snapshot):
+        return [pcs.Session(i, pcs.PCS_KIND_KV, [pcs.ring_section(
+            pcs.PCS_SEC_K, p, t[i], pcs.PCS_RING_START_FROM_SNAPSHOT if from_snapshot else s,
+            window)], keep=[p, t]) for i, s in enumerate(starts)]
+
+    snaps = ctx.checkpoint(sessions(pool, dt, False))
+    ctx.restore(snaps, sessions(out, dt2, True), verify=True)
+    for i, s in enumerate(starts):
+        slot = (s + torch.arange(window)) % window
+        rows = host[tab[i].long()[slot // page_rows], slot % page_rows]
+        assert ctx.section(snaps[i], 0).fp == oracle.fingerprint(rows.contiguous().view(-1).numpy())
+        assert torch.equal(out.cpu()[tab2[i].long()[slot // page_rows], slot % page_rows], rows)
+        ctx.delete(snaps[i])
+    ctx.sync()
