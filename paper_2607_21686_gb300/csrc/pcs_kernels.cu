@@ -1730,8 +1730,6 @@ __device__ __forceinline__ float lane_tree_sum(float v) {
   return v;
 }
 
-constexpr int kScoreIlp = 4;  // entries a warp scores at once (a multiple of 4)
-
 // Element i (0..7) of a 16-byte segment as fp32 (exact conversion).
 template <int DT>  // 1 = bf16, 0 = fp16
 __device__ __forceinline__ float seg_elem(const uint4& v, int i) {
@@ -1740,17 +1738,46 @@ __device__ __forceinline__ float seg_elem(const uint4& v, int i) {
   return __half2float(__ushort_as_half(static_cast<unsigned short>((i & 1) ? (w >> 16) : (w & 0xFFFFu))));
 }
 
-// Each warp scores a contiguous, balanced range of entries, kScoreIlp at a
-// time, following a cursor over the banks (one search per warp).  SPL = 16-byte
-// key segments per lane (D <= 256 * SPL); DT = key type (1 bf16, 0 fp16).
-// The bank's query is held in registers as fp32, with |q| computed once per
-// bank in the same fixed order; every key load of the kScoreIlp entries is
-// issued before any arithmetic.
-template <int SPL, int DT, int HM>
+// Shape of the score kernel for keys of up to `max` elements: the fixed order
+// gives lane floor(e / 8) mod 32 of 32 lanes element e, so a key of at most
+// 8 * kLanes elements has values in kLanes lanes only and 32 / kLanes entries
+// lie side by side in a warp; kSeg segments per lane; kRows rows of entries a
+// round, all their loads in flight before any arithmetic.  kBlocks leaves the
+// registers for that: cut for more blocks, the compiler sinks the loads
+// between the arithmetic (D = 768 at three blocks 88 us instead of 80, D = 64
+// with a histogram at four 98 instead of 94); at two blocks D = 264 took 132 us
+// instead of 114.
+template <int LANES, int SEG, int ROWS, int BLOCKS>
+struct ScoreShape {
+  static constexpr int kLanes = LANES, kSeg = SEG, kRows = ROWS;
+  static constexpr int kSide = 32 / LANES;       // entries side by side
+  static constexpr int kRound = ROWS * kSide;    // entries a round
+  static constexpr int kBlocks = BLOCKS;         // blocks per SM the registers are cut for
+  static_assert(ROWS % 2 == 0 && ROWS <= LANES, "rows pair up and halve over the lanes of an entry");
+};
+
+// Each warp scores a contiguous, balanced range of entries, a round at a
+// time, following a cursor over the banks (one search per warp).  DT = key
+// type (1 bf16, 0 fp16).  The bank's query is held in registers as fp32, with
+// |q| computed once per bank in the same fixed order.
+//
+// Issue slots bound the short keys (the memory system the others), so two
+// rows step together in paired fp32 operations -- (k_a, k_b) straight from
+// the conversions, each half rounded on its own as the separate multiply and
+// add -- three instructions an element and row, and a key shorter than 256
+// elements shares the warp.  Lanes past a key's end hold zeros: no sum here can
+// be -0 (they start at +0), so adding them changes nothing.
+// Measured, 512 MB of fp16 keys, kernel time (one entry after the other across
+// the warp, four in flight, q.k and k.k paired -> this): D = 64 335 -> 86 us,
+// 128 173 -> 84, 192 121 -> 95, 256 95 -> 82, 264 148 -> 114, 512 88 -> 80, 768
+// 140 -> 80, 1,024 123 -> 80 (6.7 TB/s); bf16 within 4 % of these.
+template <class SH, int DT, int HM>
 __device__ __forceinline__ void score_range(const BankDesc* __restrict__ banks, int n_banks,
                                             uint64_t n_entries, float* __restrict__ scores,
                                             bool hist, uint32_t* s_cnt, unsigned long long* s_w) {
+  constexpr int G = SH::kLanes, SPL = SH::kSeg, R = SH::kRows, E = SH::kSide;
   const int lane = threadIdx.x & 31;
+  const int t = lane & (G - 1), side = lane / G;  // this lane's segment, entry of a row
   const uint64_t gw = static_cast<uint64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
   const uint64_t nw = static_cast<uint64_t>(gridDim.x) * kWarps;
   const uint64_t e_begin = n_entries * gw / nw, e_end = n_entries * (gw + 1) / nw;
@@ -1773,113 +1800,103 @@ __device__ __forceinline__ void score_range(const BankDesc* __restrict__ banks, 
   int qbank = -1, segs = 0;
   float qnorm = 0.f;
   float qf[SPL][8];
-#pragma unroll
-  for (int j = 0; j < SPL; ++j)
-#pragma unroll
-    for (int i = 0; i < 8; ++i) qf[j][i] = 0.f;
-  for (uint64_t e0 = e_begin; e0 < e_end; e0 += kScoreIlp) {
+  uint64_t bank_end = 0;
+  BankDesc B{};
+  for (uint64_t e0 = e_begin; e0 < e_end;) {
     // Entries of this round must share one bank to use the cached query;
     // a round stops early at a bank boundary.
-    while (b + 1 < n_banks && __ldg(&banks[b + 1].entry_begin) <= e0) ++b;
-    const BankDesc& B = banks[b];
-    if (b != qbank) {  // warp-uniform: load the query, compute |q|
+    if (qbank < 0 || e0 >= bank_end) {  // warp-uniform: load the query, compute |q|
+      while (b + 1 < n_banks && __ldg(&banks[b + 1].entry_begin) <= e0) ++b;
+      B = banks[b];
+      bank_end = b + 1 < n_banks ? __ldg(&banks[b + 1].entry_begin) : n_entries;
       segs = B.D / 8;
       const uint4* qrow = reinterpret_cast<const uint4*>(B.query);
       float sq = 0.f;
 #pragma unroll
       for (int j = 0; j < SPL; ++j) {
-        const int t = lane + 32 * j;
-        const uint4 qv = t < segs ? __ldg(qrow + t) : make_uint4(0, 0, 0, 0);
+        const uint4 qv = t + 32 * j < segs ? __ldg(qrow + t + 32 * j) : make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           qf[j][i] = seg_elem<DT>(qv, i);
-          if (t < segs) sq = __fadd_rn(sq, __fmul_rn(qf[j][i], qf[j][i]));
+          sq = __fadd_rn(sq, __fmul_rn(qf[j][i], qf[j][i]));
         }
       }
-      // The tree's full sum is lane 0's; every lane finalises an entry below.
-      qnorm = __shfl_sync(kFull, __fsqrt_rn(lane_tree_sum(sq)), 0);
+#pragma unroll
+      for (int d = 1; d < G; d <<= 1) sq = __fadd_rn(sq, __shfl_xor_sync(kFull, sq, d));
+      qnorm = __fsqrt_rn(sq);
       qbank = b;
     }
-    const uint64_t bank_end = b + 1 < n_banks ? __ldg(&banks[b + 1].entry_begin) : n_entries;
     const uint64_t lim = min(static_cast<unsigned long long>(e_end), static_cast<unsigned long long>(bank_end));
-    const int cnt = static_cast<int>(min(static_cast<uint64_t>(kScoreIlp), lim - e0));
+    const int cnt = static_cast<int>(min(static_cast<uint64_t>(SH::kRound), lim - e0));
+    const uint64_t kb = static_cast<uint64_t>(B.D) * 2;  // bytes of a key
     const uint8_t* kbase = reinterpret_cast<const uint8_t*>(B.keys) +
-                           (e0 - B.entry_begin) * static_cast<uint64_t>(B.D) * 2;
-    uint4 kv[kScoreIlp][SPL];
+                           (e0 - B.entry_begin + side) * kb + 16 * t;
+    uint4 kv[R][SPL];
 #pragma unroll
-    for (int q = 0; q < kScoreIlp; ++q)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-      for (int j = 0; j < SPL; ++j) {
-        const int t = lane + 32 * j;
-        kv[q][j] = (q < cnt && t < segs) ? ld_stream(kbase + static_cast<uint64_t>(q) * B.D * 2 + 16 * t)
-                                         : make_uint4(0, 0, 0, 0);
-      }
-    // v[2q] = q.k and v[2q+1] = k.k of entry q, per lane: both chains step
-    // together in paired fp32 operations (each half rounded on its own, as
-    // the separate multiply and add).
-    static_assert(kScoreIlp % 4 == 0, "the transposed tree reduces groups of 4 entries x 2 sums");
-    float v[2 * kScoreIlp];
+      for (int j = 0; j < SPL; ++j)
+        kv[r][j] = r * E + side < cnt && t + 32 * j < segs ? ld_stream(kbase + r * E * kb + 512 * j)
+                                                           : make_uint4(0, 0, 0, 0);
+    // Per lane and row: the partial q.k and k.k, ascending elements.
+    float dot[R], kk[R];
 #pragma unroll
-    for (int q = 0; q < kScoreIlp; ++q) {
-      float2 acc = make_float2(0.f, 0.f);
+    for (int r = 0; r < R; r += 2) {
+      float2 d2 = make_float2(0.f, 0.f), k2 = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int j = 0; j < SPL; ++j) {
-        if (lane + 32 * j < segs) {
+      for (int j = 0; j < SPL; ++j)
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float ke = seg_elem<DT>(kv[q][j], i);
-            acc = __fadd2_rn(acc, __fmul2_rn(make_float2(qf[j][i], ke), make_float2(ke, ke)));
+        for (int i = 0; i < 8; ++i) {
+          const float2 ke = make_float2(seg_elem<DT>(kv[r][j], i), seg_elem<DT>(kv[r + 1][j], i));
+          d2 = __fadd2_rn(d2, __fmul2_rn(make_float2(qf[j][i], qf[j][i]), ke));
+          k2 = __fadd2_rn(k2, __fmul2_rn(ke, ke));
+        }
+      dot[r] = d2.x;
+      dot[r + 1] = d2.y;
+      kk[r] = k2.x;
+      kk[r + 1] = k2.y;
+    }
+    // The lane tree (s[l] += s[l + d], d = 1 .. 16) of all rows at once: while
+    // a lane holds more than one row, it keeps half of them, those its bit of
+    // d selects, and adds its partner's copy.  Addition is commutative, so
+    // every partial sum is the one the plain tree forms.
+    int row = 0;
+#pragma unroll
+    for (int d = 1, h = R / 2; d < G; d <<= 1, h >>= 1) {
+      if (h >= 1) {
+        const bool up = lane & d;
+        row = 2 * row + (up ? 1 : 0);
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i)
+          if (i < h) {
+            const float gd = up ? dot[i] : dot[h + i], gk = up ? kk[i] : kk[h + i];
+            dot[i] = __fadd_rn(up ? dot[h + i] : dot[i], __shfl_xor_sync(kFull, gd, d));
+            kk[i] = __fadd_rn(up ? kk[h + i] : kk[i], __shfl_xor_sync(kFull, gk, d));
           }
-        }
-      }
-      v[2 * q] = acc.x;
-      v[2 * q + 1] = acc.y;
-    }
-    // The lane tree (s[l] += s[l + d], d = 1 .. 16) of the eight sums of
-    // each group of four entries at once: at d = 1, 2, 4 each lane keeps half
-    // of its values and adds its partner's copy of them, so lane l ends with
-    // sum 4*(l&1) + 2*(l>>1&1) + (l>>2&1); d = 8, 16 finish it.  Addition is
-    // commutative, so every partial sum is the one the plain tree forms.
-    const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
-#pragma unroll
-    for (int g = 0; g < kScoreIlp / 4; ++g) {
-      const float* vg = v + 8 * g;
-      float w4[4], w2[2];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float give = b0 ? vg[i] : vg[4 + i];
-        w4[i] = __fadd_rn(b0 ? vg[4 + i] : vg[i], __shfl_xor_sync(kFull, give, 1));
-      }
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const float give = b1 ? w4[i] : w4[2 + i];
-        w2[i] = __fadd_rn(b1 ? w4[2 + i] : w4[i], __shfl_xor_sync(kFull, give, 2));
-      }
-      float w1 = __fadd_rn(b2 ? w2[1] : w2[0], __shfl_xor_sync(kFull, b2 ? w2[0] : w2[1], 4));
-      w1 = __fadd_rn(w1, __shfl_xor_sync(kFull, w1, 8));
-      w1 = __fadd_rn(w1, __shfl_xor_sync(kFull, w1, 16));
-      // Lanes 0..3 hold q.k of entry 4g + 2*(l&1) + (l>>1&1); lane l + 4 its k.k.
-      const float kk = __shfl_down_sync(kFull, w1, 4);
-      const int q = 4 * g + 2 * (lane & 1) + ((lane >> 1) & 1);
-      if (lane < 4 && q < cnt) {
-        const float den = __fmul_rn(qnorm, __fsqrt_rn(kk));
-        const float sc = den == 0.f ? 0.f : __fdiv_rn(w1, den);
-        scores[e0 + q] = sc;
-        if (HM && hist) {
-          const uint32_t d = ord32(sc) >> 21;  // key bits 63..53
-          atomicAdd(&s_cnt[d], 1u);
-          if (HM == 2) atomicAdd(&s_w[d], static_cast<unsigned long long>(B.entry_bytes));
-        }
+      } else {
+        dot[0] = __fadd_rn(dot[0], __shfl_xor_sync(kFull, dot[0], d));
+        kk[0] = __fadd_rn(kk[0], __shfl_xor_sync(kFull, kk[0], d));
       }
     }
-    e0 = e0 + cnt - kScoreIlp;  // the loop adds kScoreIlp: next round starts at e0 + cnt
+    const int q = row * E + side;
+    if (t < R && q < cnt) {
+      const float den = __fmul_rn(qnorm, __fsqrt_rn(kk[0]));
+      const float sc = den == 0.f ? 0.f : __fdiv_rn(dot[0], den);
+      scores[e0 + q] = sc;
+      if (HM && hist) {
+        const uint32_t d = ord32(sc) >> 21;  // key bits 63..53
+        atomicAdd(&s_cnt[d], 1u);
+        if (HM == 2) atomicAdd(&s_w[d], static_cast<unsigned long long>(B.entry_bytes));
+      }
+    }
+    e0 += cnt;
   }
 }
 
 // HM (global threshold): 0 none; 1 / 2 also histogram the top 11 key bits of
 // every score (2: weighted by the bank's entry bytes) and pick the first digit.
-template <int SPL, int DT, int HM>
-__global__ void __launch_bounds__(kThreads)
+template <class SH, int DT, int HM>
+__global__ void __launch_bounds__(kThreads, SH::kBlocks)
     k_score_fixed(const BankDesc* __restrict__ banks, int n_banks, uint64_t n_entries,
                   float* __restrict__ scores, GHist gh) {
   grid_dependency();
@@ -1894,7 +1911,7 @@ __global__ void __launch_bounds__(kThreads)
     }
     __syncthreads();
   }
-  score_range<SPL, DT, HM>(banks, n_banks, n_entries, scores, hist, s_cnt, s_w);
+  score_range<SH, DT, HM>(banks, n_banks, n_entries, scores, hist, s_cnt, s_w);
   if (hist) gpass_finish<HM == 1>(gh.st, 0, gh.uniform_bytes, s_cnt, s_w, &s_last);
 }
 
@@ -3462,44 +3479,56 @@ cudaError_t launch_reduce_nodes(const NodeLevel* lv, int n_secs, uint64_t* nodes
   return launch_after(k_reduce_nodes, blocks, kThreads, 0, stream, lv, n_secs, nodes, base, n_groups);
 }
 
+template <class SH, int DT>
+static cudaError_t launch_score_shape(const BankDesc* banks, int n_banks, uint64_t n_entries,
+                                      float* scores, int sm_count, cudaStream_t stream, GHist gh) {
+  // A round per warp at least; at most one resident wave (large populations
+  // fill it).
+  auto launch = [&](auto kernel) {
+    const uint64_t want = (n_entries + kWarps * SH::kRound - 1) / (kWarps * SH::kRound);
+    const uint64_t cap = static_cast<uint64_t>(sm_count) *
+                         resident_blocks(reinterpret_cast<const void*>(kernel));
+    return launch_after(kernel, static_cast<unsigned>(want < cap ? want : cap), kThreads, 0, stream,
+                        banks, n_banks, n_entries, scores, gh);
+  };
+  const int hm = gh.st ? gh.mode : 0;
+  if (hm == 0) return launch(k_score_fixed<SH, DT, 0>);
+  if (hm == 1) return launch(k_score_fixed<SH, DT, 1>);
+  return launch(k_score_fixed<SH, DT, 2>);
+}
+
+template <int DT>
+static cudaError_t launch_score_type(const BankDesc* banks, int n_banks, uint64_t n_entries,
+                                     int max_dim, float* scores, int sm_count, cudaStream_t stream,
+                                     GHist gh) {
+  auto go = [&](auto launch) { return launch(banks, n_banks, n_entries, scores, sm_count, stream, gh); };
+  if (max_dim <= 64) return go(launch_score_shape<ScoreShape<8, 1, 8, 3>, DT>);
+  if (max_dim <= 128) return go(launch_score_shape<ScoreShape<16, 1, 8, 3>, DT>);
+  if (max_dim <= 256) return go(launch_score_shape<ScoreShape<32, 1, 8, 3>, DT>);
+  if (max_dim <= 512) return go(launch_score_shape<ScoreShape<32, 2, 4, 3>, DT>);
+  if (max_dim <= 768) return go(launch_score_shape<ScoreShape<32, 3, 4, 2>, DT>);
+  return go(launch_score_shape<ScoreShape<32, 4, 4, 2>, DT>);
+}
+
 cudaError_t launch_score(const BankDesc* banks, int n_banks, uint64_t n_entries, int max_dim,
                          int key_types, float* scores, int sm_count, cudaStream_t stream,
                          GHist gh, bool* fused) {
   if (fused) *fused = false;
   if (n_entries == 0) return cudaSuccess;
-  // At least two rounds of kScoreIlp entries per warp; at most one resident
-  // wave (large populations fill it).  Eight rounds per warp took the 64-bank
-  // population's score (16,164 entries) 15.5 us under ncu.
-  const uint64_t want = (n_entries + kWarps * kScoreIlp * 2 - 1) / (kWarps * kScoreIlp * 2);
-  auto grid = [&](const void* k) {
-    const uint64_t cap = static_cast<uint64_t>(sm_count) * resident_blocks(k);
-    return static_cast<int>(want < cap ? want : cap);
-  };
   // key_types: 0 = all fp16, 1 = all bf16, 2 = mixed.
   if (key_types == 2 || max_dim > 1024) {
-    return launch_after(k_score_any, grid(reinterpret_cast<const void*>(k_score_any)), kThreads, 0,
+    // At least two rounds of four entries per warp.
+    const uint64_t want = (n_entries + 8 * kWarps - 1) / (8 * kWarps);
+    const uint64_t cap = static_cast<uint64_t>(sm_count) *
+                         resident_blocks(reinterpret_cast<const void*>(k_score_any));
+    return launch_after(k_score_any, static_cast<unsigned>(want < cap ? want : cap), kThreads, 0,
                         stream, banks, n_banks, n_entries, scores);
   }
-  const int spl = max_dim <= 256 ? 1 : max_dim <= 512 ? 2 : 4;
-  const int hm = gh.st ? gh.mode : 0;
-  cudaError_t e = cudaSuccess;
-#define PCS_SCORE(S, D, H)                                                                      \
-  e = launch_after(k_score_fixed<S, D, H>,                                                      \
-                   grid(reinterpret_cast<const void*>(k_score_fixed<S, D, H>)), kThreads, 0, stream, \
-                   banks, n_banks, n_entries, scores, gh)
-#define PCS_SCORE_H(S, D) (hm == 0 ? PCS_SCORE(S, D, 0) : hm == 1 ? PCS_SCORE(S, D, 1) : PCS_SCORE(S, D, 2))
-  if (key_types == 1) {
-    if (spl == 1) PCS_SCORE_H(1, 1);
-    else if (spl == 2) PCS_SCORE_H(2, 1);
-    else PCS_SCORE_H(4, 1);
-  } else {
-    if (spl == 1) PCS_SCORE_H(1, 0);
-    else if (spl == 2) PCS_SCORE_H(2, 0);
-    else PCS_SCORE_H(4, 0);
-  }
-#undef PCS_SCORE_H
-#undef PCS_SCORE
-  if (fused) *fused = hm != 0 && e == cudaSuccess;
+  const cudaError_t e =
+      key_types == 1
+          ? launch_score_type<1>(banks, n_banks, n_entries, max_dim, scores, sm_count, stream, gh)
+          : launch_score_type<0>(banks, n_banks, n_entries, max_dim, scores, sm_count, stream, gh);
+  if (fused) *fused = gh.st && e == cudaSuccess;
   return e;
 }
 

@@ -7,7 +7,7 @@ import torch
 
 import oracle
 from paper_2607_21686_gb300 import pcs
-from helpers import u64
+from helpers import np_view, u64
 
 pytestmark = pytest.mark.gpu
 
@@ -198,3 +198,39 @@ def test_rings_of_short_rows(ctx, dev, row, page_rows):
         assert torch.equal(out.cpu()[tab2[i].long()[slot // page_rows], slot % page_rows], rows)
         ctx.delete(snaps[i])
     ctx.sync()
+
+
+# The score kernel's shapes at their edges: keys that fill an entry's lanes and
+# that leave some idle, banks shorter and longer than a round of entries and not
+# multiples of one, narrower banks beside wider ones in a call.
+@pytest.mark.parametrize("dims", [(8,), (56,), (64,), (72,), (120, 128), (136,), (248, 256), (264,),
+                                  (504, 512), (520,), (760, 768, 8), (776,), (1016, 1024, 64)])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+def test_scores_of_every_shape(ctx, dev, dims, dtype):
+    g = torch.Generator().manual_seed(sum(dims))
+    sizes = [1, 2, 3, 7, 8, 9, 15, 16, 17, 31, 32, 33, 0, 65, 127, 700]
+    keys, queries = [], []
+    for i, n in enumerate(sizes):
+        d = dims[i % len(dims)]
+        k = torch.randn(n, d, generator=g).to(dtype)
+        if n > 2:
+            k[1] = 0                     # a zero norm scores 0
+            k[2] = torch.finfo(dtype).max  # sums past the largest float
+        keys.append(k)
+        queries.append(torch.randn(d, generator=g).to(dtype))
+    dk, dq = [k.to(dev) for k in keys], [q.to(dev) for q in queries]
+    banks = ctx.banks_array(dk, dq, [100 + 16 * (i % 3) for i in range(len(sizes))])
+    want = np.concatenate([oracle.scores(np_view(q), np_view(k)) for q, k in zip(queries, keys)
+                           if len(k)])
+    total = sum(sizes)
+    kept, off = (torch.zeros(n, dtype=torch.int32, device=dev) for n in (total, len(sizes) + 1))
+    for budget in (None, 60 * total):
+        scores = torch.full((total,), 7.0, device=dev)
+        if budget is None:
+            ctx.prune(banks, len(sizes), ctx.params(pcs.PCS_K_FIXED, k_max=1 << 20), kept, off, scores)
+        else:
+            ctx.prune_global(banks, len(sizes), budget, kept, off, scores)
+        got = scores.cpu().numpy()
+        nan = np.isnan(want)  # which NaN is not defined
+        assert np.array_equal(np.isnan(got), nan)
+        assert np.array_equal(got[~nan].view(np.uint32), want[~nan].view(np.uint32))
