@@ -251,6 +251,15 @@ cudaError_t launch_gselect(const GPlan& p, int pass, int sm_count, cudaStream_t 
 // the compaction: kept indices and bank offsets.  One cooperative launch.
 cudaError_t launch_gfinish(const GPlan& p, int first_pass, int sm_count, cudaStream_t stream);
 
+// The whole threshold and compaction of a population of at most
+// kGSmallEntries entries in at most kGSmallBanks banks, from its scores, in
+// one block.  keep_all: the budget does not bind.
+constexpr uint64_t kGSmallEntries = 16384;
+constexpr int kGSmallBanks = 1024;
+cudaError_t launch_gsmall(const BankDesc* banks, int n_banks, uint64_t entries, const float* scores,
+                          uint64_t budget, bool uniform, bool keep_all, int32_t* kept_idx,
+                          int32_t* kept_off, cudaStream_t stream);
+
 // ---- Copy-on-write page pool (pcs_pool_*) ---------------------------------
 // Reference counts and a free stack over caller memory.  A kernel either only
 // takes pages off the stack (alloc, copy leg) or only puts pages back

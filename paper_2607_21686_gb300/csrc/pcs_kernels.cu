@@ -2789,6 +2789,190 @@ __global__ void __launch_bounds__(kThreads, 4) k_gfinish(GPlan p, int first_pass
 }
 
 // ---------------------------------------------------------------------------
+// The global threshold of a small population in one block after a plain score
+// pass: thread t holds the ranks of entries [16 t, 16 t + 16) for three digit
+// passes over ord32(score) (11, 11, 10 bits, the bytes of each digit's
+// candidates summed in shared memory), ties at the threshold are kept in
+// position order while they fit, and two block scans place the kept entries.
+// Bound by the latency of its block-wide steps; it replaces the histogram of
+// the score kernel and the grid barriers of k_gfinish, which cost a population
+// of any size about 20 us.  Measured, whole calls (those two -> this): 97
+// entries 35.9 -> 21.8 us, 4,953 entries 36.4 -> 23.1 us, 4,132 in 146 banks of
+// 1,024-wide keys 47.4 -> 27.2 us, 6,463 of one size 34.8 -> 24.7 us.
+// ---------------------------------------------------------------------------
+
+constexpr int kGsThreads = 1024;
+constexpr int kGsPer = 16;
+static_assert(kGsThreads * kGsPer == kGSmallEntries, "entries of the one-block path");
+static_assert(kGBins == 2 * kGsThreads, "two bins per thread");
+
+// Inclusive block scan of one value per thread (kGsThreads threads);
+// *total = block sum.
+template <typename T>
+__device__ __forceinline__ T gs_incl_scan(T v, T* warp_sum, T* total) {
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  T incl = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const T o = __shfl_up_sync(kFull, incl, d);
+    if (lane >= d) incl += o;
+  }
+  if (lane == 31) warp_sum[wib] = incl;
+  __syncthreads();
+  T w = warp_sum[lane];  // kGsThreads / 32 = 32 warps
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const T o = __shfl_up_sync(kFull, w, d);
+    if (lane >= d) w += o;
+  }
+  *total = __shfl_sync(kFull, w, 31);
+  const T before = __shfl_sync(kFull, w, wib > 0 ? wib - 1 : 0);
+  __syncthreads();  // warp_sum may be reused
+  return wib > 0 ? before + incl : incl;
+}
+
+template <bool UNIFORM>
+__global__ void __launch_bounds__(kGsThreads, 1)
+    k_gsmall(const BankDesc* __restrict__ banks, int n_banks, uint32_t n, const float* scores,
+             uint64_t budget, int keep_all, int32_t* __restrict__ kept_idx,
+             int32_t* __restrict__ kept_off) {
+  __shared__ uint32_t s_lo[kGBins];                   // counts (UNIFORM) or low bytes per digit
+  __shared__ uint32_t s_hi[UNIFORM ? 1 : kGBins];     // high words of the bytes
+  __shared__ uint32_t s_beg[kGSmallBanks + 1];        // first entry of each bank; then n
+  __shared__ uint64_t s_bytes[UNIFORM ? 1 : kGSmallBanks];
+  __shared__ uint32_t s_rank[kGsThreads];             // kept entries before thread t's
+  __shared__ uint16_t s_keep[kGsThreads];             // and which of its own are kept
+  __shared__ uint64_t scan64[32];
+  __shared__ uint32_t scan32[32];
+  __shared__ uint32_t s_prefix;
+  __shared__ uint64_t s_left;
+  // The bank descriptors are the host's.
+  for (int b = threadIdx.x; b < n_banks; b += kGsThreads) {
+    s_beg[b] = static_cast<uint32_t>(banks[b].entry_begin);
+    if (!UNIFORM) s_bytes[b] = banks[b].entry_bytes;
+  }
+  const uint64_t ubytes = banks[0].entry_bytes;
+  if (threadIdx.x == 0) {
+    s_beg[n_banks] = n;
+    s_prefix = 0;
+    s_left = budget;
+  }
+  grid_dependency();
+  const uint32_t i0 = threadIdx.x * kGsPer;
+  const uint32_t mine = i0 < n ? min(static_cast<uint32_t>(kGsPer), n - i0) : 0u;
+  uint32_t u[kGsPer];
+#pragma unroll
+  for (int j = 0; j < kGsPer; ++j) u[j] = j < static_cast<int>(mine) ? ord32(scores[i0 + j]) : 0u;
+  __syncthreads();
+  // The bank of this thread's first entry (the last one starting at or before it).
+  int b0 = 0;
+  if (mine) {
+    int hi = n_banks - 1;
+    while (b0 < hi) {
+      const int mid = (b0 + hi + 1) >> 1;
+      if (s_beg[mid] <= i0) b0 = mid;
+      else hi = mid - 1;
+    }
+  }
+  // f(j, bytes of entry i0 + j) for this thread's entries in order.
+  auto for_entries = [&](auto&& f) {
+    int b = b0;
+    uint32_t next = mine ? s_beg[b + 1] : 0;
+#pragma unroll
+    for (int j = 0; j < kGsPer; ++j) {
+      if (j < static_cast<int>(mine)) {
+        while (i0 + j >= next) next = s_beg[++b + 1];
+        f(j, UNIFORM ? ubytes : s_bytes[b]);
+      }
+    }
+  };
+  uint32_t keep = 0;
+  if (keep_all) {
+    keep = (1u << mine) - 1u;
+  } else {
+    uint32_t mask = 0;
+#pragma unroll 1
+    for (int pass = 0; pass < 3; ++pass) {
+      const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0, top = pass == 2 ? 1023 : 2047;
+      for (int i = threadIdx.x; i < kGBins; i += kGsThreads) {
+        s_lo[i] = 0;
+        if (!UNIFORM) s_hi[i] = 0;
+      }
+      __syncthreads();
+      const uint32_t prefix = s_prefix;
+      const uint64_t left = s_left;
+      for_entries([&](int j, uint64_t bytes) {
+        if ((u[j] & mask) != prefix) return;
+        const uint32_t d = (u[j] >> shift) & top;
+        if (UNIFORM) {
+          atomicAdd(&s_lo[d], 1u);
+        } else {
+          const uint32_t lo = static_cast<uint32_t>(bytes);
+          const uint32_t old = atomicAdd(&s_lo[d], lo);
+          const uint32_t hi = static_cast<uint32_t>(bytes >> 32) + (old + lo < lo ? 1u : 0u);
+          if (hi) atomicAdd(&s_hi[d], hi);
+        }
+      });
+      __syncthreads();
+      // Digits from the top, two per thread: the first whose bytes overrun
+      // what is left of the budget.  (The population does not fit, so there
+      // is one.)
+      uint64_t w[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int d = top - 2 * static_cast<int>(threadIdx.x) - k;
+        w[k] = d < 0 ? 0
+                     : UNIFORM ? s_lo[d] * ubytes
+                               : s_lo[d] | (static_cast<uint64_t>(s_hi[d]) << 32);
+      }
+      uint64_t total;
+      const uint64_t incl = gs_incl_scan(w[0] + w[1], scan64, &total);
+      const int fit = __syncthreads_count(incl <= left);
+      if (static_cast<int>(threadIdx.x) == fit) {
+        const uint64_t before = incl - w[0] - w[1];
+        const int k = before + w[0] > left ? 0 : 1;
+        s_prefix = prefix | (static_cast<uint32_t>(top - 2 * fit - k) << shift);
+        s_left = left - before - (k ? w[0] : 0);
+      }
+      mask |= static_cast<uint32_t>(top) << shift;
+      __syncthreads();
+    }
+    // Every entry above the threshold, and those at it, in position order,
+    // while their bytes fit.
+    const uint32_t T = s_prefix;
+    const uint64_t left = s_left;
+    uint64_t tie = 0, total;
+    for_entries([&](int j, uint64_t bytes) {
+      if (u[j] == T) tie += bytes;
+    });
+    uint64_t at = gs_incl_scan(tie, scan64, &total) - tie;
+    for_entries([&](int j, uint64_t bytes) {
+      if (u[j] == T) at += bytes;
+      if (u[j] > T || (u[j] == T && at <= left)) keep |= 1u << j;
+    });
+  }
+  uint32_t kept;
+  const uint32_t rank = gs_incl_scan(static_cast<uint32_t>(__popc(keep)), scan32, &kept) - __popc(keep);
+  s_rank[threadIdx.x] = rank;
+  s_keep[threadIdx.x] = static_cast<uint16_t>(keep);
+  __syncthreads();
+  if (keep) {
+    uint32_t r = rank;
+    int b = b0;
+    for (uint32_t m = keep; m; m &= m - 1) {
+      const uint32_t i = i0 + __ffs(m) - 1;
+      while (i >= s_beg[b + 1]) ++b;
+      kept_idx[r++] = static_cast<int32_t>(i - s_beg[b]);
+    }
+  }
+  for (int b = threadIdx.x; b <= n_banks; b += kGsThreads) {
+    const uint32_t i = s_beg[b], t = i / kGsPer;
+    kept_off[b] = static_cast<int32_t>(
+        i >= n ? kept : s_rank[t] + __popc(s_keep[t] & ((1u << (i % kGsPer)) - 1u)));
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Copy-on-write page pool
 //
 // A page's count is the number of table slots that hold it.  A fork shares
@@ -3667,6 +3851,18 @@ cudaError_t launch_gfinish(const GPlan& p, int first_pass, int sm_count, cudaStr
   return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads), args, 0, stream);
 }
 
+
+cudaError_t launch_gsmall(const BankDesc* banks, int n_banks, uint64_t entries, const float* scores,
+                          uint64_t budget, bool uniform, bool keep_all, int32_t* kept_idx,
+                          int32_t* kept_off, cudaStream_t stream) {
+  if (entries == 0 || entries > kGSmallEntries || n_banks < 1 || n_banks > kGSmallBanks)
+    return cudaErrorInvalidValue;
+  const uint32_t n = static_cast<uint32_t>(entries);
+  return uniform ? launch_after(k_gsmall<true>, 1, kGsThreads, 0, stream, banks, n_banks, n, scores,
+                                budget, keep_all ? 1 : 0, kept_idx, kept_off)
+                 : launch_after(k_gsmall<false>, 1, kGsThreads, 0, stream, banks, n_banks, n, scores,
+                                budget, keep_all ? 1 : 0, kept_idx, kept_off);
+}
 
 cudaError_t launch_selftest_wait(int which, const uint32_t* never_set, uint32_t* err,
                                  cudaStream_t stream) {

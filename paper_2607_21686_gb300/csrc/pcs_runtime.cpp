@@ -2043,6 +2043,26 @@ static pcs_status prune_global_impl(pcs_ctx* c, const pcs_bank* banks, int32_t n
     PCS_CUDA(cudaMemsetAsync(kept_off, 0, 4ull * (n + 1), stream));
     return PCS_OK;
   }
+  if (!ex && entries <= kGSmallEntries && n <= kGSmallBanks) {
+    // Small: a plain score pass, then one block (its descriptors are the
+    // banks' alone).
+    const uint64_t o_sc = round_up(sizeof(BankDesc) * n, kRecordAlign);
+    uint8_t* ws = nullptr;
+    st = ws_acquire(c, o_sc + (scores ? 0 : 4ull * entries), stream, &ws);
+    if (st) return st;
+    c->plan.resize(o_sc);
+    put(c->plan, 0, d);
+    PCS_CUDA(plan_copy(c, ws, sizeof(BankDesc) * n, stream));
+    float* sc = scores ? scores : reinterpret_cast<float*>(ws + o_sc);
+    const auto* dbanks = reinterpret_cast<const BankDesc*>(ws);
+    PCS_CUDA(launch_bank_scores(c, banks, n, dbanks, entries, sc, stream));
+    {
+      LaunchScope ls(c, kKGFinish, stream);
+      PCS_CUDA(launch_gsmall(dbanks, n, entries, sc, budget, uniform, total <= budget, kept_idx,
+                             kept_off, stream));
+    }
+    return ws_release(c, stream);
+  }
   const uint64_t tiles = (entries + kGTile - 1) / kGTile;
   // Bank of entry min(t * kGTile, entries - 1), t = 0..tiles.
   std::vector<uint32_t> tile_bank(tiles + 1);

@@ -234,3 +234,32 @@ def test_scores_of_every_shape(ctx, dev, dims, dtype):
         nan = np.isnan(want)  # which NaN is not defined
         assert np.array_equal(np.isnan(got), nan)
         assert np.array_equal(got[~nan].view(np.uint32), want[~nan].view(np.uint32))
+
+
+# The one-block global threshold at its limits (16,384 entries, 1,024 banks) and
+# just past them: runs of ties across threads and banks, banks of one entry and
+# empty ones, entry bytes of no byte, of few and past 32 bits.
+@pytest.mark.parametrize("entries,n_banks", [(1, 1), (15, 3), (16, 16), (16384, 1), (16385, 1),
+                                             (16384, 1024), (16380, 1025), (5000, 700)])
+@pytest.mark.parametrize("kind", ["uniform", "mixed", "wide"])
+def test_global_threshold_of_small_populations(ctx, dev, entries, n_banks, kind):
+    rnd = np.random.default_rng(entries + n_banks)
+    cuts = np.sort(rnd.integers(0, entries + 1, n_banks - 1))
+    sizes = np.diff(np.concatenate([[0], cuts, [entries]])).tolist()
+    pick = torch.randn(40, 16, generator=torch.Generator().manual_seed(entries)).half()
+    keys = [pick[torch.from_numpy(rnd.integers(0, 40, s))] for s in sizes]
+    q = pick[3] + pick[5]
+    eb = {"uniform": [48] * n_banks, "mixed": rnd.integers(0, 5000, n_banks).tolist(),
+          "wide": ((1 << 32) + rnd.integers(-2, 1 << 20, n_banks)).tolist()}[kind]
+    s32 = np.concatenate([oracle.scores(np_view(q), np_view(k)) for k in keys if len(k)])
+    dk, dq = [k.to(dev) for k in keys], q.to(dev)
+    banks = ctx.banks_array(dk, [dq] * n_banks, eb)
+    total = sum(a * b for a, b in zip(sizes, eb))
+    for budget in sorted({0, min(eb), total // 3, total * 2 // 3 + 1, max(total - 1, 0), total}):
+        kept = torch.full((entries,), -7, dtype=torch.int32, device=dev)
+        off = torch.full((n_banks + 1,), -7, dtype=torch.int32, device=dev)
+        ctx.prune_global(banks, n_banks, budget, kept, off)
+        want, woff = oracle.prune_global(s32, sizes, eb, budget)
+        assert off.cpu().tolist() == woff.tolist(), budget
+        assert kept.cpu().tolist()[:woff[-1]] == want.tolist(), budget
+    ctx.sync()
