@@ -132,17 +132,33 @@ cudaError_t launch_stream(int mode, const SecDesc* secs, WorkList wl, int group_
 cudaError_t launch_bulk(int mode, bool shift, const SecDesc* secs, WorkList wl, uint64_t* nodes,
                         uint32_t* dev_err, uint32_t* sched, int sm_count, cudaStream_t stream);
 
-// One launch for a small call: the register streaming pass over wl (no
+// One launch for a small call: the register streaming pass over its tasks (no
 // node reduction) and the finalisation of `mode` (hash: n_items buffers; pack
 // / restore_verify: n_items sessions of at most max_secs sections), each item
 // by the warp that completes it.  `ticket` and `done` (a word per item, at
 // most kSmallMaxItems) are zero on entry and on exit.
 constexpr int kSmallMaxItems = 64;
-cudaError_t launch_small(int mode, const SecDesc* secs, WorkList wl, int group_log2,
-                         uint64_t* nodes, uint32_t* dev_err, uint32_t* ticket, uint32_t* done,
-                         int n_items, int max_secs, const SessDesc* sess, const Entry* entries,
-                         uint64_t* fp_out, const uint64_t* fp_before, uint8_t* flags,
-                         uint32_t* bad, int sm_count, int blocks_per_sm, cudaStream_t stream);
+constexpr uint64_t kSmallPlanMax = 31744;  // descriptors that travel as a kernel parameter
+struct SmallArgs {
+  const uint8_t* plan;     // the descriptors on the device (not read if they are a parameter)
+  uint32_t o_secs, o_sess, o_entries, o_ids, o_begin;  // offsets in the descriptors
+  int32_t n_list;          // work list items
+  uint32_t n_tasks;
+  int32_t glog2;
+  uint64_t* nodes;
+  uint32_t* err;
+  uint32_t* ticket;
+  uint32_t* done;
+  int32_t n_items, max_secs;
+  uint64_t* fp_out;
+  const uint64_t* fp_before;
+  uint8_t* flags;
+  uint32_t* bad;
+};
+// host_plan: the descriptors (`bytes` of them, at most kSmallPlanMax, in
+// memory readable to kSmallPlanMax), sent with the launch; null: a.plan.
+cudaError_t launch_small(int mode, const uint8_t* host_plan, uint64_t bytes, const SmallArgs& a,
+                         int sm_count, int blocks_per_sm, cudaStream_t stream);
 
 // One level of the node reduction of stream i: count nodes at src, reduced
 // by aligned groups of 32 to ceil(count / 32) nodes at dst.

@@ -74,6 +74,14 @@ __device__ __forceinline__ uint64_t ld_l2(const uint64_t* p) {
   return __ldcg(reinterpret_cast<const unsigned long long*>(p));
 }
 
+// A word of a call's descriptors: from the workspace (GLOBAL), through the
+// read-only path, or from where else they are (a kernel parameter).
+template <bool GLOBAL, typename T>
+__device__ __forceinline__ T fetch(const T* p) {
+  if constexpr (GLOBAL) return __ldg(p);
+  else return *p;
+}
+
 // A hint to bring the 128-byte line holding `p` into this SM's L1.
 __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
@@ -519,13 +527,14 @@ __device__ __forceinline__ uint64_t move_chunks(const SecDesc& s, uint64_t c, in
 // warp-uniform task: each round the lanes probe 32 evenly spaced entries of
 // the range still open and keep the part after the last probe <= task, so
 // that 12,544 items take three dependent loads instead of fourteen.
-__device__ __forceinline__ int find_item(const uint32_t* __restrict__ begin, int lo, int n_items,
-                                        uint32_t task, int lane) {
+template <bool GLOBAL = true>
+__device__ __forceinline__ int find_item(const uint32_t* begin, int lo, int n_items, uint32_t task,
+                                         int lane) {
   int span = n_items - lo;  // the answer lies in [lo, lo + span)
   while (span > 1) {
     const int step = (span + 31) >> 5;
     const int i = lo + lane * step;
-    const bool le = i < lo + span && __ldg(begin + i) <= task;
+    const bool le = i < lo + span && fetch<GLOBAL>(begin + i) <= task;
     const unsigned m = __ballot_sync(kFull, le);  // lane 0 probes lo: never empty
     const int last = 31 - __clz(m);
     lo += last * step;
@@ -546,8 +555,8 @@ __device__ __forceinline__ int find_item(const uint32_t* __restrict__ begin, int
 // an odd address 1,263 -> 220 us (4.9 TB/s), at a 4-byte one 405 -> 220 us;
 // 2,000 observations of 196,613 bytes, three of four off a boundary: pack 693 ->
 // 184 us, verified restore 862 -> 211 us.
-template <int MODE, typename F>
-__device__ __forceinline__ void run_stream_tasks(const SecDesc* __restrict__ secs, const WorkList& wl,
+template <int MODE, bool GLOBAL, typename F>
+__device__ __forceinline__ void run_stream_tasks(const SecDesc* secs, const WorkList& wl,
                                                  int glog2, uint64_t* __restrict__ nodes,
                                                  uint32_t* err, SecDesc* sdesc, F&& after_task) {
   using T = ModeTraits<MODE>;
@@ -561,19 +570,20 @@ __device__ __forceinline__ void run_stream_tasks(const SecDesc* __restrict__ sec
   // read before waiting for the kernel ahead.
   const SecDesc& s = sdesc[wib];
   auto load_desc = [&](int j) {
-    const SecDesc* src = &secs[__ldg(wl.ids + j)];
+    const SecDesc* src = &secs[fetch<GLOBAL>(wl.ids + j)];
     __syncwarp();
     if (lane < static_cast<int>(sizeof(SecDesc) / 16))
-      reinterpret_cast<uint4*>(&sdesc[wib])[lane] = __ldg(reinterpret_cast<const uint4*>(src) + lane);
+      reinterpret_cast<uint4*>(&sdesc[wib])[lane] =
+          fetch<GLOBAL>(reinterpret_cast<const uint4*>(src) + lane);
     __syncwarp();
   };
   int j = 0, cur = -1;
-  if (t0 < t1) load_desc(cur = j = find_item(wl.begin, 0, wl.n_items, t0, lane));
+  if (t0 < t1) load_desc(cur = j = find_item<GLOBAL>(wl.begin, 0, wl.n_items, t0, lane));
   grid_dependency();
   for (uint32_t task = t0; task < t1; ++task) {
-    while (j + 1 < wl.n_items && __ldg(wl.begin + j + 1) <= task) ++j;
+    while (j + 1 < wl.n_items && fetch<GLOBAL>(wl.begin + j + 1) <= task) ++j;
     if (j != cur) load_desc(cur = j);
-    const uint32_t local = task - __ldg(wl.begin + j);
+    const uint32_t local = task - fetch<GLOBAL>(wl.begin + j);
     const uint64_t c0 = static_cast<uint64_t>(local) << glog2;
     const uint64_t c1 = min(c0 + (1ull << glog2), static_cast<unsigned long long>(s.n_chunks));
     // A pair whose chunks and neighbouring vectors lie inside the stream takes
@@ -598,7 +608,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     k_stream(const SecDesc* __restrict__ secs, WorkList wl, int glog2,
              uint64_t* __restrict__ nodes, uint32_t* err) {
   __shared__ SecDesc sdesc[kWarps];
-  run_stream_tasks<MODE>(secs, wl, glog2, nodes, err, sdesc, [](const SecDesc&, int) {});
+  run_stream_tasks<MODE, true>(secs, wl, glog2, nodes, err, sdesc, [](const SecDesc&, int) {});
 }
 
 // ---------------------------------------------------------------------------
@@ -1322,9 +1332,8 @@ __device__ uint64_t session_fp(const uint64_t* fps, uint32_t stride, uint32_t n,
 // Restore with verification: compare recomputed fps with the record.
 // The whole block handles sessions b0, b0 + stride, ...
 template <int MODE>
-__device__ void finalize_sessions_block(const SecDesc* __restrict__ secs,
-                                        const SessDesc* __restrict__ sess, int n_sess,
-                                        const Entry* __restrict__ entries, uint64_t* nodes,
+__device__ void finalize_sessions_block(const SecDesc* secs, const SessDesc* sess, int n_sess,
+                                        const Entry* entries, uint64_t* nodes,
                                         uint8_t* corrupt, uint32_t* bad, int b0, int stride,
                                         uint64_t* smem, uint32_t* s_bad) {
   const int lane = threadIdx.x & 31;
@@ -1418,23 +1427,22 @@ struct SessLane {
   uint64_t bytes;                 // and its length
 };
 
-__device__ __forceinline__ SessLane session_lane(const SessDesc& S, const SecDesc* __restrict__ secs,
-                                                 int lane) {
+template <bool GLOBAL = true>
+__device__ __forceinline__ SessLane session_lane(const SessDesc& S, const SecDesc* secs, int lane) {
   SessLane l{0, 0, 0};
   if (lane < static_cast<int>(S.n_sections)) {
     const SecDesc* sj = secs + S.sec_begin + lane;
-    l.fin_begin = __ldg(&sj->fin_begin);
-    l.fin_count = __ldg(&sj->fin_count);
-    l.bytes = __ldg(reinterpret_cast<const unsigned long long*>(&sj->bytes));
+    l.fin_begin = fetch<GLOBAL>(&sj->fin_begin);
+    l.fin_count = fetch<GLOBAL>(&sj->fin_count);
+    l.bytes = fetch<GLOBAL>(reinterpret_cast<const unsigned long long*>(&sj->bytes));
   }
   return l;
 }
 
 template <int MODE, bool L2>
 __device__ __forceinline__ void finalize_session_warp(const SessDesc& S, const SessLane& l, int b,
-                                                      const Entry* __restrict__ entries,
-                                                      uint64_t* nodes, uint8_t* corrupt,
-                                                      uint32_t* bad, int lane) {
+                                                      const Entry* entries, uint64_t* nodes,
+                                                      uint8_t* corrupt, uint32_t* bad, int lane) {
   Entry* table = reinterpret_cast<Entry*>(S.record + kHeaderBytes);
   const int ns = static_cast<int>(S.n_sections);
   // A restore's stored fps (lane j: section j's), read once; each section's
@@ -1535,41 +1543,59 @@ __global__ void __launch_bounds__(kThreads)
 // a time -> this): 34 sessions of 14,280 bytes pack 50.6 -> 6.0 us, verified
 // restore 56.7 -> 6.8 us; 64 of 10,000 bytes 89.4 -> 5.5 and 99.8 -> 5.6 us; one
 // of 196,608 bytes 6.2 and 6.3 us either way.
-template <int MODE>
+//
+// BYTES > 0: the call's descriptors travel as a kernel parameter of that size
+// (`blob`; launch_small picks the smallest that holds them), else they are at
+// a.plan in the workspace, where a copy engine put them ahead of the launch:
+// the copy, and the hand-over from copy engine to kernel, cost a call
+// more than its kernel.  Measured, checkpoint + verified restore + delete of
+// one session of 196,608 bytes 31.4 -> 20.1 us, of 34 small ones 31.7 -> 25.8,
+// of 64 (27 KB of descriptors) 36.2 -> 31.5; fingerprints of 8 buffers 11.1 -> 5.8.
+template <int BYTES>
+struct PlanBlob {
+  alignas(16) uint8_t b[BYTES > 0 ? BYTES : 16];
+};
+
+template <int MODE, int BYTES>
 __global__ void __launch_bounds__(kThreads, 2)
-    k_small(const SecDesc* __restrict__ secs, WorkList wl, int glog2, uint64_t* nodes,
-            uint32_t* err, uint32_t* ticket, uint32_t* done, int n_items, int max_secs,
-            const SessDesc* __restrict__ sess, const Entry* __restrict__ entries, uint64_t* fp_out,
-            const uint64_t* fp_before, uint8_t* flags, uint32_t* bad) {
+    k_small(const __grid_constant__ PlanBlob<BYTES> blob, const SmallArgs a) {
+  constexpr bool GLOBAL = BYTES == 0;
+  const uint8_t* plan = GLOBAL ? a.plan : blob.b;
+  const SecDesc* secs = reinterpret_cast<const SecDesc*>(plan + a.o_secs);
+  const SessDesc* sess = reinterpret_cast<const SessDesc*>(plan + a.o_sess);
+  const Entry* entries = reinterpret_cast<const Entry*>(plan + a.o_entries);
+  const WorkList wl{reinterpret_cast<const uint32_t*>(plan + a.o_ids),
+                    reinterpret_cast<const uint32_t*>(plan + a.o_begin), a.n_list, a.n_tasks};
+  uint64_t* nodes = a.nodes;
   __shared__ SecDesc sdesc[kWarps];
   const int lane = threadIdx.x & 31;
-  if (MODE == kModeHash || max_secs <= 32) {
-    run_stream_tasks<MODE>(secs, wl, glog2, nodes, err, sdesc, [&](const SecDesc& s, int j) {
-      const uint32_t i = MODE == kModeHash ? __ldg(wl.ids + j) : s.sess;
+  if (MODE == kModeHash || a.max_secs <= 32) {
+    run_stream_tasks<MODE, GLOBAL>(secs, wl, a.glog2, nodes, a.err, sdesc, [&](const SecDesc& s, int j) {
+      const uint32_t i = MODE == kModeHash ? fetch<GLOBAL>(wl.ids + j) : s.sess;
       SessDesc S{};
       SessLane l{};
       if (MODE != kModeHash) {
         S = sess[i];
-        l = session_lane(S, secs, lane);
+        l = session_lane<GLOBAL>(S, secs, lane);
       }
       const uint32_t total = MODE == kModeHash ? s.n_tasks : S.n_tasks;
       uint32_t before = 0;
       if (lane == 0) {
         __threadfence();  // the task's node, before it counts as done
-        before = atomicAdd(done + i, 1u);
+        before = atomicAdd(a.done + i, 1u);
       }
       if (__shfl_sync(kFull, before, 0) + 1 != total) return;
       __threadfence();
-      if (lane == 0) done[i] = 0;
+      if (lane == 0) a.done[i] = 0;
       if (MODE == kModeHash) {
         const uint64_t fp = stream_fp<true>(s, nodes, lane);
         if (lane == 0) {
-          if (fp_out) fp_out[i] = fp;
-          if (fp_before) flags[i] = fp != fp_before[i] ? 1 : 0;
+          if (a.fp_out) a.fp_out[i] = fp;
+          if (a.fp_before) a.flags[i] = fp != a.fp_before[i] ? 1 : 0;
         }
       } else {
         finalize_session_warp<MODE == kModeHash ? kModePack : MODE, true>(
-            S, l, static_cast<int>(i), entries, nodes, nullptr, bad, lane);
+            S, l, static_cast<int>(i), entries, nodes, nullptr, a.bad, lane);
       }
     });
     return;
@@ -1577,17 +1603,17 @@ __global__ void __launch_bounds__(kThreads, 2)
   __shared__ uint64_t smem[64];  // up to 2048 sections per session
   __shared__ uint32_t s_bad;
   __shared__ bool s_last;
-  run_stream_tasks<MODE>(secs, wl, glog2, nodes, err, sdesc, [](const SecDesc&, int) {});
+  run_stream_tasks<MODE, GLOBAL>(secs, wl, a.glog2, nodes, a.err, sdesc, [](const SecDesc&, int) {});
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  if (threadIdx.x == 0) s_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
   if (MODE != kModeHash)
-    finalize_sessions_block<MODE>(secs, sess, n_items, entries, nodes, nullptr, bad, 0, 1, smem,
+    finalize_sessions_block<MODE>(secs, sess, a.n_items, entries, nodes, nullptr, a.bad, 0, 1, smem,
                                   &s_bad);
-  if (threadIdx.x == 0) *ticket = 0;
+  if (threadIdx.x == 0) *a.ticket = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -3594,24 +3620,44 @@ cudaError_t launch_bulk(int mode, bool shift, const SecDesc* secs, WorkList wl, 
   }
 }
 
-cudaError_t launch_small(int mode, const SecDesc* secs, WorkList wl, int group_log2,
-                         uint64_t* nodes, uint32_t* dev_err, uint32_t* ticket, uint32_t* done,
-                         int n_items, int max_secs, const SessDesc* sess, const Entry* entries,
-                         uint64_t* fp_out, const uint64_t* fp_before, uint8_t* flags,
-                         uint32_t* bad, int sm_count, int blocks_per_sm, cudaStream_t stream) {
-  if (wl.n_tasks == 0) return cudaErrorInvalidValue;
-  const uint64_t want = (static_cast<uint64_t>(wl.n_tasks) + kWarps - 1) / kWarps;
+template <int MODE, int BYTES>
+static cudaError_t launch_small_mode(const uint8_t* host_plan, SmallArgs a, int blocks,
+                                     cudaStream_t stream) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  static const PlanBlob<0> none{};
+  const void* blob = BYTES > 0 ? static_cast<const void*>(host_plan) : static_cast<const void*>(&none);
+  void* args[] = {const_cast<void*>(blob), &a};
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(k_small<MODE, BYTES>), args);
+}
+
+template <int MODE>
+static cudaError_t launch_small_size(const uint8_t* host_plan, uint64_t bytes, const SmallArgs& a,
+                                     int blocks, cudaStream_t stream) {
+  static_assert(kSmallPlanMax == 31744, "the largest parameter below");
+  if (!host_plan) return launch_small_mode<MODE, 0>(host_plan, a, blocks, stream);
+  if (bytes <= 1008) return launch_small_mode<MODE, 1008>(host_plan, a, blocks, stream);
+  if (bytes <= 7936) return launch_small_mode<MODE, 7936>(host_plan, a, blocks, stream);
+  return launch_small_mode<MODE, 31744>(host_plan, a, blocks, stream);
+}
+
+cudaError_t launch_small(int mode, const uint8_t* host_plan, uint64_t bytes, const SmallArgs& a,
+                         int sm_count, int blocks_per_sm, cudaStream_t stream) {
+  if (a.n_tasks == 0 || (host_plan && bytes > kSmallPlanMax)) return cudaErrorInvalidValue;
+  const uint64_t want = (static_cast<uint64_t>(a.n_tasks) + kWarps - 1) / kWarps;
   const uint64_t cap = static_cast<uint64_t>(sm_count) * blocks_per_sm;
   const int blocks = static_cast<int>(want < cap ? want : cap);
-  auto launch = [&](auto kernel) {
-    return launch_after(kernel, blocks, kThreads, 0, stream, secs, wl, group_log2, nodes, dev_err,
-                        ticket, done, n_items, max_secs, sess, entries, fp_out, fp_before, flags,
-                        bad);
-  };
   switch (mode) {
-    case kModeHash: return launch(k_small<kModeHash>);
-    case kModePack: return launch(k_small<kModePack>);
-    case kModeRestoreV: return launch(k_small<kModeRestoreV>);
+    case kModeHash: return launch_small_size<kModeHash>(host_plan, bytes, a, blocks, stream);
+    case kModePack: return launch_small_size<kModePack>(host_plan, bytes, a, blocks, stream);
+    case kModeRestoreV: return launch_small_size<kModeRestoreV>(host_plan, bytes, a, blocks, stream);
     default: return cudaErrorInvalidValue;
   }
 }

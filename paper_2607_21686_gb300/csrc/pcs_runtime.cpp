@@ -1089,6 +1089,28 @@ void put_lists(std::vector<uint8_t>& plan, const StreamPlan& P, const ListLayout
   put_lists(plan.data(), P, L);
 }
 
+// Does a small call's plan travel with its launch, as a kernel parameter?
+bool plan_in_launch(bool fused, uint64_t bytes) { return fused && bytes <= kSmallPlanMax; }
+
+// The arguments of a small call's one kernel: descriptors at ws (or with the
+// launch), nodes, header words.
+SmallArgs small_args(pcs_ctx* c, const StreamPlan& P, const ListLayout& L, uint8_t* ws,
+                     uint64_t* nodes, uint32_t* words, int n_items) {
+  SmallArgs a{};
+  a.plan = ws;
+  a.o_ids = static_cast<uint32_t>(L.reg_ids);
+  a.o_begin = static_cast<uint32_t>(L.reg_begin);
+  a.n_list = static_cast<int32_t>(P.reg_ids.size());
+  a.n_tasks = P.reg_tasks;
+  a.glog2 = P.glog2;
+  a.nodes = nodes;
+  a.err = c->words;
+  a.ticket = words;
+  a.done = words + kWordDone;
+  a.n_items = n_items;
+  return a;
+}
+
 // Launch both streaming kernels of a plan (TMA-staged first).
 cudaError_t launch_streams(pcs_ctx* c, int mode, const SecDesc* dsecs, const StreamPlan& P,
                            const ListLayout& L, uint8_t* ws, uint64_t* nodes,
@@ -1132,20 +1154,21 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
   uint8_t* ws = nullptr;
   pcs_status st = ws_acquire(c, L.total, stream, &ws);
   if (st) return st;
-  c->plan.resize(L.nodes);
+  const bool sent = plan_in_launch(fused, LL.end);
+  c->plan.resize(sent ? kSmallPlanMax : L.nodes);
   put(c->plan, L.secs, d);
   put_lists(c->plan, P, LL);
-  PCS_CUDA(plan_copy(c, ws, L.nodes, stream));
+  if (!sent) PCS_CUDA(plan_copy(c, ws, L.nodes, stream));
   auto* dsecs = reinterpret_cast<const SecDesc*>(ws + L.secs);
   auto* nodes = reinterpret_cast<uint64_t*>(ws + L.nodes);
   if (fused) {
-    WorkList wl{reinterpret_cast<const uint32_t*>(ws + LL.reg_ids),
-                reinterpret_cast<const uint32_t*>(ws + LL.reg_begin),
-                static_cast<int>(P.reg_ids.size()), P.reg_tasks};
+    SmallArgs a = small_args(c, P, LL, ws, nodes, c->call_words, n);
+    a.fp_out = fp_out;
+    a.fp_before = fp_before;
+    a.flags = flags;
     LaunchScope ls(c, kKStreamHash, stream);
-    PCS_CUDA(launch_small(kModeHash, dsecs, wl, P.glog2, nodes, c->words, c->call_words,
-                          c->call_words + kWordDone, n, 0, nullptr, nullptr, fp_out, fp_before,
-                          flags, nullptr, c->sm_count, c->stream_bps, stream));
+    PCS_CUDA(launch_small(kModeHash, sent ? c->plan.data() : nullptr, LL.end, a, c->sm_count,
+                          c->stream_bps, stream));
     return ws_release(c, stream);
   }
   PCS_CUDA(launch_streams(c, kModeHash, dsecs, P, LL, ws, nodes, stream));
@@ -1220,6 +1243,7 @@ void drop_snapshot(pcs_ctx* c, pcs_snapshot* h) {
 struct Prepared {
   int mode = kModePack;  // kModePack, kModeRestore, kModeRestoreV
   bool fused = false;    // one k_small launch (small calls)
+  bool in_launch = false;  // with the descriptors as its parameter, not in the workspace
   int verify = 0;        // restore: 0, 1 or 2
   int32_t n = 0;         // sessions
   int32_t max_secs = 0;  // most sections in one session
@@ -1231,10 +1255,14 @@ struct Prepared {
 
 // The bytes [0, L.nodes) of a plan's descriptors: a plain call writes them
 // straight into a pinned plan slot (one copy less; plan_send then sends
-// them), a prepared call into pr->plan, which it keeps.
+// them), or into pr->plan if they travel with its launch; a prepared call into
+// pr->plan, which it keeps, and from there to the device once: a run that
+// sent them with its launch again was 4 % slower (8 sessions).
 uint8_t* plan_target(pcs_ctx* c, Prepared* pr, bool to_slot) {
-  if (to_slot) return plan_dst(c, pr->L.nodes, pr->plan);
-  pr->plan.resize(pr->L.nodes);
+  pr->in_launch = to_slot && plan_in_launch(pr->fused, pr->LL.end);
+  if (to_slot && !pr->in_launch) return plan_dst(c, pr->L.nodes, pr->plan);
+  if (to_slot) c->plan_slot_used = -1;
+  pr->plan.resize(pr->in_launch ? kSmallPlanMax : pr->L.nodes);
   return pr->plan.data();
 }
 
@@ -1282,16 +1310,20 @@ cudaError_t launch_prepared(pcs_ctx* c, const Prepared& pr, uint8_t* ws, uint32_
   const auto* dsecs = reinterpret_cast<const SecDesc*>(ws + pr.L.secs);
   const auto* dsess = reinterpret_cast<const SessDesc*>(ws + pr.L.sess);
   auto* nodes = reinterpret_cast<uint64_t*>(ws + pr.L.nodes);
-  WorkList wl{reinterpret_cast<const uint32_t*>(ws + pr.LL.reg_ids),
-              reinterpret_cast<const uint32_t*>(ws + pr.LL.reg_begin),
-              static_cast<int>(pr.P.reg_ids.size()), pr.P.reg_tasks};
+  const uint8_t* sent = pr.in_launch ? pr.plan.data() : nullptr;
+  auto args = [&]() {
+    SmallArgs a = small_args(c, pr.P, pr.LL, ws, nodes, words, pr.n);
+    a.o_secs = static_cast<uint32_t>(pr.L.secs);
+    a.o_sess = static_cast<uint32_t>(pr.L.sess);
+    a.o_entries = static_cast<uint32_t>(pr.L.entries);
+    a.max_secs = pr.max_secs;
+    return a;
+  };
   if (pr.mode == kModePack) {
     const auto* dent = reinterpret_cast<const Entry*>(ws + pr.L.entries);
     if (pr.fused) {
       LaunchScope ls(c, kKStreamPack, stream);
-      return launch_small(kModePack, dsecs, wl, pr.P.glog2, nodes, c->words, words,
-                          words + kWordDone, pr.n, pr.max_secs, dsess, dent, nullptr, nullptr,
-                          nullptr, nullptr, c->sm_count, c->stream_bps, stream);
+      return launch_small(kModePack, sent, pr.LL.end, args(), c->sm_count, c->stream_bps, stream);
     }
     cudaError_t e = launch_streams(c, kModePack, dsecs, pr.P, pr.LL, ws, nodes, stream);
     if (e != cudaSuccess) return e;
@@ -1302,9 +1334,9 @@ cudaError_t launch_prepared(pcs_ctx* c, const Prepared& pr, uint8_t* ws, uint32_
   uint32_t* bad = pr.verify == 1 ? words + 1 : c->words + 2;
   if (pr.fused) {
     LaunchScope ls(c, kKStreamRestoreV, stream);
-    return launch_small(kModeRestoreV, dsecs, wl, pr.P.glog2, nodes, c->words, words,
-                        words + kWordDone, pr.n, pr.max_secs, dsess, nullptr, nullptr, nullptr,
-                        nullptr, bad, c->sm_count, c->stream_bps, stream);
+    SmallArgs a = args();
+    a.bad = bad;
+    return launch_small(kModeRestoreV, sent, pr.LL.end, a, c->sm_count, c->stream_bps, stream);
   }
   cudaError_t e = launch_streams(c, pr.verify ? kModeRestoreV : kModeRestore, dsecs, pr.P, pr.LL,
                                  ws, pr.verify ? nodes : nullptr, stream);
@@ -2255,7 +2287,8 @@ pcs_status pcs_checkpoint(pcs_ctx* c, const pcs_session* sessions, int32_t n, ui
   uint8_t* ws = nullptr;
   st = ws_acquire(c, pr.L.total, stream, &ws);
   if (st) return undo(st);
-  cudaError_t e = plan_send(c, ws, pr.L.nodes, pr.plan, stream);
+  cudaError_t e = cudaSuccess;
+  if (!pr.in_launch) e = plan_send(c, ws, pr.L.nodes, pr.plan, stream);
   if (e == cudaSuccess) e = launch_prepared(c, pr, ws, c->call_words, stream);
   if (e != cudaSuccess) return undo(cuda_fail(e, "checkpoint launch"));
   blk->written = record_event(c->events, stream);
@@ -2395,7 +2428,7 @@ pcs_status pcs_restore(pcs_ctx* c, pcs_snapshot* const* snaps, int32_t n, const 
   uint8_t* ws = nullptr;
   st = ws_acquire(c, pr.L.total, stream, &ws);
   if (st) return st;
-  PCS_CUDA(plan_send(c, ws, pr.L.nodes, pr.plan, stream));
+  if (!pr.in_launch) PCS_CUDA(plan_send(c, ws, pr.L.nodes, pr.plan, stream));
   // verify == 1: count failures of this call in words[1] and wait for them;
   // verify == 2: accumulate them in words[2] for the next pcs_sync.
   uint32_t* words = c->call_words;
