@@ -5,6 +5,7 @@
 
 #include <atomic>
 #include <cstdint>
+#include <cstring>
 
 #include <cuda_runtime.h>
 
@@ -184,8 +185,18 @@ cudaError_t launch_finalize(int mode, const SecDesc* secs, const SessDesc* sess,
 
 
 
-cudaError_t launch_topk(const BankDesc* banks, int n_banks, const float* scores,
-                        int32_t* kept_idx, cudaStream_t stream);
+// The banks of a call: on the device, or (dev null, at most kBankBlob of them)
+// in host memory, to travel with the launch.
+constexpr int kBankBlob = 60;  // 3,840 bytes
+struct Banks {
+  const BankDesc* host;
+  const BankDesc* dev;
+  int n;
+};
+// Kept indices per bank; with kept_off, also the offsets of the lists
+// (kept_off[n] = kept_total).
+cudaError_t launch_topk(const Banks& banks, const float* scores, int32_t* kept_idx,
+                        int32_t* kept_off, int32_t kept_total, cudaStream_t stream);
 // One thread waits for what never happens (which = 0: an mbarrier's second
 // arrival; 1: *never_set >= 1), gives up after the kernels' wait bound and
 // sets the timeout bit in *err.
@@ -255,8 +266,8 @@ struct GPlan {
 // Scores of every entry; with gh.st set (and a fixed-width kernel), also the
 // first digit pass of the global threshold.  Returns through *fused whether
 // that pass was done.
-cudaError_t launch_score(const BankDesc* banks, int n_banks, uint64_t n_entries, int max_dim,
-                         int key_types, float* scores, int sm_count, cudaStream_t stream,
+cudaError_t launch_score(const Banks& banks, uint64_t n_entries, int max_dim, int key_types,
+                         float* scores, int sm_count, cudaStream_t stream,
                          GHist gh = GHist{}, bool* fused = nullptr);
 
 // The bins of pass `pass` (0..kGPasses-1) of the byte-weighted radix select
@@ -272,8 +283,8 @@ cudaError_t launch_gfinish(const GPlan& p, int first_pass, int sm_count, cudaStr
 // one block.  keep_all: the budget does not bind.
 constexpr uint64_t kGSmallEntries = 16384;
 constexpr int kGSmallBanks = 1024;
-cudaError_t launch_gsmall(const BankDesc* banks, int n_banks, uint64_t entries, const float* scores,
-                          uint64_t budget, bool uniform, bool keep_all, int32_t* kept_idx,
+cudaError_t launch_gsmall(const Banks& banks, uint64_t entries, const float* scores, uint64_t budget,
+                          bool uniform, bool keep_all, int32_t* kept_idx,
                           int32_t* kept_off, cudaStream_t stream);
 
 // ---- Copy-on-write page pool (pcs_pool_*) ---------------------------------
@@ -311,13 +322,36 @@ struct MmPair {
   uint32_t shift;       // offset of b from a 16-byte boundary
 };
 
+// The plan of a call as k_mismatch's parameter: up to N pairs, or where they
+// are on the device.  extra: the bytes only one buffer of a pair has.
+constexpr int kMmBlob = 512;  // pairs that travel with a launch at most (24.6 KB)
+template <int N>
+struct MmBlob {
+  MmPair pair[N];
+  uint64_t unit_begin[N + 1];
+  uint64_t extra[N];
+  __host__ __device__ const MmPair* pairs() const { return pair; }
+  __host__ __device__ const uint64_t* begins() const { return unit_begin; }
+  __host__ __device__ uint64_t more(int i) const { return extra[i]; }
+};
+template <>
+struct MmBlob<0> {
+  const MmPair* pair;
+  const uint64_t* unit_begin;
+  __host__ __device__ const MmPair* pairs() const { return pair; }
+  __host__ __device__ const uint64_t* begins() const { return unit_begin; }
+  __host__ __device__ uint64_t more(int) const { return 0; }
+};
+
 // Pair i owns units [unit_begin[i], unit_begin[i+1]) (units of kMmUnit bytes
-// after its head; at least one if it compares any byte).  sums[i] starts at
-// the count to add the mismatches to; counts[i] = the total.  `ticket`: a
+// after its head; at least one if it compares any byte); counts[i] = its
+// mismatches and extra bytes.  host (at most kMmBlob pairs): the arrays are in
+// host memory and travel with the launch; sums are zero on entry and on exit.
+// Else they are on the device and sums[i] = extra[i] on entry.  `ticket`: a
 // device word, zero on entry and on exit.
-cudaError_t launch_mismatch(const MmPair* pairs, const uint64_t* unit_begin, int32_t n,
-                            uint64_t units, uint64_t* sums, uint64_t* counts, uint32_t* ticket,
-                            int sm_count, cudaStream_t stream);
+cudaError_t launch_mismatch(bool host, const MmPair* pairs, const uint64_t* unit_begin,
+                            const uint64_t* extra, int32_t n, uint64_t units, uint64_t* sums,
+                            uint64_t* counts, uint32_t* ticket, int sm_count, cudaStream_t stream);
 
 // ---- Reads against buffers (pcs_classify_reads) ---------------------------
 // The non-empty buffers sorted by start; maxend[i] = max(end[0..i]).
@@ -334,9 +368,42 @@ struct ReadPlan {
   int32_t slices;         // set by the launcher: slices of the address range
   int32_t slice_shift;    // and log2 of their bytes
 };
-// flags[i] = a read overlaps buffer i; every flag is written.  m > 0.
-cudaError_t launch_classify_reads(ReadPlan p, const uint64_t* addr, const uint64_t* bytes,
-                                  int64_t m, uint8_t* flags, int sm_count, cudaStream_t stream);
+// A plan's arrays as k_classify_reads' parameter: up to N buffers, or nothing
+// (they are where the plan points, on the device).
+// Buffers that travel with a launch at most (3.6 KB): every block stages the
+// arrays, from the constant bank an element at a time (765 buffers and 2,268
+// blocks took 30.7 us that way, 15.9 us from the workspace; 128 and fewer gain
+// at every length of the log).
+constexpr int kReadBlob = 128;
+template <int N>
+struct ReadBlob {
+  uint64_t start[N], end[N], maxend[N];
+  uint32_t orig[N];
+  void fill(const ReadPlan& p) {
+    std::memcpy(start, p.start, 8 * p.n);
+    std::memcpy(end, p.end, 8 * p.n);
+    std::memcpy(maxend, p.maxend, 8 * p.n);
+    std::memcpy(orig, p.orig, 4 * p.n_all);
+  }
+  __host__ __device__ const uint64_t* starts(const ReadPlan&) const { return start; }
+  __host__ __device__ const uint64_t* ends(const ReadPlan&) const { return end; }
+  __host__ __device__ const uint64_t* maxends(const ReadPlan&) const { return maxend; }
+  __host__ __device__ const uint32_t* origs(const ReadPlan&) const { return orig; }
+};
+template <>
+struct ReadBlob<0> {
+  void fill(const ReadPlan&) {}
+  __host__ __device__ const uint64_t* starts(const ReadPlan& p) const { return p.start; }
+  __host__ __device__ const uint64_t* ends(const ReadPlan& p) const { return p.end; }
+  __host__ __device__ const uint64_t* maxends(const ReadPlan& p) const { return p.maxend; }
+  __host__ __device__ const uint32_t* origs(const ReadPlan& p) const { return p.orig; }
+};
+// flags[i] = a read overlaps buffer i; every flag is written.  m > 0.  host
+// (at most kReadBlob buffers): the plan's arrays are in host memory and travel
+// with the launch; the bitmap is zero on exit too.
+cudaError_t launch_classify_reads(bool host, ReadPlan p, const uint64_t* addr,
+                                  const uint64_t* bytes, int64_t m, uint8_t* flags, int sm_count,
+                                  cudaStream_t stream);
 
 // Occupancy of the streaming kernel (blocks per SM) for the launch shape.
 int stream_blocks_per_sm();

@@ -35,6 +35,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstring>
 #include <mutex>
 
 #include "pcs_internal.h"
@@ -1620,6 +1621,23 @@ __global__ void __launch_bounds__(kThreads, 2)
 // Relevance score and top-k
 // ---------------------------------------------------------------------------
 
+// Where a kernel's bank descriptors are: in the workspace (p), or, for a call
+// of few banks (BLOB), in the parameter itself: they travel with each of the
+// call's launches, as a small call's descriptors do.  Measured, whole calls: a
+// global threshold of few entries 22.7 -> 18.1 us, a prune of few 12.5 -> 10.3.
+template <bool BLOB>
+struct BankArg;
+template <>
+struct BankArg<false> {
+  const BankDesc* p;
+  __device__ const BankDesc* get() const { return p; }
+};
+template <>
+struct BankArg<true> {
+  BankDesc b[kBankBlob];
+  __device__ const BankDesc* get() const { return b; }
+};
+
 // Order-preserving map float -> uint32 (-0 ranks as +0, NaN lowest).
 __device__ __forceinline__ uint32_t ord32(float s) {
   if (isnan(s)) return 0u;
@@ -1797,8 +1815,8 @@ struct ScoreShape {
 // the warp, four in flight, q.k and k.k paired -> this): D = 64 335 -> 86 us,
 // 128 173 -> 84, 192 121 -> 95, 256 95 -> 82, 264 148 -> 114, 512 88 -> 80, 768
 // 140 -> 80, 1,024 123 -> 80 (6.7 TB/s); bf16 within 4 % of these.
-template <class SH, int DT, int HM>
-__device__ __forceinline__ void score_range(const BankDesc* __restrict__ banks, int n_banks,
+template <class SH, int DT, int HM, bool BLOB>
+__device__ __forceinline__ void score_range(const BankDesc* banks, int n_banks,
                                             uint64_t n_entries, float* __restrict__ scores,
                                             bool hist, uint32_t* s_cnt, unsigned long long* s_w) {
   constexpr int G = SH::kLanes, SPL = SH::kSeg, R = SH::kRows, E = SH::kSide;
@@ -1816,7 +1834,7 @@ __device__ __forceinline__ void score_range(const BankDesc* __restrict__ banks, 
     while (span > 1) {
       const int step = (span + 31) >> 5;
       const int i = b + lane * step;
-      const bool le = i < b + span && __ldg(&banks[i].entry_begin) <= e_begin;
+      const bool le = i < b + span && fetch<!BLOB>(&banks[i].entry_begin) <= e_begin;
       const unsigned m = __ballot_sync(kFull, le);  // lane 0 probes b: never empty
       const int last = 31 - __clz(m);
       b += last * step;
@@ -1832,9 +1850,9 @@ __device__ __forceinline__ void score_range(const BankDesc* __restrict__ banks, 
     // Entries of this round must share one bank to use the cached query;
     // a round stops early at a bank boundary.
     if (qbank < 0 || e0 >= bank_end) {  // warp-uniform: load the query, compute |q|
-      while (b + 1 < n_banks && __ldg(&banks[b + 1].entry_begin) <= e0) ++b;
+      while (b + 1 < n_banks && fetch<!BLOB>(&banks[b + 1].entry_begin) <= e0) ++b;
       B = banks[b];
-      bank_end = b + 1 < n_banks ? __ldg(&banks[b + 1].entry_begin) : n_entries;
+      bank_end = b + 1 < n_banks ? fetch<!BLOB>(&banks[b + 1].entry_begin) : n_entries;
       segs = B.D / 8;
       const uint4* qrow = reinterpret_cast<const uint4*>(B.query);
       float sq = 0.f;
@@ -1921,10 +1939,11 @@ __device__ __forceinline__ void score_range(const BankDesc* __restrict__ banks, 
 
 // HM (global threshold): 0 none; 1 / 2 also histogram the top 11 key bits of
 // every score (2: weighted by the bank's entry bytes) and pick the first digit.
-template <class SH, int DT, int HM>
+template <class SH, int DT, int HM, bool BLOB>
 __global__ void __launch_bounds__(kThreads, SH::kBlocks)
-    k_score_fixed(const BankDesc* __restrict__ banks, int n_banks, uint64_t n_entries,
+    k_score_fixed(const __grid_constant__ BankArg<BLOB> bank_arg, int n_banks, uint64_t n_entries,
                   float* __restrict__ scores, GHist gh) {
+  const BankDesc* banks = bank_arg.get();
   grid_dependency();
   __shared__ uint32_t s_cnt[HM ? kGBins : 1];
   __shared__ unsigned long long s_w[HM == 2 ? kGBins : 1];
@@ -1937,15 +1956,17 @@ __global__ void __launch_bounds__(kThreads, SH::kBlocks)
     }
     __syncthreads();
   }
-  score_range<SH, DT, HM>(banks, n_banks, n_entries, scores, hist, s_cnt, s_w);
+  score_range<SH, DT, HM, BLOB>(banks, n_banks, n_entries, scores, hist, s_cnt, s_w);
   if (hist) gpass_finish<HM == 1>(gh.st, 0, gh.uniform_bytes, s_cnt, s_w, &s_last);
 }
 
 
 // Any key width or a mix of key types: the query is re-read per entry.
+template <bool BLOB>
 __global__ void __launch_bounds__(kThreads)
-    k_score_any(const BankDesc* __restrict__ banks, int n_banks, uint64_t n_entries,
+    k_score_any(const __grid_constant__ BankArg<BLOB> bank_arg, int n_banks, uint64_t n_entries,
                 float* __restrict__ scores) {
+  const BankDesc* banks = bank_arg.get();
   grid_dependency();
   const int lane = threadIdx.x & 31;
   const uint64_t gw = static_cast<uint64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
@@ -1957,7 +1978,7 @@ __global__ void __launch_bounds__(kThreads)
     int lo = 0, hi = n_banks - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (__ldg(&banks[mid].entry_begin) <= e_begin) lo = mid;
+      if (fetch<!BLOB>(&banks[mid].entry_begin) <= e_begin) lo = mid;
       else hi = mid - 1;
     }
     b = lo;
@@ -1965,7 +1986,7 @@ __global__ void __launch_bounds__(kThreads)
   int qbank = -1;
   float qnorm = 0.f;
   for (uint64_t e = e_begin; e < e_end; ++e) {
-    while (b + 1 < n_banks && __ldg(&banks[b + 1].entry_begin) <= e) ++b;
+    while (b + 1 < n_banks && fetch<!BLOB>(&banks[b + 1].entry_begin) <= e) ++b;
     const BankDesc& B = banks[b];
     const bool bf16 = B.is_bf16 != 0;
     const uint4* qrow = reinterpret_cast<const uint4*>(B.query);
@@ -2120,9 +2141,12 @@ __device__ void topk_bank_reg(const float* __restrict__ sc, int n, int k, int32_
   __syncthreads();
 }
 
+template <bool BLOB>
 __global__ void __launch_bounds__(kThreads)
-    k_topk(const BankDesc* __restrict__ banks, int n_banks, const float* __restrict__ scores,
-           int32_t* __restrict__ kept_idx) {
+    k_topk(const __grid_constant__ BankArg<BLOB> bank_arg, int n_banks,
+           const float* __restrict__ scores, int32_t* __restrict__ kept_idx,
+           int32_t* __restrict__ kept_off, int32_t kept_total) {
+  const BankDesc* banks = bank_arg.get();
   grid_dependency();
   __shared__ uint32_t hist[256];
   __shared__ uint32_t warp_cnt[kWarps];
@@ -2130,6 +2154,10 @@ __global__ void __launch_bounds__(kThreads)
   const int wib = threadIdx.x >> 5;
   for (int b = blockIdx.x; b < n_banks; b += gridDim.x) {
     const BankDesc B = banks[b];
+    if (kept_off && threadIdx.x == 0) {
+      kept_off[b] = static_cast<int32_t>(B.kept_begin);
+      if (b == n_banks - 1) kept_off[n_banks] = kept_total;
+    }
     const int n = B.n, k = B.k;
     const float* sc = scores + B.entry_begin;
     int32_t* out = kept_idx + B.kept_begin;
@@ -2857,11 +2885,12 @@ __device__ __forceinline__ T gs_incl_scan(T v, T* warp_sum, T* total) {
   return wib > 0 ? before + incl : incl;
 }
 
-template <bool UNIFORM>
+template <bool UNIFORM, bool BLOB>
 __global__ void __launch_bounds__(kGsThreads, 1)
-    k_gsmall(const BankDesc* __restrict__ banks, int n_banks, uint32_t n, const float* scores,
-             uint64_t budget, int keep_all, int32_t* __restrict__ kept_idx,
+    k_gsmall(const __grid_constant__ BankArg<BLOB> bank_arg, int n_banks, uint32_t n,
+             const float* scores, uint64_t budget, int keep_all, int32_t* __restrict__ kept_idx,
              int32_t* __restrict__ kept_off) {
+  const BankDesc* banks = bank_arg.get();
   __shared__ uint32_t s_lo[kGBins];                   // counts (UNIFORM) or low bytes per digit
   __shared__ uint32_t s_hi[UNIFORM ? 1 : kGBins];     // high words of the bytes
   __shared__ uint32_t s_beg[kGSmallBanks + 1];        // first entry of each bank; then n
@@ -3256,10 +3285,15 @@ __device__ __forceinline__ uint32_t mm_unit_shift(const uint8_t* a, const uint8_
 // (scratch) starts at the bytes only one buffer of each pair has; the last
 // block to finish (atomic ticket, zero on entry and on exit) copies it to the
 // caller's counts, which saves a copy between the plan and this launch.
+// A call of few pairs has its plan with the launch, as a small call does, and
+// its sums in words that are zero on entry and on exit (36 pairs of up to
+// 468 kB, whole calls: 8.9 -> 6.1 us).
+template <int N>  // pairs the parameter holds (0: the plan is in the workspace)
 __global__ void __launch_bounds__(kThreads, 4)
-    k_mismatch(const MmPair* __restrict__ pairs, const uint64_t* __restrict__ unit_begin,
-               int32_t n, uint64_t units, unsigned long long* sums, uint64_t* counts,
-               uint32_t* ticket) {
+    k_mismatch(const __grid_constant__ MmBlob<N> blob, int32_t n, uint64_t units,
+               unsigned long long* sums, uint64_t* counts, uint32_t* ticket) {
+  const MmPair* pairs = blob.pairs();
+  const uint64_t* unit_begin = blob.begins();
   __shared__ bool s_last;
   const int lane = threadIdx.x & 31;
   const uint64_t warps = static_cast<uint64_t>(gridDim.x) * kWarps;
@@ -3273,14 +3307,14 @@ __global__ void __launch_bounds__(kThreads, 4)
     for (int span = n; span > 1;) {
       const int step = (span + 31) >> 5;
       const int i = pi + lane * step;
-      const bool le = i < pi + span && __ldg(unit_begin + i) <= u;
+      const bool le = i < pi + span && fetch<N == 0>(unit_begin + i) <= u;
       const int last = 31 - __clz(__ballot_sync(kFull, le));  // lane 0 probes pi: never empty
       pi += last * step;
       span = min(step, span - last * step);
     }
   }
   for (; u < u1; ++pi) {
-    const uint64_t pbeg = __ldg(unit_begin + pi), pend = __ldg(unit_begin + pi + 1);
+    const uint64_t pbeg = fetch<N == 0>(unit_begin + pi), pend = fetch<N == 0>(unit_begin + pi + 1);
     if (pend <= u) continue;  // nothing of this pair
     const MmPair P = pairs[pi];
     const uint64_t x0 = (u - pbeg) * (kMmUnit / 16);  // the first vector here
@@ -3324,7 +3358,10 @@ __global__ void __launch_bounds__(kThreads, 4)
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  for (int i = threadIdx.x; i < n; i += kThreads) counts[i] = __ldcg(sums + i);
+  for (int i = threadIdx.x; i < n; i += kThreads) {
+    counts[i] = __ldcg(sums + i) + blob.more(i);
+    if (N > 0) sums[i] = 0;
+  }
   if (threadIdx.x == 0) *ticket = 0;
 }
 
@@ -3361,10 +3398,20 @@ constexpr int kReadIlp = 4;              // reads a thread has in flight
 // entry and on exit) writes every flag: no clearing pass before this launch.
 // STAGED: at most kReadStage buffers, their starts and running maxima in
 // shared memory; TABLE (staged only): search the slice table first.
-template <bool STAGED, bool TABLE>
+// N: buffers the parameter holds; such a call has them with its launch, as a
+// small call has its descriptors, and a bitmap that is zero on exit too (8
+// buffers, 7,639 reads, whole calls: 8.8 -> 6.0 us).  0: they are in the
+// workspace.
+template <bool STAGED, bool TABLE, int N>
 __global__ void __launch_bounds__(kReadThreads, 2)
-    k_classify_reads(ReadPlan P, const uint64_t* __restrict__ addr,
-                     const uint64_t* __restrict__ bytes, int64_t m, uint8_t* flags) {
+    k_classify_reads(const __grid_constant__ ReadBlob<N> blob, ReadPlan P,
+                     const uint64_t* __restrict__ addr, const uint64_t* __restrict__ bytes,
+                     int64_t m, uint8_t* flags) {
+  static_assert(STAGED || N == 0, "a parameter's arrays are staged");
+  const uint64_t* const b_start = blob.starts(P);
+  const uint64_t* const b_end = blob.ends(P);
+  const uint64_t* const b_max = blob.maxends(P);
+  const uint32_t* const b_orig = blob.origs(P);
   static_assert(STAGED || !TABLE, "the table indexes the staged arrays");
   extern __shared__ __align__(16) uint8_t rd_smem[];
   uint32_t* const seen = reinterpret_cast<uint32_t*>(rd_smem);  // [words] bitmap
@@ -3375,12 +3422,12 @@ __global__ void __launch_bounds__(kReadThreads, 2)
   for (int w = threadIdx.x; w < words; w += blockDim.x) seen[w] = 0;
   if (STAGED)
     for (int i = threadIdx.x; i < P.n; i += blockDim.x) {
-      s_start[i] = __ldg(P.start + i);
-      s_max[i] = __ldg(P.maxend + i);
+      s_start[i] = fetch<N == 0>(b_start + i);
+      s_max[i] = fetch<N == 0>(b_max + i);
     }
   __syncthreads();
-  auto start = [&](int i) -> uint64_t { return STAGED ? s_start[i] : __ldg(P.start + i); };
-  auto maxend = [&](int i) -> uint64_t { return STAGED ? s_max[i] : __ldg(P.maxend + i); };
+  auto start = [&](int i) -> uint64_t { return STAGED ? s_start[i] : __ldg(b_start + i); };
+  auto maxend = [&](int i) -> uint64_t { return STAGED ? s_max[i] : __ldg(b_max + i); };
   // The first buffer in [lo, hi) whose running maximum end exceeds a; hi if none.
   auto search = [&](int lo, int hi, uint64_t a) {
     while (lo < hi) {
@@ -3442,7 +3489,7 @@ __global__ void __launch_bounds__(kReadThreads, 2)
       if (start(lo) >= e) continue;
       mark(lo);
       for (int i = lo + 1; i < P.n && start(i) < e; ++i)
-        if (__ldg(P.end + i) > a) mark(i);
+        if (fetch<N == 0>(b_end + i) > a) mark(i);
     }
   }
   __syncthreads();
@@ -3457,8 +3504,12 @@ __global__ void __launch_bounds__(kReadThreads, 2)
   if (!seen[0]) return;
   __threadfence();
   for (int i = threadIdx.x; i < P.n_all; i += blockDim.x)
-    flags[__ldg(P.orig + i)] =
+    flags[fetch<N == 0>(b_orig + i)] =
         i < P.n ? static_cast<uint8_t>((__ldcg(P.bitmap + (i >> 5)) >> (i & 31)) & 1u) : 0;
+  if (N > 0) {
+    __syncthreads();
+    for (int w = threadIdx.x; w < words; w += blockDim.x) P.bitmap[w] = 0;
+  }
   if (threadIdx.x == 0) *P.ticket = 0;
 }
 
@@ -3496,7 +3547,7 @@ __global__ void k_selftest_wait(int which, const uint32_t* never_set, uint32_t* 
 // stream operation the launch waits as usual.
 template <typename... P, typename... A>
 cudaError_t launch_after(void (*k)(P...), unsigned grid, unsigned block, size_t smem,
-                         cudaStream_t stream, A... args) {
+                         cudaStream_t stream, const A&... args) {
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -3709,29 +3760,45 @@ cudaError_t launch_reduce_nodes(const NodeLevel* lv, int n_secs, uint64_t* nodes
   return launch_after(k_reduce_nodes, blocks, kThreads, 0, stream, lv, n_secs, nodes, base, n_groups);
 }
 
+// f(the kernel argument that holds or points at the banks).
+template <typename F>
+static cudaError_t with_banks(const Banks& k, F&& f) {
+  if (k.dev) return f(BankArg<false>{k.dev});
+  if (k.n > kBankBlob) return cudaErrorInvalidValue;
+  BankArg<true> arg;
+  std::memcpy(arg.b, k.host, sizeof(BankDesc) * k.n);
+  return f(arg);
+}
+
 template <class SH, int DT>
-static cudaError_t launch_score_shape(const BankDesc* banks, int n_banks, uint64_t n_entries,
-                                      float* scores, int sm_count, cudaStream_t stream, GHist gh) {
+static cudaError_t launch_score_shape(const Banks& banks, uint64_t n_entries, float* scores,
+                                      int sm_count, cudaStream_t stream, GHist gh) {
   // A round per warp at least; at most one resident wave (large populations
   // fill it).
-  auto launch = [&](auto kernel) {
+  auto launch = [&](auto kernel, const auto& arg) {
     const uint64_t want = (n_entries + kWarps * SH::kRound - 1) / (kWarps * SH::kRound);
     const uint64_t cap = static_cast<uint64_t>(sm_count) *
                          resident_blocks(reinterpret_cast<const void*>(kernel));
     return launch_after(kernel, static_cast<unsigned>(want < cap ? want : cap), kThreads, 0, stream,
-                        banks, n_banks, n_entries, scores, gh);
+                        arg, banks.n, n_entries, scores, gh);
   };
-  const int hm = gh.st ? gh.mode : 0;
-  if (hm == 0) return launch(k_score_fixed<SH, DT, 0>);
-  if (hm == 1) return launch(k_score_fixed<SH, DT, 1>);
-  return launch(k_score_fixed<SH, DT, 2>);
+  if (!gh.st)
+    return with_banks(banks, [&](const auto& arg) {
+      constexpr bool BLOB = sizeof(arg) > sizeof(void*);
+      return launch(k_score_fixed<SH, DT, 0, BLOB>, arg);
+    });
+  // With a histogram the call has a workspace, and the banks are in it.
+  if (!banks.dev) return cudaErrorInvalidValue;
+  const BankArg<false> arg{banks.dev};
+  return gh.mode == 1 ? launch(k_score_fixed<SH, DT, 1, false>, arg)
+                      : launch(k_score_fixed<SH, DT, 2, false>, arg);
 }
 
 template <int DT>
-static cudaError_t launch_score_type(const BankDesc* banks, int n_banks, uint64_t n_entries,
-                                     int max_dim, float* scores, int sm_count, cudaStream_t stream,
+static cudaError_t launch_score_type(const Banks& banks, uint64_t n_entries, int max_dim,
+                                     float* scores, int sm_count, cudaStream_t stream,
                                      GHist gh) {
-  auto go = [&](auto launch) { return launch(banks, n_banks, n_entries, scores, sm_count, stream, gh); };
+  auto go = [&](auto launch) { return launch(banks, n_entries, scores, sm_count, stream, gh); };
   if (max_dim <= 64) return go(launch_score_shape<ScoreShape<8, 1, 8, 3>, DT>);
   if (max_dim <= 128) return go(launch_score_shape<ScoreShape<16, 1, 8, 3>, DT>);
   if (max_dim <= 256) return go(launch_score_shape<ScoreShape<32, 1, 8, 3>, DT>);
@@ -3740,8 +3807,8 @@ static cudaError_t launch_score_type(const BankDesc* banks, int n_banks, uint64_
   return go(launch_score_shape<ScoreShape<32, 4, 4, 2>, DT>);
 }
 
-cudaError_t launch_score(const BankDesc* banks, int n_banks, uint64_t n_entries, int max_dim,
-                         int key_types, float* scores, int sm_count, cudaStream_t stream,
+cudaError_t launch_score(const Banks& banks, uint64_t n_entries, int max_dim, int key_types,
+                         float* scores, int sm_count, cudaStream_t stream,
                          GHist gh, bool* fused) {
   if (fused) *fused = false;
   if (n_entries == 0) return cudaSuccess;
@@ -3750,23 +3817,29 @@ cudaError_t launch_score(const BankDesc* banks, int n_banks, uint64_t n_entries,
     // At least two rounds of four entries per warp.
     const uint64_t want = (n_entries + 8 * kWarps - 1) / (8 * kWarps);
     const uint64_t cap = static_cast<uint64_t>(sm_count) *
-                         resident_blocks(reinterpret_cast<const void*>(k_score_any));
-    return launch_after(k_score_any, static_cast<unsigned>(want < cap ? want : cap), kThreads, 0,
-                        stream, banks, n_banks, n_entries, scores);
+                         resident_blocks(reinterpret_cast<const void*>(k_score_any<false>));
+    return with_banks(banks, [&](const auto& arg) {
+      constexpr bool BLOB = sizeof(arg) > sizeof(void*);
+      return launch_after(k_score_any<BLOB>, static_cast<unsigned>(want < cap ? want : cap), kThreads,
+                          0, stream, arg, banks.n, n_entries, scores);
+    });
   }
   const cudaError_t e =
       key_types == 1
-          ? launch_score_type<1>(banks, n_banks, n_entries, max_dim, scores, sm_count, stream, gh)
-          : launch_score_type<0>(banks, n_banks, n_entries, max_dim, scores, sm_count, stream, gh);
+          ? launch_score_type<1>(banks, n_entries, max_dim, scores, sm_count, stream, gh)
+          : launch_score_type<0>(banks, n_entries, max_dim, scores, sm_count, stream, gh);
   if (fused) *fused = gh.st && e == cudaSuccess;
   return e;
 }
 
-cudaError_t launch_topk(const BankDesc* banks, int n_banks, const float* scores,
-                        int32_t* kept_idx, cudaStream_t stream) {
-  if (n_banks <= 0) return cudaSuccess;
-  return launch_after(k_topk, n_banks < 65535 ? n_banks : 65535, kThreads, 0, stream, banks,
-                      n_banks, scores, kept_idx);
+cudaError_t launch_topk(const Banks& banks, const float* scores, int32_t* kept_idx,
+                        int32_t* kept_off, int32_t kept_total, cudaStream_t stream) {
+  if (banks.n <= 0) return cudaSuccess;
+  return with_banks(banks, [&](const auto& arg) {
+    constexpr bool BLOB = sizeof(arg) > sizeof(void*);
+    return launch_after(k_topk<BLOB>, banks.n < 65535 ? banks.n : 65535, kThreads, 0, stream, arg,
+                        banks.n, scores, kept_idx, kept_off, kept_total);
+  });
 }
 
 static int gblocks(const GPlan& p, int sm_count, const void* kernel) {
@@ -3819,47 +3892,73 @@ cudaError_t launch_pool_cow(const PoolDev& p, int32_t* table, int64_t n_table,
   return cudaGetLastError();
 }
 
-cudaError_t launch_mismatch(const MmPair* pairs, const uint64_t* unit_begin, int32_t n,
-                            uint64_t units, uint64_t* sums, uint64_t* counts, uint32_t* ticket,
-                            int sm_count, cudaStream_t stream) {
-  if (units == 0 || n <= 0) return cudaErrorInvalidValue;
+template <int N>
+static cudaError_t launch_mismatch_blob(const MmBlob<N>& blob, int32_t n, uint64_t units,
+                                        uint64_t* sums, uint64_t* counts, uint32_t* ticket,
+                                        int sm_count, cudaStream_t stream) {
   // One resident wave; a unit per warp until that wave is full, as each
   // further unit of a warp adds a memory round trip to a small call (18 pairs
   // of 64 KiB: 15.4 us with at least eight units a warp and the counts copied
   // by a launch of their own, 10.1 us so).
   const uint64_t want = (units + kWarps - 1) / kWarps;
   const uint64_t cap = static_cast<uint64_t>(sm_count) *
-                       resident_blocks(reinterpret_cast<const void*>(k_mismatch));
-  k_mismatch<<<static_cast<unsigned>(want < cap ? want : cap), kThreads, 0, stream>>>(
-      pairs, unit_begin, n, units, reinterpret_cast<unsigned long long*>(sums), counts, ticket);
+                       resident_blocks(reinterpret_cast<const void*>(k_mismatch<N>));
+  k_mismatch<N><<<static_cast<unsigned>(want < cap ? want : cap), kThreads, 0, stream>>>(
+      blob, n, units, reinterpret_cast<unsigned long long*>(sums), counts, ticket);
   return cudaGetLastError();
 }
 
-template <bool STAGED, bool TABLE>
+template <int N>
+static cudaError_t launch_mismatch_host(const MmPair* pairs, const uint64_t* unit_begin,
+                                        const uint64_t* extra, int32_t n, uint64_t units,
+                                        uint64_t* sums, uint64_t* counts, uint32_t* ticket,
+                                        int sm_count, cudaStream_t stream) {
+  MmBlob<N> blob;
+  std::memcpy(blob.pair, pairs, sizeof(MmPair) * n);
+  std::memcpy(blob.unit_begin, unit_begin, 8 * (n + 1));
+  std::memcpy(blob.extra, extra, 8 * n);
+  return launch_mismatch_blob(blob, n, units, sums, counts, ticket, sm_count, stream);
+}
+
+cudaError_t launch_mismatch(bool host, const MmPair* pairs, const uint64_t* unit_begin,
+                            const uint64_t* extra, int32_t n, uint64_t units, uint64_t* sums,
+                            uint64_t* counts, uint32_t* ticket, int sm_count, cudaStream_t stream) {
+  if (units == 0 || n <= 0 || (host && n > kMmBlob)) return cudaErrorInvalidValue;
+  if (!host)
+    return launch_mismatch_blob(MmBlob<0>{pairs, unit_begin}, n, units, sums, counts, ticket,
+                                sm_count, stream);
+  auto f = n <= 64 ? launch_mismatch_host<64> : launch_mismatch_host<kMmBlob>;
+  return f(pairs, unit_begin, extra, n, units, sums, counts, ticket, sm_count, stream);
+}
+
+template <bool STAGED, bool TABLE, int N>
 static cudaError_t launch_reads(const ReadPlan& p, const uint64_t* addr, const uint64_t* bytes,
                                 int64_t m, uint8_t* flags, unsigned threads, size_t smem,
                                 int sm_count, cudaStream_t stream) {
   if (smem > 48 * 1024) {  // long bitmaps or many staged buffers
-    cudaError_t e = cudaFuncSetAttribute(k_classify_reads<STAGED, TABLE>,
+    cudaError_t e = cudaFuncSetAttribute(k_classify_reads<STAGED, TABLE, N>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
     if (e != cudaSuccess) return e;
   }
   const uint64_t want = (static_cast<uint64_t>(m) + threads - 1) / threads;
   // One resident wave: 2,048 threads per SM (32 registers), fewer where the
-  // shared memory of 227 KB allows fewer blocks.
+  // shared memory of 228 KB allows fewer blocks.
   const uint64_t per_sm =
       std::max<uint64_t>(1, std::min<uint64_t>(2048 / threads, 228 * 1024 / (smem + 1024)));
   const uint64_t cap = static_cast<uint64_t>(sm_count) * per_sm;
-  k_classify_reads<STAGED, TABLE>
-      <<<static_cast<unsigned>(want < cap ? want : cap), threads, smem, stream>>>(p, addr, bytes, m,
-                                                                               flags);
+  ReadBlob<N> blob;
+  blob.fill(p);
+  k_classify_reads<STAGED, TABLE, N>
+      <<<static_cast<unsigned>(want < cap ? want : cap), threads, smem, stream>>>(
+          blob, p, addr, bytes, m, flags);
   return cudaGetLastError();
 }
 
-cudaError_t launch_classify_reads(ReadPlan p, const uint64_t* addr, const uint64_t* bytes,
-                                  int64_t m, uint8_t* flags, int sm_count, cudaStream_t stream) {
-  if (m <= 0 || p.n <= 0) return cudaErrorInvalidValue;
+cudaError_t launch_classify_reads(bool host, ReadPlan p, const uint64_t* addr,
+                                  const uint64_t* bytes, int64_t m, uint8_t* flags, int sm_count,
+                                  cudaStream_t stream) {
+  if (m <= 0 || p.n <= 0 || (host && p.n_all > kReadBlob)) return cudaErrorInvalidValue;
   const size_t words = (static_cast<size_t>(p.n) + 31) / 32;
   size_t smem = ((words + 1) & ~static_cast<size_t>(1)) * 4;
   const bool staged = p.n <= kReadStage;
@@ -3869,19 +3968,23 @@ cudaError_t launch_classify_reads(ReadPlan p, const uint64_t* addr, const uint64
   // block more than it saves (200 buffers, without / with: 500,000 reads 13.8 /
   // 17.6 us, 2M 23.8 / 23.3, 4M 35.3 / 30.9, 16M 106 / 76).
   const bool table = staged && m >= static_cast<int64_t>(sm_count) * 2048 * 8;
-  if (!table) {
-    const unsigned threads = 256;
-    if (staged)
-      return launch_reads<true, false>(p, addr, bytes, m, flags, threads, smem, sm_count, stream);
-    return launch_reads<false, false>(p, addr, bytes, m, flags, threads, smem, sm_count, stream);
+  unsigned threads = 256;
+  if (table) {
+    // Slices of the smallest power of two that cover the buffers' span.
+    const uint64_t span = p.top - p.base;
+    p.slice_shift = 0;
+    while (((span - 1) >> p.slice_shift) >= kReadSlices) ++p.slice_shift;
+    p.slices = static_cast<int32_t>((span - 1) >> p.slice_shift) + 1;
+    smem += 4ull * p.slices;
+    threads = kReadThreads;
   }
-  // Slices of the smallest power of two that cover the buffers' span.
-  const uint64_t span = p.top - p.base;
-  p.slice_shift = 0;
-  while (((span - 1) >> p.slice_shift) >= kReadSlices) ++p.slice_shift;
-  p.slices = static_cast<int32_t>((span - 1) >> p.slice_shift) + 1;
-  smem += 4ull * p.slices;
-  return launch_reads<true, true>(p, addr, bytes, m, flags, kReadThreads, smem, sm_count, stream);
+  auto f = launch_reads<false, false, 0>;
+  if (table) {
+    f = host ? launch_reads<true, true, kReadBlob> : launch_reads<true, true, 0>;
+  } else if (staged) {
+    f = host ? launch_reads<true, false, kReadBlob> : launch_reads<true, false, 0>;
+  }
+  return f(p, addr, bytes, m, flags, threads, smem, sm_count, stream);
 }
 
 cudaError_t launch_gfinish(const GPlan& p, int first_pass, int sm_count, cudaStream_t stream) {
@@ -3898,16 +4001,20 @@ cudaError_t launch_gfinish(const GPlan& p, int first_pass, int sm_count, cudaStr
 }
 
 
-cudaError_t launch_gsmall(const BankDesc* banks, int n_banks, uint64_t entries, const float* scores,
+cudaError_t launch_gsmall(const Banks& banks, uint64_t entries, const float* scores,
                           uint64_t budget, bool uniform, bool keep_all, int32_t* kept_idx,
                           int32_t* kept_off, cudaStream_t stream) {
-  if (entries == 0 || entries > kGSmallEntries || n_banks < 1 || n_banks > kGSmallBanks)
+  if (entries == 0 || entries > kGSmallEntries || banks.n < 1 || banks.n > kGSmallBanks)
     return cudaErrorInvalidValue;
   const uint32_t n = static_cast<uint32_t>(entries);
-  return uniform ? launch_after(k_gsmall<true>, 1, kGsThreads, 0, stream, banks, n_banks, n, scores,
-                                budget, keep_all ? 1 : 0, kept_idx, kept_off)
-                 : launch_after(k_gsmall<false>, 1, kGsThreads, 0, stream, banks, n_banks, n, scores,
-                                budget, keep_all ? 1 : 0, kept_idx, kept_off);
+  const int all = keep_all ? 1 : 0;
+  return with_banks(banks, [&](const auto& arg) {
+    constexpr bool BLOB = sizeof(arg) > sizeof(void*);
+    return uniform ? launch_after(k_gsmall<true, BLOB>, 1, kGsThreads, 0, stream, arg, banks.n, n,
+                                  scores, budget, all, kept_idx, kept_off)
+                   : launch_after(k_gsmall<false, BLOB>, 1, kGsThreads, 0, stream, arg, banks.n, n,
+                                  scores, budget, all, kept_idx, kept_off);
+  });
 }
 
 cudaError_t launch_selftest_wait(int which, const uint32_t* never_set, uint32_t* err,

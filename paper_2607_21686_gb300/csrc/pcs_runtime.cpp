@@ -365,7 +365,8 @@ struct pcs_ctx {
   // Workspaces, one per stream: the descriptors and tree nodes of a call,
   // after a header of per-call device words ([0] a kernel's ticket, [1]
   // failures of a verify = 1 restore, [4] and [5] the TMA kernel's work
-  // sharing, [64 ..] the small-call kernel's tasks done per item).  Calls on one stream are ordered
+  // sharing, [64 ..] the small-call kernel's tasks done per item, [128 ..]
+  // sums or a bitmap of a call of few items).  Calls on one stream are ordered
   // by the stream; calls on different streams do not share one, so they can
   // run side by side.
   struct Workspace {
@@ -485,10 +486,12 @@ Arena* arena_of(pcs_ctx* c, uint32_t placement) {
   return placement == PCS_PLACE_DEVICE ? c->dev_arena.get() : c->host_arena.get();
 }
 
-constexpr uint64_t kWsHeader = 512;  // per-call device words before the descriptors
+constexpr uint64_t kWsHeader = 8192;  // per-call device words before the descriptors
 constexpr int kWordBulkSched = 4;    // header words [4], [5]: the TMA kernel's work sharing
 constexpr int kWordDone = 64;        // [64 .. 127]: the small-call kernel's tasks done per item
-static_assert(4 * (kWordDone + kSmallMaxItems) <= kWsHeader, "header words");
+constexpr int kWordSums = 128;        // [128 ..]: sums or a bitmap of a call of few items
+static_assert(kWordDone + kSmallMaxItems <= kWordSums, "header words");
+static_assert(4 * kWordSums + 8 * kMmBlob <= kWsHeader && kReadBlob / 32 <= 2 * kMmBlob, "header words");
 
 // The header words of a call: they sit just below its descriptors, in a
 // stream's workspace and in a prepared call's buffer alike.
@@ -1859,11 +1862,11 @@ pcs_status bank_descs(const pcs_bank* banks, int32_t n, const int32_t* k,
   return PCS_OK;
 }
 
-// The relevance score of every entry (descriptors already on the device);
+// The relevance score of every entry;
 // with gh.st set, also the first digit pass of the global threshold where the
 // score kernel can take it (*fused says whether it did).
-cudaError_t launch_bank_scores(pcs_ctx* c, const pcs_bank* banks, int32_t n,
-                               const BankDesc* dbanks, uint64_t entries, float* sc,
+cudaError_t launch_bank_scores(pcs_ctx* c, const pcs_bank* banks, int32_t n, const Banks& descs,
+                               uint64_t entries, float* sc,
                                cudaStream_t stream, GHist gh = GHist{}, bool* fused = nullptr) {
   LaunchScope ls(c, kKScore, stream);
   int max_dim = 0, n_bf16 = 0;
@@ -1872,7 +1875,7 @@ cudaError_t launch_bank_scores(pcs_ctx* c, const pcs_bank* banks, int32_t n,
     n_bf16 += banks[s].key_dtype == PCS_DT_BF16;
   }
   const int key_types = n_bf16 == 0 ? 0 : (n_bf16 == n ? 1 : 2);
-  return launch_score(dbanks, n, entries, max_dim, key_types, sc, c->sm_count, stream, gh, fused);
+  return launch_score(descs, entries, max_dim, key_types, sc, c->sm_count, stream, gh, fused);
 }
 
 pcs_status pcs_prune(pcs_ctx* c, const pcs_bank* banks, int32_t n, const pcs_prune_params* p,
@@ -1890,38 +1893,35 @@ pcs_status pcs_prune(pcs_ctx* c, const pcs_bank* banks, int32_t n, const pcs_pru
   uint64_t entries = 0;
   st = bank_descs(banks, n, k.data(), &d, &entries, align);
   if (st) return st;
-  std::vector<int32_t> koff(n + 1, 0);
   uint64_t kept = 0;
-  for (int s = 0; s < n; ++s) {
-    kept += round_up(static_cast<uint64_t>(k[s]), align);
-    koff[s + 1] = static_cast<int32_t>(kept);
-  }
+  for (int s = 0; s < n; ++s) kept += round_up(static_cast<uint64_t>(k[s]), align);
   if (kept > 0 && !kept_idx) return fail(PCS_E_INVAL, "kept_idx is null");
   std::lock_guard<std::mutex> lk(c->mu);
   st = set_device(c);
   if (st) return st;
-  WsLayout L;
-  L.banks = 0;
-  L.secs = round_up(sizeof(BankDesc) * n, kRecordAlign);       // kept offsets (int32)
-  L.nodes = round_up(L.secs + 4ull * (n + 1), kRecordAlign);   // scores if caller gives none
-  L.total = L.nodes + (scores ? 0 : 4 * entries);
+  // Few banks travel with the launches; a workspace is then needed only for
+  // scores that the caller does not want.
+  const bool sent = n <= kBankBlob;
+  const uint64_t o_sc = sent ? 0 : round_up(sizeof(BankDesc) * n, kRecordAlign);
   uint8_t* ws = nullptr;
-  st = ws_acquire(c, L.total, stream, &ws);
-  if (st) return st;
-  c->plan.resize(L.nodes);
-  put(c->plan, L.banks, d);
-  put(c->plan, L.secs, koff);
-  PCS_CUDA(plan_copy(c, ws, L.nodes, stream));
-  if (kept_off)
-    PCS_CUDA(cudaMemcpyAsync(kept_off, ws + L.secs, 4ull * (n + 1), cudaMemcpyDeviceToDevice, stream));
-  float* sc = scores ? scores : reinterpret_cast<float*>(ws + L.nodes);
-  auto* dbanks = reinterpret_cast<const BankDesc*>(ws + L.banks);
-  PCS_CUDA(launch_bank_scores(c, banks, n, dbanks, entries, sc, stream));
+  if (!sent || !scores) {
+    st = ws_acquire(c, o_sc + (scores ? 0 : 4 * entries), stream, &ws);
+    if (st) return st;
+    c->plan_slot_used = -1;
+  }
+  if (!sent) {
+    c->plan.resize(sizeof(BankDesc) * n);
+    put(c->plan, 0, d);
+    PCS_CUDA(plan_copy(c, ws, c->plan.size(), stream));
+  }
+  float* sc = scores ? scores : reinterpret_cast<float*>(ws + o_sc);
+  const Banks descs{d.data(), sent ? nullptr : reinterpret_cast<const BankDesc*>(ws), n};
+  PCS_CUDA(launch_bank_scores(c, banks, n, descs, entries, sc, stream));
   {
     LaunchScope ls(c, kKTopk, stream);
-    PCS_CUDA(launch_topk(dbanks, n, sc, kept_idx, stream));
+    PCS_CUDA(launch_topk(descs, sc, kept_idx, kept_off, static_cast<int32_t>(kept), stream));
   }
-  return ws_release(c, stream);
+  return ws ? ws_release(c, stream) : PCS_OK;
 }
 
 pcs_status pcs_topk(pcs_ctx* c, const float* keys, const int32_t* n, const int32_t* k,
@@ -1931,7 +1931,6 @@ pcs_status pcs_topk(pcs_ctx* c, const float* keys, const int32_t* n, const int32
   if (n_banks == 0) return PCS_OK;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   std::vector<BankDesc> d(n_banks);
-  std::vector<int32_t> koff(n_banks + 1, 0);
   uint64_t entries = 0, kept = 0;
   for (int b = 0; b < n_banks; ++b) {
     if (n[b] < 0 || k[b] < 0) return fail(PCS_E_INVAL, "bank %d: negative n or k", b);
@@ -1941,7 +1940,6 @@ pcs_status pcs_topk(pcs_ctx* c, const float* keys, const int32_t* n, const int32
     d[b].k = std::min(k[b], n[b]);
     entries += n[b];
     kept += d[b].k;
-    koff[b + 1] = static_cast<int32_t>(kept);
   }
   if (entries > 0 && !keys) return fail(PCS_E_INVAL, "keys is null");
   if (kept > 0 && !kept_idx) return fail(PCS_E_INVAL, "kept_idx is null");
@@ -1949,23 +1947,21 @@ pcs_status pcs_topk(pcs_ctx* c, const float* keys, const int32_t* n, const int32
   std::lock_guard<std::mutex> lk(c->mu);
   pcs_status st = set_device(c);
   if (st) return st;
-  const uint64_t off_at = round_up(sizeof(BankDesc) * n_banks, kRecordAlign);
-  const uint64_t total = off_at + 4ull * (n_banks + 1);
+  const bool sent = n_banks <= kBankBlob;
   uint8_t* ws = nullptr;
-  st = ws_acquire(c, total, stream, &ws);
-  if (st) return st;
-  c->plan.resize(total);
-  put(c->plan, 0, d);
-  put(c->plan, off_at, koff);
-  PCS_CUDA(plan_copy(c, ws, total, stream));
-  if (kept_off)
-    PCS_CUDA(cudaMemcpyAsync(kept_off, ws + off_at, 4ull * (n_banks + 1), cudaMemcpyDeviceToDevice,
-                             stream));
+  if (!sent) {
+    st = ws_acquire(c, sizeof(BankDesc) * n_banks, stream, &ws);
+    if (st) return st;
+    c->plan.resize(sizeof(BankDesc) * n_banks);
+    put(c->plan, 0, d);
+    PCS_CUDA(plan_copy(c, ws, c->plan.size(), stream));
+  }
   {
     LaunchScope ls(c, kKTopk, stream);
-    PCS_CUDA(launch_topk(reinterpret_cast<const BankDesc*>(ws), n_banks, keys, kept_idx, stream));
+    PCS_CUDA(launch_topk({d.data(), reinterpret_cast<const BankDesc*>(ws), n_banks}, keys, kept_idx,
+                         kept_off, static_cast<int32_t>(kept), stream));
   }
-  return ws_release(c, stream);
+  return ws ? ws_release(c, stream) : PCS_OK;
 }
 
 // Digit schedule of the 64-bit ranking key (the same as the kernels'):
@@ -2078,22 +2074,28 @@ static pcs_status prune_global_impl(pcs_ctx* c, const pcs_bank* banks, int32_t n
   if (!ex && entries <= kGSmallEntries && n <= kGSmallBanks) {
     // Small: a plain score pass, then one block (its descriptors are the
     // banks' alone).
-    const uint64_t o_sc = round_up(sizeof(BankDesc) * n, kRecordAlign);
+    const bool sent = n <= kBankBlob;
+    const uint64_t o_sc = sent ? 0 : round_up(sizeof(BankDesc) * n, kRecordAlign);
     uint8_t* ws = nullptr;
-    st = ws_acquire(c, o_sc + (scores ? 0 : 4ull * entries), stream, &ws);
-    if (st) return st;
-    c->plan.resize(o_sc);
-    put(c->plan, 0, d);
-    PCS_CUDA(plan_copy(c, ws, sizeof(BankDesc) * n, stream));
+    if (!sent || !scores) {
+      st = ws_acquire(c, o_sc + (scores ? 0 : 4ull * entries), stream, &ws);
+      if (st) return st;
+      c->plan_slot_used = -1;
+    }
+    if (!sent) {
+      c->plan.resize(sizeof(BankDesc) * n);
+      put(c->plan, 0, d);
+      PCS_CUDA(plan_copy(c, ws, c->plan.size(), stream));
+    }
     float* sc = scores ? scores : reinterpret_cast<float*>(ws + o_sc);
-    const auto* dbanks = reinterpret_cast<const BankDesc*>(ws);
-    PCS_CUDA(launch_bank_scores(c, banks, n, dbanks, entries, sc, stream));
+    const Banks descs{d.data(), sent ? nullptr : reinterpret_cast<const BankDesc*>(ws), n};
+    PCS_CUDA(launch_bank_scores(c, banks, n, descs, entries, sc, stream));
     {
       LaunchScope ls(c, kKGFinish, stream);
-      PCS_CUDA(launch_gsmall(dbanks, n, entries, sc, budget, uniform, total <= budget, kept_idx,
+      PCS_CUDA(launch_gsmall(descs, entries, sc, budget, uniform, total <= budget, kept_idx,
                              kept_off, stream));
     }
-    return ws_release(c, stream);
+    return ws ? ws_release(c, stream) : PCS_OK;
   }
   const uint64_t tiles = (entries + kGTile - 1) / kGTile;
   // Bank of entry min(t * kGTile, entries - 1), t = 0..tiles.
@@ -2151,8 +2153,8 @@ static pcs_status prune_global_impl(pcs_ctx* c, const pcs_bank* banks, int32_t n
     gh.mode = uniform ? 1 : 2;
   }
   bool fused = false;
-  PCS_CUDA(launch_bank_scores(c, banks, n, reinterpret_cast<const BankDesc*>(ws), entries, sc,
-                              stream, gh, &fused));
+  PCS_CUDA(launch_bank_scores(c, banks, n, {d.data(), reinterpret_cast<const BankDesc*>(ws), n},
+                              entries, sc, stream, gh, &fused));
   GPlan gp{};
   gp.scores = sc;
   gp.ebeg = reinterpret_cast<const uint64_t*>(ws + o_ebeg);
@@ -2967,26 +2969,35 @@ pcs_status pcs_mismatch(pcs_ctx* c, const pcs_buf* a, const pcs_buf* b, int32_t 
   std::lock_guard<std::mutex> lk(c->mu);
   pcs_status st = set_device(c);
   if (st) return st;
+  const bool sent = n <= kMmBlob && tiles > 0;
   const uint64_t o_tb = round_up(sizeof(MmPair) * n, kRecordAlign);
   const uint64_t o_ex = round_up(o_tb + 8ull * (n + 1), kRecordAlign);
-  const uint64_t total = o_ex + 8ull * n;
+  const uint64_t total = sent ? 0 : o_ex + 8ull * n;
   uint8_t* ws = nullptr;
   st = ws_acquire(c, total, stream, &ws);
   if (st) return st;
-  c->plan.assign(total, 0);
-  put(c->plan, 0, pairs);
-  put(c->plan, o_tb, tb);
-  put(c->plan, o_ex, extra);
-  PCS_CUDA(plan_copy(c, ws, total, stream));
+  c->plan_slot_used = -1;
+  if (!sent) {
+    c->plan.assign(total, 0);
+    put(c->plan, 0, pairs);
+    put(c->plan, o_tb, tb);
+    put(c->plan, o_ex, extra);
+    PCS_CUDA(plan_copy(c, ws, total, stream));
+  }
   // Counts start at the bytes only one buffer has.
   if (tiles == 0) {
     PCS_CUDA(cudaMemcpyAsync(counts, ws + o_ex, 8ull * n, cudaMemcpyDeviceToDevice, stream));
   } else {
     LaunchScope ls(c, kKMismatch, stream);
-    PCS_CUDA(launch_mismatch(reinterpret_cast<const MmPair*>(ws),
-                             reinterpret_cast<const uint64_t*>(ws + o_tb), n, tiles,
-                             reinterpret_cast<uint64_t*>(ws + o_ex), counts, c->call_words,
-                             c->sm_count, stream));
+    if (sent)
+      PCS_CUDA(launch_mismatch(true, pairs.data(), tb.data(), extra.data(), n, tiles,
+                               reinterpret_cast<uint64_t*>(c->call_words + kWordSums), counts,
+                               c->call_words, c->sm_count, stream));
+    else
+      PCS_CUDA(launch_mismatch(false, reinterpret_cast<const MmPair*>(ws),
+                               reinterpret_cast<const uint64_t*>(ws + o_tb), nullptr, n, tiles,
+                               reinterpret_cast<uint64_t*>(ws + o_ex), counts, c->call_words,
+                               c->sm_count, stream));
   }
   return ws_release(c, stream);
 }
@@ -3024,32 +3035,43 @@ pcs_status pcs_classify_reads(pcs_ctx* c, const pcs_buf* bufs, int32_t n, const 
     PCS_CUDA(cudaMemsetAsync(flags, 0, n, stream));
     return PCS_OK;
   }
+  const bool sent = n <= kReadBlob;
   const uint64_t o_en = round_up(8ull * nn, 256), o_mx = round_up(o_en + 8ull * nn, 256);
   const uint64_t o_or = round_up(o_mx + 8ull * nn, 256), o_bm = round_up(o_or + 4ull * n, 256);
-  const uint64_t total = o_bm + 4ull * ((nn + 31) / 32);
+  const uint64_t total = sent ? 0 : o_bm + 4ull * ((nn + 31) / 32);
   uint8_t* ws = nullptr;
   st = ws_acquire(c, total, stream, &ws);
   if (st) return st;
-  c->plan.assign(total, 0);
-  put(c->plan, 0, st_);
-  put(c->plan, o_en, en);
-  put(c->plan, o_mx, mx);
-  put(c->plan, o_or, ord);
-  PCS_CUDA(plan_copy(c, ws, total, stream));
+  c->plan_slot_used = -1;
   ReadPlan rp{};
-  rp.start = reinterpret_cast<const uint64_t*>(ws);
-  rp.end = reinterpret_cast<const uint64_t*>(ws + o_en);
-  rp.maxend = reinterpret_cast<const uint64_t*>(ws + o_mx);
-  rp.orig = reinterpret_cast<const uint32_t*>(ws + o_or);
-  rp.bitmap = reinterpret_cast<uint32_t*>(ws + o_bm);
   rp.ticket = c->call_words;
   rp.n = nn;
   rp.n_all = n;
   rp.base = st_[0];
   rp.top = mx[nn - 1];
+  if (sent) {
+    rp.start = st_.data();
+    rp.end = en.data();
+    rp.maxend = mx.data();
+    rp.orig = ord.data();
+    rp.bitmap = c->call_words + kWordSums;
+  } else {
+    c->plan.assign(total, 0);
+    put(c->plan, 0, st_);
+    put(c->plan, o_en, en);
+    put(c->plan, o_mx, mx);
+    put(c->plan, o_or, ord);
+    PCS_CUDA(plan_copy(c, ws, total, stream));
+    rp.start = reinterpret_cast<const uint64_t*>(ws);
+    rp.end = reinterpret_cast<const uint64_t*>(ws + o_en);
+    rp.maxend = reinterpret_cast<const uint64_t*>(ws + o_mx);
+    rp.orig = reinterpret_cast<const uint32_t*>(ws + o_or);
+    rp.bitmap = reinterpret_cast<uint32_t*>(ws + o_bm);
+  }
   {
     LaunchScope ls(c, kKClassifyReads, stream);
-    PCS_CUDA(launch_classify_reads(rp, addr, bytes, m, flags, c->sm_count, stream));
+    PCS_CUDA(launch_classify_reads(sent, rp, addr, bytes, m, flags, c->sm_count,
+                                   stream));
   }
   return ws_release(c, stream);
 }
