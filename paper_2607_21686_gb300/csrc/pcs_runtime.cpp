@@ -389,6 +389,7 @@ struct pcs_ctx {
   Ev plan_slot_busy[8];
   int plan_slot = 0;
   int plan_slot_used = -1;     // slot of the call in progress, or -1
+  bool uploaded = false;       // its descriptors are sent by a kernel, the last launched so far
   uint8_t* stage = nullptr;    // pinned staging for file I/O
   uint64_t stage_bytes = 0;
   uint64_t launches = 0;       // kernels launched by this context
@@ -420,7 +421,7 @@ enum KernelKind {
   kKStreamHash, kKStreamPack, kKStreamRestore, kKStreamRestoreV, kKFinalizeHash,
   kKFinalizePack, kKFinalizeRestoreV, kKScore, kKTopk, kKBulkHash, kKBulkPack,
   kKBulkRestore, kKBulkRestoreV, kKReduce, kKGSelect, kKGFinish, kKPoolAlloc, kKPoolShare,
-  kKPoolCow, kKPoolRelease, kKMismatch, kKClassifyReads, kKernelKinds
+  kKPoolCow, kKPoolRelease, kKMismatch, kKClassifyReads, kKUpload, kKernelKinds
 };
 static_assert(kKernelKinds <= 32, "kernel timing table");
 const char* kKernelNames[kKernelKinds] = {
@@ -428,7 +429,7 @@ const char* kKernelNames[kKernelKinds] = {
     "k_finalize<hash>", "k_finalize<pack>", "k_finalize<restore_verify>", "k_score", "k_topk",
     "k_hash", "k_bulk<pack>", "k_bulk<restore>", "k_bulk<restore_verify>",
     "k_reduce_nodes", "k_gselect", "k_gfinish", "k_pool_alloc", "k_pool_share", "k_pool_cow",
-    "k_pool_release", "k_mismatch", "k_classify_reads"};
+    "k_pool_release", "k_mismatch", "k_classify_reads", "k_upload"};
 
 cudaEvent_t timing_event(pcs_ctx* c) {
   if (!c->timing_events.empty()) {
@@ -530,6 +531,7 @@ pcs_status ws_acquire(pcs_ctx* c, uint64_t bytes, cudaStream_t stream, uint8_t**
 }
 
 constexpr uint64_t kPlanSlotBytes = 256 << 10;  // smallest pinned plan slot
+constexpr uint64_t kUploadMax = 1ull << 20;     // larger plans are copied by a copy engine
 constexpr uint64_t kPlanSlotMax = 64ull << 20;  // larger plans are copied from pageable memory
 constexpr int kPlanSlots = 8;
 
@@ -551,7 +553,7 @@ uint8_t* plan_slot(pcs_ctx* c, uint64_t bytes) {
         uint64_t cap = kPlanSlotBytes;
         while (cap < bytes) cap *= 2;
         void* p = nullptr;
-        if (cudaHostAlloc(&p, cap, cudaHostAllocDefault) == cudaSuccess) {
+        if (cudaHostAlloc(&p, cap, cudaHostAllocMapped) == cudaSuccess) {
           c->plan_slot_buf[i] = static_cast<uint8_t*>(p);
           c->plan_slot_cap[i] = cap;
         } else {
@@ -577,18 +579,30 @@ uint8_t* plan_dst(pcs_ctx* c, uint64_t bytes, std::vector<uint8_t>& fallback) {
   return fallback.data();
 }
 
-// Send descriptors written where plan_dst said into the workspace.
+// Send descriptors written where plan_dst said into the workspace: by a kernel
+// where they are in a pinned slot and at most kUploadMax, else by a copy.
+// c->uploaded says which, for the launch that follows.  One launch is not
+// worth a kernel ahead of it (`by_kernel` false): it costs the host about a
+// microsecond more than the copy, which bounds such calls (a log against 150
+// buffers 11.5 -> 12.2 us).
 cudaError_t plan_send(pcs_ctx* c, uint8_t* ws, uint64_t bytes,
-                        const std::vector<uint8_t>& fallback, cudaStream_t stream) {
+                      const std::vector<uint8_t>& fallback, cudaStream_t stream,
+                      bool by_kernel = true) {
+  c->uploaded = by_kernel && c->plan_slot_used >= 0 && bytes <= kUploadMax;
+  if (c->uploaded) {
+    LaunchScope ls(c, kKUpload, stream);
+    return launch_upload(ws, c->plan_slot_buf[c->plan_slot_used], bytes, stream);
+  }
   const uint8_t* src = c->plan_slot_used >= 0 ? c->plan_slot_buf[c->plan_slot_used] : fallback.data();
   return cudaMemcpyAsync(ws, src, bytes, cudaMemcpyHostToDevice, stream);
 }
 
 // Copy the call's descriptors (c->plan, `bytes`) into the workspace, through
 // a pinned slot when one is free.
-cudaError_t plan_copy(pcs_ctx* c, uint8_t* ws, uint64_t bytes, cudaStream_t stream) {
+cudaError_t plan_copy(pcs_ctx* c, uint8_t* ws, uint64_t bytes, cudaStream_t stream,
+                      bool by_kernel = true) {
   if (uint8_t* slot = plan_slot(c, bytes)) std::memcpy(slot, c->plan.data(), bytes);
-  return plan_send(c, ws, bytes, c->plan, stream);
+  return plan_send(c, ws, bytes, c->plan, stream, by_kernel);
 }
 
 // End of a call's use of the workspace (and of its plan slot): `done`, if
@@ -1117,7 +1131,7 @@ SmallArgs small_args(pcs_ctx* c, const StreamPlan& P, const ListLayout& L, uint8
 // Launch both streaming kernels of a plan (TMA-staged first).
 cudaError_t launch_streams(pcs_ctx* c, int mode, const SecDesc* dsecs, const StreamPlan& P,
                            const ListLayout& L, uint8_t* ws, uint64_t* nodes,
-                           cudaStream_t stream);
+                           cudaStream_t stream, bool early);
 
 // Fingerprint (and optionally classify) contiguous buffers.
 pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t* fp_out,
@@ -1174,7 +1188,7 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
                           c->stream_bps, stream));
     return ws_release(c, stream);
   }
-  PCS_CUDA(launch_streams(c, kModeHash, dsecs, P, LL, ws, nodes, stream));
+  PCS_CUDA(launch_streams(c, kModeHash, dsecs, P, LL, ws, nodes, stream, !c->uploaded));
   {
     LaunchScope ls(c, kKFinalizeHash, stream);
     PCS_CUDA(launch_finalize(kModeHash, dsecs, nullptr, n, nullptr, nodes, fp_out, fp_before,
@@ -1185,23 +1199,24 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
 
 cudaError_t launch_streams(pcs_ctx* c, int mode, const SecDesc* dsecs, const StreamPlan& P,
                            const ListLayout& L, uint8_t* ws, uint64_t* nodes,
-                           cudaStream_t stream) {
+                           cudaStream_t stream, bool early) {
   cudaError_t e = cudaSuccess;
   if (P.bulk_tasks) {
     WorkList wl{reinterpret_cast<const uint32_t*>(ws + L.bulk_ids),
                 reinterpret_cast<const uint32_t*>(ws + L.bulk_begin),
                 static_cast<int>(P.bulk_ids.size()), P.bulk_tasks};
     LaunchScope ls(c, bulk_kind(mode), stream);
-    e = launch_bulk(mode, P.bulk_shift, dsecs, wl, nodes, c->words, header_words(ws) + kWordBulkSched, c->sm_count,
+    e = launch_bulk(mode, P.bulk_shift, early, dsecs, wl, nodes, c->words, header_words(ws) + kWordBulkSched, c->sm_count,
                     stream);
     if (e != cudaSuccess) return e;
+    early = true;
   }
   if (P.reg_tasks) {
     WorkList wl{reinterpret_cast<const uint32_t*>(ws + L.reg_ids),
                 reinterpret_cast<const uint32_t*>(ws + L.reg_begin),
                 static_cast<int>(P.reg_ids.size()), P.reg_tasks};
     LaunchScope ls(c, stream_kind(mode), stream);
-    e = launch_stream(mode, dsecs, wl, P.glog2, nodes, c->words, grid_sms(c, P), c->stream_bps,
+    e = launch_stream(mode, early, dsecs, wl, P.glog2, nodes, c->words, grid_sms(c, P), c->stream_bps,
                       stream);
     if (e != cudaSuccess) return e;
   }
@@ -1309,7 +1324,7 @@ uint32_t* plan_words(const pcs_plan* p) { return reinterpret_cast<uint32_t*>(p->
 // Launch a prepared call whose descriptors are at `ws` (nodes after them);
 // `words` are the call's header words (ticket of the fused kernel).
 cudaError_t launch_prepared(pcs_ctx* c, const Prepared& pr, uint8_t* ws, uint32_t* words,
-                            cudaStream_t stream) {
+                            cudaStream_t stream, bool early = true) {
   const auto* dsecs = reinterpret_cast<const SecDesc*>(ws + pr.L.secs);
   const auto* dsess = reinterpret_cast<const SessDesc*>(ws + pr.L.sess);
   auto* nodes = reinterpret_cast<uint64_t*>(ws + pr.L.nodes);
@@ -1328,7 +1343,7 @@ cudaError_t launch_prepared(pcs_ctx* c, const Prepared& pr, uint8_t* ws, uint32_
       LaunchScope ls(c, kKStreamPack, stream);
       return launch_small(kModePack, sent, pr.LL.end, args(), c->sm_count, c->stream_bps, stream);
     }
-    cudaError_t e = launch_streams(c, kModePack, dsecs, pr.P, pr.LL, ws, nodes, stream);
+    cudaError_t e = launch_streams(c, kModePack, dsecs, pr.P, pr.LL, ws, nodes, stream, early);
     if (e != cudaSuccess) return e;
     LaunchScope ls(c, kKFinalizePack, stream);
     return launch_finalize(kModePack, dsecs, dsess, pr.n, dent, nodes, nullptr, nullptr, nullptr,
@@ -1342,7 +1357,7 @@ cudaError_t launch_prepared(pcs_ctx* c, const Prepared& pr, uint8_t* ws, uint32_
     return launch_small(kModeRestoreV, sent, pr.LL.end, a, c->sm_count, c->stream_bps, stream);
   }
   cudaError_t e = launch_streams(c, pr.verify ? kModeRestoreV : kModeRestore, dsecs, pr.P, pr.LL,
-                                 ws, pr.verify ? nodes : nullptr, stream);
+                                 ws, pr.verify ? nodes : nullptr, stream, early);
   if (e != cudaSuccess || !pr.verify) return e;
   LaunchScope ls(c, kKFinalizeRestoreV, stream);
   return launch_finalize(kModeRestoreV, dsecs, dsess, pr.n, nullptr, nodes, nullptr, nullptr,
@@ -1915,8 +1930,10 @@ pcs_status pcs_prune(pcs_ctx* c, const pcs_bank* banks, int32_t n, const pcs_pru
     PCS_CUDA(plan_copy(c, ws, c->plan.size(), stream));
   }
   float* sc = scores ? scores : reinterpret_cast<float*>(ws + o_sc);
-  const Banks descs{d.data(), sent ? nullptr : reinterpret_cast<const BankDesc*>(ws), n};
+  Banks descs{d.data(), sent ? nullptr : reinterpret_cast<const BankDesc*>(ws), n};
+  descs.early = sent || !c->uploaded;
   PCS_CUDA(launch_bank_scores(c, banks, n, descs, entries, sc, stream));
+  if (entries > 0) descs.early = true;
   {
     LaunchScope ls(c, kKTopk, stream);
     PCS_CUDA(launch_topk(descs, sc, kept_idx, kept_off, static_cast<int32_t>(kept), stream));
@@ -1954,7 +1971,7 @@ pcs_status pcs_topk(pcs_ctx* c, const float* keys, const int32_t* n, const int32
     if (st) return st;
     c->plan.resize(sizeof(BankDesc) * n_banks);
     put(c->plan, 0, d);
-    PCS_CUDA(plan_copy(c, ws, c->plan.size(), stream));
+    PCS_CUDA(plan_copy(c, ws, c->plan.size(), stream, false));
   }
   {
     LaunchScope ls(c, kKTopk, stream);
@@ -2088,7 +2105,8 @@ static pcs_status prune_global_impl(pcs_ctx* c, const pcs_bank* banks, int32_t n
       PCS_CUDA(plan_copy(c, ws, c->plan.size(), stream));
     }
     float* sc = scores ? scores : reinterpret_cast<float*>(ws + o_sc);
-    const Banks descs{d.data(), sent ? nullptr : reinterpret_cast<const BankDesc*>(ws), n};
+    Banks descs{d.data(), sent ? nullptr : reinterpret_cast<const BankDesc*>(ws), n};
+    descs.early = sent || !c->uploaded;
     PCS_CUDA(launch_bank_scores(c, banks, n, descs, entries, sc, stream));
     {
       LaunchScope ls(c, kKGFinish, stream);
@@ -2153,7 +2171,8 @@ static pcs_status prune_global_impl(pcs_ctx* c, const pcs_bank* banks, int32_t n
     gh.mode = uniform ? 1 : 2;
   }
   bool fused = false;
-  PCS_CUDA(launch_bank_scores(c, banks, n, {d.data(), reinterpret_cast<const BankDesc*>(ws), n},
+  PCS_CUDA(launch_bank_scores(c, banks, n,
+                              {d.data(), reinterpret_cast<const BankDesc*>(ws), n, !c->uploaded},
                               entries, sc, stream, gh, &fused));
   GPlan gp{};
   gp.scores = sc;
@@ -2290,8 +2309,9 @@ pcs_status pcs_checkpoint(pcs_ctx* c, const pcs_session* sessions, int32_t n, ui
   st = ws_acquire(c, pr.L.total, stream, &ws);
   if (st) return undo(st);
   cudaError_t e = cudaSuccess;
+  c->uploaded = false;
   if (!pr.in_launch) e = plan_send(c, ws, pr.L.nodes, pr.plan, stream);
-  if (e == cudaSuccess) e = launch_prepared(c, pr, ws, c->call_words, stream);
+  if (e == cudaSuccess) e = launch_prepared(c, pr, ws, c->call_words, stream, !c->uploaded);
   if (e != cudaSuccess) return undo(cuda_fail(e, "checkpoint launch"));
   blk->written = record_event(c->events, stream);
   st = ws_release(c, stream, blk->written);
@@ -2376,7 +2396,7 @@ pcs_status pcs_fork_many(pcs_ctx* c, pcs_snapshot* const* parents, int32_t n,
   cudaError_t e = plan_copy(c, ws, total, stream);
   if (e == cudaSuccess)
     e = launch_streams(c, kModeRestore, reinterpret_cast<const SecDesc*>(ws), P, LL, ws, nullptr,
-                       stream);
+                       stream, !c->uploaded);
   if (e != cudaSuccess) return undo(cuda_fail(e, "fork copy"));
   Ev done = record_event(c->events, stream);
   st = ws_release(c, stream, done);
@@ -2430,12 +2450,14 @@ pcs_status pcs_restore(pcs_ctx* c, pcs_snapshot* const* snaps, int32_t n, const 
   uint8_t* ws = nullptr;
   st = ws_acquire(c, pr.L.total, stream, &ws);
   if (st) return st;
+  c->uploaded = false;
   if (!pr.in_launch) PCS_CUDA(plan_send(c, ws, pr.L.nodes, pr.plan, stream));
   // verify == 1: count failures of this call in words[1] and wait for them;
   // verify == 2: accumulate them in words[2] for the next pcs_sync.
   uint32_t* words = c->call_words;
+  const bool early = !c->uploaded || verify == 1;  // (after a memset the launch waits anyway)
   if (verify == 1) PCS_CUDA(cudaMemsetAsync(words + 1, 0, 4, stream));
-  PCS_CUDA(launch_prepared(c, pr, ws, words, stream));
+  PCS_CUDA(launch_prepared(c, pr, ws, words, stream, early));
   for (int s = 0; s < n; ++s) {
     if (s > 0 && snaps[s]->block == snaps[s - 1]->block) continue;
     st = note_use(c, snaps[s]->block, stream);
@@ -2982,7 +3004,7 @@ pcs_status pcs_mismatch(pcs_ctx* c, const pcs_buf* a, const pcs_buf* b, int32_t 
     put(c->plan, 0, pairs);
     put(c->plan, o_tb, tb);
     put(c->plan, o_ex, extra);
-    PCS_CUDA(plan_copy(c, ws, total, stream));
+    PCS_CUDA(plan_copy(c, ws, total, stream, false));
   }
   // Counts start at the bytes only one buffer has.
   if (tiles == 0) {
@@ -3061,7 +3083,7 @@ pcs_status pcs_classify_reads(pcs_ctx* c, const pcs_buf* bufs, int32_t n, const 
     put(c->plan, o_en, en);
     put(c->plan, o_mx, mx);
     put(c->plan, o_or, ord);
-    PCS_CUDA(plan_copy(c, ws, total, stream));
+    PCS_CUDA(plan_copy(c, ws, total, stream, false));
     rp.start = reinterpret_cast<const uint64_t*>(ws);
     rp.end = reinterpret_cast<const uint64_t*>(ws + o_en);
     rp.maxend = reinterpret_cast<const uint64_t*>(ws + o_mx);
