@@ -121,9 +121,11 @@ constexpr uint64_t kBulkMinRowBytes = 512;
 // one ahead on the stream has finished; false right after launch_upload.
 
 // Register kernel: warp tasks of 2^group_log2 chunks, 128-bit loads/stores.
-cudaError_t launch_stream(int mode, bool early, const SecDesc* secs, WorkList wl, int group_log2,
-                          uint64_t* nodes, uint32_t* dev_err, int sm_count, int blocks_per_sm,
-                          cudaStream_t stream);
+// `beside`: the launch just before it on the stream is the same call's
+// launch_bulk, and the two run side by side.
+cudaError_t launch_stream(int mode, bool early, bool beside, const SecDesc* secs, WorkList wl,
+                          int group_log2, uint64_t* nodes, uint32_t* dev_err, int sm_count,
+                          int blocks_per_sm, cudaStream_t stream);
 
 // TMA-staged kernel: tasks of kBulkTileChunks chunks staged through shared
 // memory with cp.async.bulk; one persistent block per SM.  `sched`: two

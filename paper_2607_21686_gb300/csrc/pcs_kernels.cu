@@ -97,9 +97,15 @@ __device__ __forceinline__ void prefetch_l1(const void* p) {
 // scheduled.  Before this point a kernel reads only what the host wrote
 // before the launch (work lists and section, session and bank
 // descriptors), which no kernel writes.
-__device__ __forceinline__ void grid_dependency() {
+__device__ __forceinline__ void grid_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void grid_release() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dependency() {
+  grid_wait();
+  grid_release();
 }
 
 // Absorb one 16-byte segment (two little-endian words) into a lane chain.
@@ -559,7 +565,8 @@ __device__ __forceinline__ int find_item(const uint32_t* begin, int lo, int n_it
 template <int MODE, bool GLOBAL, typename F>
 __device__ __forceinline__ void run_stream_tasks(const SecDesc* secs, const WorkList& wl,
                                                  int glog2, uint64_t* __restrict__ nodes,
-                                                 uint32_t* err, SecDesc* sdesc, F&& after_task) {
+                                                 uint32_t* err, SecDesc* sdesc, bool beside,
+                                                 F&& after_task) {
   using T = ModeTraits<MODE>;
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
@@ -580,7 +587,8 @@ __device__ __forceinline__ void run_stream_tasks(const SecDesc* secs, const Work
   };
   int j = 0, cur = -1;
   if (t0 < t1) load_desc(cur = j = find_item<GLOBAL>(wl.begin, 0, wl.n_items, t0, lane));
-  grid_dependency();
+  if (beside) grid_release();
+  else grid_dependency();
   for (uint32_t task = t0; task < t1; ++task) {
     while (j + 1 < wl.n_items && fetch<GLOBAL>(wl.begin + j + 1) <= task) ++j;
     if (j != cur) load_desc(cur = j);
@@ -604,12 +612,21 @@ __device__ __forceinline__ void run_stream_tasks(const SecDesc* secs, const Work
   }
 }
 
+// beside: the kernel ahead on the stream is the TMA (or hash) kernel of the
+// same call, which shares nothing with this one, so this one runs beside it
+// and waits for it only before it ends (what follows them waits for both so).
+// It can start once every block ahead has passed its own wait, so whatever
+// came before the call is finished and visible by then.  Measured, whole
+// calls: planned checkpoint + restore of odd observations 14.7 -> 11.6 us, the
+// classification of buffers off and on a boundary 80.8 -> 75.6 and 90.3 -> 87.7.
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, 2)
     k_stream(const SecDesc* __restrict__ secs, WorkList wl, int glog2,
-             uint64_t* __restrict__ nodes, uint32_t* err) {
+             uint64_t* __restrict__ nodes, uint32_t* err, bool beside) {
   __shared__ SecDesc sdesc[kWarps];
-  run_stream_tasks<MODE, true>(secs, wl, glog2, nodes, err, sdesc, [](const SecDesc&, int) {});
+  run_stream_tasks<MODE, true>(secs, wl, glog2, nodes, err, sdesc, beside,
+                               [](const SecDesc&, int) {});
+  if (beside) grid_wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -1571,7 +1588,8 @@ __global__ void __launch_bounds__(kThreads, 2)
   __shared__ SecDesc sdesc[kWarps];
   const int lane = threadIdx.x & 31;
   if (MODE == kModeHash || a.max_secs <= 32) {
-    run_stream_tasks<MODE, GLOBAL>(secs, wl, a.glog2, nodes, a.err, sdesc, [&](const SecDesc& s, int j) {
+    run_stream_tasks<MODE, GLOBAL>(secs, wl, a.glog2, nodes, a.err, sdesc, false,
+                                   [&](const SecDesc& s, int j) {
       const uint32_t i = MODE == kModeHash ? fetch<GLOBAL>(wl.ids + j) : s.sess;
       SessDesc S{};
       SessLane l{};
@@ -1604,7 +1622,8 @@ __global__ void __launch_bounds__(kThreads, 2)
   __shared__ uint64_t smem[64];  // up to 2048 sections per session
   __shared__ uint32_t s_bad;
   __shared__ bool s_last;
-  run_stream_tasks<MODE, GLOBAL>(secs, wl, a.glog2, nodes, a.err, sdesc, [](const SecDesc&, int) {});
+  run_stream_tasks<MODE, GLOBAL>(secs, wl, a.glog2, nodes, a.err, sdesc, false,
+                                 [](const SecDesc&, int) {});
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) s_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
@@ -3669,28 +3688,23 @@ cudaError_t launch_upload(void* dst, const void* src, uint64_t bytes, cudaStream
 
 int stream_blocks_per_sm() { return occupancy<kModePack>(); }
 
-cudaError_t launch_stream(int mode, bool early, const SecDesc* secs, WorkList wl, int group_log2,
-                          uint64_t* nodes, uint32_t* dev_err, int sm_count, int blocks_per_sm,
-                          cudaStream_t stream) {
+cudaError_t launch_stream(int mode, bool early, bool beside, const SecDesc* secs, WorkList wl,
+                          int group_log2, uint64_t* nodes, uint32_t* dev_err, int sm_count,
+                          int blocks_per_sm, cudaStream_t stream) {
   if (wl.n_tasks == 0) return cudaSuccess;
   const uint64_t want = (static_cast<uint64_t>(wl.n_tasks) + kWarps - 1) / kWarps;
   const uint64_t cap = static_cast<uint64_t>(sm_count) * blocks_per_sm;
   const int blocks = static_cast<int>(want < cap ? want : cap);
+  auto launch = [&](auto kernel) {
+    return launch_on(early, kernel, blocks, kThreads, 0, stream, secs, wl, group_log2, nodes,
+                     dev_err, beside);
+  };
   switch (mode) {
-    case kModeHash:
-      return launch_on(early, k_stream<kModeHash>, blocks, kThreads, 0, stream, secs, wl, group_log2,
-                          nodes, dev_err);
-    case kModePack:
-      return launch_on(early, k_stream<kModePack>, blocks, kThreads, 0, stream, secs, wl, group_log2,
-                          nodes, dev_err);
-    case kModeRestore:
-      return launch_on(early, k_stream<kModeRestore>, blocks, kThreads, 0, stream, secs, wl,
-                          group_log2, nodes, dev_err);
-    case kModeRestoreV:
-      return launch_on(early, k_stream<kModeRestoreV>, blocks, kThreads, 0, stream, secs, wl,
-                          group_log2, nodes, dev_err);
-    default:
-      return cudaErrorInvalidValue;
+    case kModeHash: return launch(k_stream<kModeHash>);
+    case kModePack: return launch(k_stream<kModePack>);
+    case kModeRestore: return launch(k_stream<kModeRestore>);
+    case kModeRestoreV: return launch(k_stream<kModeRestoreV>);
+    default: return cudaErrorInvalidValue;
   }
 }
 

@@ -1216,7 +1216,7 @@ cudaError_t launch_streams(pcs_ctx* c, int mode, const SecDesc* dsecs, const Str
                 reinterpret_cast<const uint32_t*>(ws + L.reg_begin),
                 static_cast<int>(P.reg_ids.size()), P.reg_tasks};
     LaunchScope ls(c, stream_kind(mode), stream);
-    e = launch_stream(mode, early, dsecs, wl, P.glog2, nodes, c->words, grid_sms(c, P), c->stream_bps,
+    e = launch_stream(mode, early, P.bulk_tasks > 0, dsecs, wl, P.glog2, nodes, c->words, grid_sms(c, P), c->stream_bps,
                       stream);
     if (e != cudaSuccess) return e;
   }
