@@ -145,6 +145,10 @@ struct Slab {
   std::map<uint64_t, Range> free;  // offset -> free range
 };
 
+// A call's section tables, kept by every block whose snapshots point into them
+// (one count per block, not per snapshot).
+using Tables = std::shared_ptr<const std::vector<Entry>>;
+
 struct Block {
   Slab* slab = nullptr;
   uint64_t off = 0;
@@ -152,6 +156,7 @@ struct Block {
   uint8_t* ptr = nullptr;
   uint32_t placement = PCS_PLACE_DEVICE;
   int refs = 0;
+  std::vector<Tables> tables;                 // section tables of its snapshots
   Ev written;                                 // completion of the write
   std::map<cudaStream_t, Ev> uses;            // latest use per stream
 };
@@ -335,12 +340,11 @@ struct pcs_snapshot {
   uint64_t payload_start = 0;
   uint32_t session_id = 0;
   uint32_t kind = 0;
-  // Host copy of the section table (fp = 0): n_sections entries from
-  // `first` of an array shared by the snapshots of one call and their forks.
-  std::shared_ptr<const std::vector<Entry>> tables;
-  uint32_t first = 0;
+  // Host copy of the section table (fp = 0): n_sections entries, in an array
+  // that the block keeps (shared by the snapshots of one call and their forks).
+  const Entry* entries = nullptr;
   uint32_t n_sections = 0;
-  const Entry* table() const { return tables->data() + first; }
+  const Entry* table() const { return entries; }
   uint8_t* record() const { return block->ptr + offset; }
 };
 
@@ -350,6 +354,26 @@ struct pcs_pool {
 };
 
 struct pcs_plan;
+
+namespace {
+
+// Allocator of arrays whose elements are written right after a resize: they
+// are left uninitialised.
+template <class T>
+struct RawAlloc : std::allocator<T> {
+  template <class U>
+  struct rebind {
+    using other = RawAlloc<U>;
+  };
+  template <class U, class... A>
+  void construct(U* p, A&&... a) {
+    if constexpr (sizeof...(A) == 0) ::new (static_cast<void*>(p)) U;
+    else ::new (static_cast<void*>(p)) U(std::forward<A>(a)...);
+  }
+};
+using SecVec = std::vector<SecDesc, RawAlloc<SecDesc>>;
+
+}  // namespace
 
 struct pcs_ctx {
   int device = 0;
@@ -381,6 +405,7 @@ struct pcs_ctx {
   // failures until the next pcs_sync, [4] a flag nothing writes (self-test).
   uint32_t* words = nullptr;
   std::vector<uint8_t> plan;   // host staging of the descriptors
+  SecVec secs;                 // descriptors of the call in progress (see sec_array)
   // Pinned slots for the plans of calls: a true async copy, no driver-side
   // staging of pageable memory (which can hold the host until the stream
   // has caught up).  Each slot grows to the largest plan it has carried.
@@ -692,8 +717,19 @@ pcs_status check_section(const pcs_section& s, int sess, int i, bool target) {
   return PCS_OK;
 }
 
-SecDesc make_desc(const pcs_section& s, uint8_t* payload, uint32_t ring_start) {
-  SecDesc d{};
+// The call's descriptors, n of them, uninitialised: kept from call to call (a
+// call on thousands of sessions writes about a megabyte of them) up to 64 MiB.
+SecVec& sec_array(pcs_ctx* c, uint64_t n) {
+  constexpr uint64_t kKeep = (64ull << 20) / sizeof(SecDesc);
+  if (c->secs.capacity() > kKeep && n <= kKeep) SecVec().swap(c->secs);
+  c->secs.clear();
+  c->secs.resize(n);
+  return c->secs;
+}
+
+// Everything but the work (set by plan_streams).
+void make_desc(SecDesc& d, const pcs_section& s, uint8_t* payload, uint32_t ring_start,
+               uint32_t sess) {
   d.lbase = static_cast<uint8_t*>(s.base);
   d.payload = payload;
   d.index = s.index;
@@ -704,6 +740,7 @@ SecDesc make_desc(const pcs_section& s, uint8_t* payload, uint32_t ring_start) {
   d.ring_start = ring_start;
   d.window = s.window;
   d.page_rows = s.page_rows;
+  d.row_shift = 0;
   if (s.layout == PCS_LAYOUT_RING && s.bytes > 0 && s.row_bytes < kBulkMinRowBytes) {
     // Rows too short for bulk copies of their own: the rows of a page lie back
     // to back, so the ring is walked by its pages, whose bytes in slot order
@@ -725,7 +762,7 @@ SecDesc make_desc(const pcs_section& s, uint8_t* payload, uint32_t ring_start) {
   d.n_chunks = n_chunks_of(s.bytes);
   const uintptr_t a = reinterpret_cast<uintptr_t>(s.base);
   d.align = (a & 15u) == 0 ? 16u : ((a & 3u) == 0 ? 4u : 1u);
-  return d;
+  d.sess = sess;
 }
 
 // Device allocations known to one call, as [lo, hi) address ranges, and the
@@ -824,7 +861,7 @@ bool bulk_eligible(const pcs_ctx* c, const SecDesc& d, bool payload_device, bool
 #endif
 constexpr int kLinkSmDiv = PCS_LINK_SM_DIV;
 
-bool link_bound_call(const std::vector<SecDesc>& d, const std::vector<char>& bulk,
+bool link_bound_call(const SecVec& d, const std::vector<char>& bulk,
                      const std::vector<char>& payload_device, PtrCache& cache) {
   bool any = false;
   for (size_t i = 0; i < d.size(); ++i) {
@@ -844,20 +881,20 @@ int grid_sms(const pcs_ctx* c, const StreamPlan& P) {
 // is launch latency, which the shared-memory pipeline does not shorten.
 constexpr uint64_t kSmallCallBytes = 1ull << 20;
 
-uint64_t total_bytes(const std::vector<SecDesc>& d) {
+uint64_t total_bytes(const SecVec& d) {
   uint64_t t = 0;
   for (const auto& x : d) t += x.bytes;
   return t;
 }
 
 // The tasks of each session's streams (after plan_streams).
-void count_tasks(const std::vector<SecDesc>& d, std::vector<SessDesc>& sd) {
+void count_tasks(const SecVec& d, std::vector<SessDesc>& sd) {
   for (auto& x : sd) x.n_tasks = 0;
   for (const auto& x : d) sd[x.sess].n_tasks += x.n_tasks;
 }
 
 // Give every stream its node slots and its kernel.  bulk[i] says which.
-bool plan_streams(const pcs_ctx* c, std::vector<SecDesc>& d, const std::vector<char>& bulk,
+bool plan_streams(const pcs_ctx* c, SecVec& d, const std::vector<char>& bulk,
                   StreamPlan& P, bool allow_reduce = true) {
   uint64_t reg_chunks = 0;
   size_t n_bulk = 0;
@@ -870,7 +907,7 @@ bool plan_streams(const pcs_ctx* c, std::vector<SecDesc>& d, const std::vector<c
   P.reg_ids.reserve(d.size() - n_bulk);
   P.reg_begin.reserve(d.size() - n_bulk);
   P.glog2 = choose_group_log2(c, reg_chunks);
-  uint64_t node = 0, tb = 0, tr = 0;
+  uint64_t node = 0, tb = 0, tr = 0, max_count = 0;
   for (size_t i = 0; i < d.size(); ++i) {
     uint64_t n;
     if (bulk[i]) {
@@ -885,8 +922,9 @@ bool plan_streams(const pcs_ctx* c, std::vector<SecDesc>& d, const std::vector<c
       P.reg_begin.push_back(static_cast<uint32_t>(tr));
       tr += n;
     }
-    d[i].task_begin = static_cast<uint32_t>(node);
-    d[i].n_tasks = static_cast<uint32_t>(n);
+    d[i].task_begin = d[i].fin_begin = static_cast<uint32_t>(node);
+    d[i].n_tasks = d[i].fin_count = static_cast<uint32_t>(n);
+    max_count = std::max(max_count, n);
     node += n;
   }
   P.bulk_tasks = static_cast<uint32_t>(tb);
@@ -901,12 +939,6 @@ bool plan_streams(const pcs_ctx* c, std::vector<SecDesc>& d, const std::vector<c
   // register tree: the 64-bank step, whose latent sections have up to 512
   // tiles, 0.236 -> 0.234 ms without its two reduction launches; with the
   // earlier tree of 32-node groups a threshold of 256 was the better one).
-  for (auto& x : d) {
-    x.fin_begin = x.task_begin;
-    x.fin_count = x.n_tasks;
-  }
-  uint64_t max_count = 0;
-  for (const auto& x : d) max_count = std::max<uint64_t>(max_count, x.n_tasks);
   uint64_t groups = 0;
   if (allow_reduce && max_count > kFinRegNodes) {
     while (max_count > 32) {
@@ -948,7 +980,7 @@ bool plan_streams(const pcs_ctx* c, std::vector<SecDesc>& d, const std::vector<c
 // kernels themselves.
 // ---------------------------------------------------------------------------
 
-std::string check_streams(const std::vector<SecDesc>& d, const std::vector<char>& bulk,
+std::string check_streams(const SecVec& d, const std::vector<char>& bulk,
                           const StreamPlan& P) {
   char msg[256];
   auto bad = [&](const char* fmt, auto... a) {
@@ -1025,7 +1057,7 @@ std::string check_streams(const std::vector<SecDesc>& d, const std::vector<char>
 // Records of a checkpoint or restore: sessions cover the streams in order,
 // record s lies in its block [block[s].first, block[s].second), each payload
 // inside its record.
-std::string check_sessions(const std::vector<SecDesc>& d, const std::vector<SessDesc>& sd,
+std::string check_sessions(const SecVec& d, const std::vector<SessDesc>& sd,
                            const std::vector<std::pair<const uint8_t*, const uint8_t*>>& block) {
   char msg[256];
   uint32_t next = 0;
@@ -1086,12 +1118,12 @@ ListLayout list_layout(const StreamPlan& P, uint64_t base) {
   return L;
 }
 
-template <class T>
-void put(uint8_t* plan, uint64_t off, const std::vector<T>& v) {
-  if (!v.empty()) std::memcpy(plan + off, v.data(), v.size() * sizeof(T));
+template <class V>
+void put(uint8_t* plan, uint64_t off, const V& v) {
+  if (!v.empty()) std::memcpy(plan + off, v.data(), v.size() * sizeof(v[0]));
 }
-template <class T>
-void put(std::vector<uint8_t>& plan, uint64_t off, const std::vector<T>& v) {
+template <class V>
+void put(std::vector<uint8_t>& plan, uint64_t off, const V& v) {
   put(plan.data(), off, v);
 }
 
@@ -1139,7 +1171,7 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   if (n < 0 || (n > 0 && !bufs)) return fail(PCS_E_INVAL, "bad buffer list");
   if (n == 0) return PCS_OK;
-  std::vector<SecDesc> d(n);
+  SecVec& d = sec_array(c, n);
   uint64_t chunks = 0;
   for (int i = 0; i < n; ++i) {
     if (bufs[i].bytes > 0 && !bufs[i].ptr) return fail(PCS_E_INVAL, "buffer %d: null pointer", i);
@@ -1147,7 +1179,7 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
     s.layout = PCS_LAYOUT_CONTIG;
     s.base = const_cast<void*>(bufs[i].ptr);
     s.bytes = bufs[i].bytes;
-    d[i] = make_desc(s, nullptr, 0);
+    make_desc(d[i], s, nullptr, 0, 0);
     chunks += d[i].n_chunks;
   }
   (void)chunks;
@@ -1394,11 +1426,11 @@ pcs_status build_checkpoint(pcs_ctx* c, const pcs_session* sessions, int32_t n, 
   Block* blk = nullptr;
   pcs_status st = arena_of(c, placement)->alloc(rec_off[n], stream, &blk);
   if (st) return st;
-  std::vector<SecDesc> d;
+  SecVec& d = sec_array(c, total_secs);
+  uint32_t nd = 0;  // descriptors written
   std::vector<SessDesc> sd(n);
   auto ent_shared = std::make_shared<std::vector<Entry>>();
   std::vector<Entry>& ent = *ent_shared;  // the section tables of every record
-  d.reserve(total_secs);
   ent.reserve(total_secs);
   handles->resize(n);
   for (int s = 0; s < n; ++s) {
@@ -1411,21 +1443,21 @@ pcs_status build_checkpoint(pcs_ctx* c, const pcs_session* sessions, int32_t n, 
     h->payload_start = pstart[s];
     h->session_id = S.session_id;
     h->kind = S.kind;
-    h->first = static_cast<uint32_t>(ent.size());
+    h->entries = ent.data() + ent.size();  // (reserved above: the array does not move)
     h->n_sections = static_cast<uint32_t>(S.n_sections);
     sd[s].record = rec;
     sd[s].total_bytes = h->total_bytes;
     sd[s].payload_start = pstart[s];
-    sd[s].sec_begin = static_cast<uint32_t>(d.size());
+    sd[s].sec_begin = nd;
     sd[s].n_sections = static_cast<uint32_t>(S.n_sections);
     sd[s].session_id = S.session_id;
     sd[s].kind = S.kind;
     uint64_t off = pstart[s];
     for (int i = 0; i < S.n_sections; ++i) {
       const pcs_section& x = S.sections[i];
-      d.push_back(make_desc(x, rec + off, x.ring_start));
-      d.back().sess = static_cast<uint32_t>(s);
-      Entry e{};
+      make_desc(d[nd++], x, rec + off, x.ring_start, static_cast<uint32_t>(s));
+      ent.emplace_back();
+      Entry& e = ent.back();
       e.type = x.type;
       e.dtype = x.dtype;
       e.layer = x.layer;
@@ -1436,12 +1468,11 @@ pcs_status build_checkpoint(pcs_ctx* c, const pcs_session* sessions, int32_t n, 
       e.dim0 = x.dim0;
       e.dim1 = x.dim1;
       e.aux = x.layout == PCS_LAYOUT_RING ? x.ring_start : 0;
-      ent.push_back(e);
       off = round_up(off + x.bytes, kRecordAlign);
     }
     (*handles)[s] = std::move(h);
   }
-  for (auto& h : *handles) h->tables = ent_shared;
+  blk->tables.push_back(ent_shared);
   PtrCache cache;
   std::vector<char> bulk(d.size());
   const bool small = total_bytes(d) <= kSmallCallBytes;
@@ -1490,24 +1521,29 @@ pcs_status build_checkpoint(pcs_ctx* c, const pcs_session* sessions, int32_t n, 
 pcs_status build_restore(pcs_ctx* c, pcs_snapshot* const* snaps, int32_t n,
                          const pcs_session* targets, int verify, Prepared* pr,
                          bool to_slot = false) {
-  std::vector<SecDesc> d;
   std::vector<SessDesc> sd(n);
   std::vector<char> payload_dev;
+  // Every target's section count is its snapshot's, so the descriptors number
+  // what the snapshots hold.
   uint64_t want = 0;
-  for (int s = 0; s < n; ++s) want += targets[s].n_sections > 0 ? targets[s].n_sections : 0;
-  d.reserve(std::min<uint64_t>(want, 1ull << 24));
-  payload_dev.reserve(d.capacity());
   for (int s = 0; s < n; ++s) {
     pcs_snapshot* h = check_handle(c, snaps[s]);
     if (!h) return fail(PCS_E_HANDLE, "snapshot %d: unknown handle", s);
-    const pcs_session& T = targets[s];
-    if (T.n_sections != static_cast<int32_t>(h->n_sections) || !T.sections)
+    if (targets[s].n_sections != static_cast<int32_t>(h->n_sections) || !targets[s].sections)
       return fail(PCS_E_INVAL, "session %d: target has %d sections, snapshot %zu", s,
-                  T.n_sections, h->n_sections);
+                  targets[s].n_sections, static_cast<size_t>(h->n_sections));
+    want += h->n_sections;
+  }
+  SecVec& d = sec_array(c, want);
+  uint32_t nd = 0;  // descriptors written
+  payload_dev.resize(want);
+  for (int s = 0; s < n; ++s) {
+    pcs_snapshot* h = snaps[s];
+    const pcs_session& T = targets[s];
     sd[s].record = h->record();
     sd[s].total_bytes = h->total_bytes;
     sd[s].payload_start = h->payload_start;
-    sd[s].sec_begin = static_cast<uint32_t>(d.size());
+    sd[s].sec_begin = nd;
     sd[s].n_sections = static_cast<uint32_t>(T.n_sections);
     sd[s].session_id = h->session_id;
     sd[s].kind = h->kind;
@@ -1525,9 +1561,8 @@ pcs_status build_restore(pcs_ctx* c, pcs_snapshot* const* snaps, int32_t n,
           return fail(PCS_E_INVAL, "session %d section %d: no stored ring start fits", s, i);
         rs = static_cast<uint32_t>(e.aux);
       }
-      d.push_back(make_desc(x, h->record() + e.offset, rs));
-      d.back().sess = static_cast<uint32_t>(s);
-      payload_dev.push_back(h->block->placement == PCS_PLACE_DEVICE);
+      payload_dev[nd] = h->block->placement == PCS_PLACE_DEVICE;
+      make_desc(d[nd++], x, h->record() + e.offset, rs, static_cast<uint32_t>(s));
     }
   }
   PtrCache cache;
@@ -2364,16 +2399,15 @@ pcs_status pcs_fork_many(pcs_ctx* c, pcs_snapshot* const* parents, int32_t n,
   }
   // A fork is a restore of the whole record into a contiguous target: the
   // streaming kernels copy it (no hashing), TMA-staged when both are in HBM.
-  std::vector<SecDesc> d(n);
+  SecVec& d = sec_array(c, n);
   std::vector<char> bulk(n);
-  PtrCache cache;
   uint64_t bytes = 0;
   for (int i = 0; i < n; ++i) {
     pcs_section x{};
     x.layout = PCS_LAYOUT_CONTIG;
     x.base = blk[parents[i]->block->placement]->ptr + off[i];
     x.bytes = parents[i]->total_bytes;
-    d[i] = make_desc(x, parents[i]->record(), 0);
+    make_desc(d[i], x, parents[i]->record(), 0, 0);
     bytes += x.bytes;
   }
   const bool small = bytes <= kSmallCallBytes;
@@ -2407,6 +2441,16 @@ pcs_status pcs_fork_many(pcs_ctx* c, pcs_snapshot* const* parents, int32_t n,
     if (!blk[pl]) continue;
     blk[pl]->written = done;
     blk[pl]->refs = 0;
+    // The children's tables are their parents'.
+    auto& t = blk[pl]->tables;
+    for (int i = 0; i < n; ++i) {
+      const Block* from = parents[i]->block;
+      if (from->placement != static_cast<uint32_t>(pl)) continue;
+      if (i > 0 && from == parents[i - 1]->block) continue;
+      t.insert(t.end(), from->tables.begin(), from->tables.end());
+    }
+    std::sort(t.begin(), t.end());
+    t.erase(std::unique(t.begin(), t.end()), t.end());
   }
   c->live.reserve(n);
   for (int i = 0; i < n; ++i) {
@@ -2816,7 +2860,8 @@ pcs_status pcs_snapshot_read_file(pcs_ctx* c, const char* path, uint32_t placeme
   h->kind = kind;
   for (auto& e : table) e.fp = 0;
   h->n_sections = static_cast<uint32_t>(table.size());
-  h->tables = std::make_shared<const std::vector<Entry>>(std::move(table));
+  blk->tables.push_back(std::make_shared<const std::vector<Entry>>(std::move(table)));
+  h->entries = blk->tables.back()->data();
   *out = h.release();
   c->live.insert(*out);
   return PCS_OK;
