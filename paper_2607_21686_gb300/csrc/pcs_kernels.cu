@@ -617,8 +617,9 @@ __device__ __forceinline__ void run_stream_tasks(const SecDesc* secs, const Work
 // and waits for it only before it ends (what follows them waits for both so).
 // It can start once every block ahead has passed its own wait, so whatever
 // came before the call is finished and visible by then.  Measured, whole
-// calls: planned checkpoint + restore of odd observations 14.7 -> 11.6 us, the
-// classification of buffers off and on a boundary 80.8 -> 75.6 and 90.3 -> 87.7.
+// calls: planned checkpoint + restore of 5 odd observations 14.7 -> 11.6 us, of
+// 37 29.0 -> 22.4; 36 banks with 64-wide keys, planned, 80.8 -> 75.6; the
+// classification of packed buffers 90.3 -> 87.7.
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, 2)
     k_stream(const SecDesc* __restrict__ secs, WorkList wl, int glog2,
