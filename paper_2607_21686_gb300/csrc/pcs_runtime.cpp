@@ -2022,7 +2022,7 @@ static const int kGDigitBits[kGPasses] = {11, 11, 10, 11, 11, 10};
 static const int kGDigitShift[kGPasses] = {53, 42, 32, 21, 10, 0};
 
 // The digit choice of one pass from histograms summed over all parts (the
-// device's gselect_pick, on the host).  Returns true once the threshold is
+// device's gpick_block, on the host).  Returns true once the threshold is
 // known.
 static bool host_pick(int pass, const uint64_t* counts, const uint64_t* bytes, GState* g) {
   const int bits = kGDigitBits[pass], shift = kGDigitShift[pass];
