@@ -17,7 +17,7 @@ constexpr uint32_t kHeaderBytes = 64;
 constexpr uint32_t kEntryBytes = 64;
 constexpr uint32_t kMagic = 0x31534350u;  // "PCS1"
 constexpr uint32_t kVersion = 1;
-constexpr int kMaxGroupLog2 = 5;         // at most 32 chunks per warp task
+constexpr int kMaxGroupLog2 = 5;         // static fingerprints: at most 32 chunks per warp task
 
 // Errors a kernel records (OR-ed into the context's device error word).
 constexpr uint32_t kDevErrIndex = 1u;    // a row / page id out of range
