@@ -2552,8 +2552,10 @@ __device__ __forceinline__ int gbank_tile(const GPlan& p, int lo, int hi, uint64
   return b;
 }
 
-template <bool UNIFORM>
-__global__ void __launch_bounds__(kThreads, 3) k_gfinish(GPlan p, int first_pass) {
+// BLOCKS resident per SM: three without spills, or four whose registers spill
+// (see launch_gfinish).
+template <bool UNIFORM, int BLOCKS>
+__global__ void __launch_bounds__(kThreads, BLOCKS) k_gfinish(GPlan p, int first_pass) {
   __shared__ __align__(16) uint32_t ch[kGBins];
   __shared__ unsigned long long wh[UNIFORM ? 1 : kGBins];
   __shared__ GLocal s;
@@ -4085,10 +4087,21 @@ cudaError_t launch_classify_reads(bool host, ReadPlan p, const uint64_t* addr,
 
 cudaError_t launch_gfinish(const GPlan& p, int first_pass, int sm_count, cudaStream_t stream) {
   if (p.tiles <= 0) return cudaSuccess;
-  const void* k = p.uniform ? reinterpret_cast<const void*>(k_gfinish<true>)
-                            : reinterpret_cast<const void*>(k_gfinish<false>);
-  // Every block must be resident at once: at most one wave.
-  const int cap = sm_count * resident_blocks(k);
+  // Every block must be resident at once: at most one wave, each block with as
+  // many tiles as it takes.  The build of four blocks per SM spills, and is
+  // taken only where its wider wave saves every block a tile.  Both measured
+  // (whole calls, 64-wide keys, three / four blocks per SM): 1.86 M entries, one
+  // tile each 75.5 / 75.8 us; 1.95 M, two against one 85.6 / 80.8; 2.4 M 95.3 /
+  // 91.4; 2.6 M, two each 100.4 / 103.0; 3.7 M 121.8 / 128.6; 4.4 M, three
+  // against two 145.7 / 143.9.
+  const void* k3 = p.uniform ? reinterpret_cast<const void*>(k_gfinish<true, 3>)
+                             : reinterpret_cast<const void*>(k_gfinish<false, 3>);
+  const void* k4 = p.uniform ? reinterpret_cast<const void*>(k_gfinish<true, 4>)
+                             : reinterpret_cast<const void*>(k_gfinish<false, 4>);
+  const int cap3 = sm_count * resident_blocks(k3), cap4 = sm_count * resident_blocks(k4);
+  const bool wide = (p.tiles + cap4 - 1) / cap4 < (p.tiles + cap3 - 1) / cap3;
+  const void* k = wide ? k4 : k3;
+  const int cap = wide ? cap4 : cap3;
   const int grid = p.tiles < cap ? p.tiles : cap;
   GPlan a = p;
   int fp = first_pass;

@@ -263,3 +263,30 @@ def test_global_threshold_of_small_populations(ctx, dev, entries, n_banks, kind)
         assert off.cpu().tolist() == woff.tolist(), budget
         assert kept.cpu().tolist()[:woff[-1]] == want.tolist(), budget
     ctx.sync()
+
+
+# The cooperative global threshold at the sizes where its launch shape changes on
+# 152 SMs: 456 and 608 tiles of 4,096 entries fill three and four blocks per SM
+# (one tile more: two tiles a block), 912 and 1,216 their second rounds.
+@pytest.mark.parametrize("entries", [456 * 4096, 456 * 4096 + 1, 608 * 4096, 608 * 4096 + 1,
+                                     912 * 4096 + 1, 1216 * 4096 + 5])
+@pytest.mark.parametrize("kind", ["uniform", "mixed"])
+def test_global_threshold_at_launch_shape_edges(ctx, dev, entries, kind):
+    rnd = np.random.default_rng(entries)
+    sizes = np.diff(np.concatenate([[0], np.sort(rnd.integers(0, entries, 8)), [entries]])).tolist()
+    eb = [48] * 9 if kind == "uniform" else rnd.integers(1, 5000, 9).tolist()
+    gen = torch.Generator(device=dev).manual_seed(entries)
+    keys = torch.randn(entries, 8, generator=gen, device=dev).half()
+    q = torch.randn(8, generator=gen, device=dev).half()
+    cuts = np.cumsum([0] + sizes)
+    banks = ctx.banks_array([keys[a:b] for a, b in zip(cuts[:-1], cuts[1:])], [q] * 9, eb)
+    scores = torch.empty(entries, dtype=torch.float32, device=dev)
+    total = sum(a * b for a, b in zip(sizes, eb))
+    for budget in (total * 2 // 3 + 1, total // 50):
+        kept = torch.full((entries,), -7, dtype=torch.int32, device=dev)
+        off = torch.full((10,), -7, dtype=torch.int32, device=dev)
+        ctx.prune_global(banks, 9, budget, kept, off, scores)
+        want, woff = oracle.prune_global(scores.cpu().numpy(), sizes, eb, budget)
+        assert off.cpu().tolist() == woff.tolist(), budget
+        assert np.array_equal(kept.cpu().numpy()[:woff[-1]], want), budget
+    ctx.sync()
