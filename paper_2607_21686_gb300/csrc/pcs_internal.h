@@ -118,7 +118,8 @@ constexpr uint64_t kBulkMinRowBytes = 512;
 
 // Kernel launchers (pcs_kernels.cu).  All enqueue on `stream`, return the
 // CUDA error of the launch.  `early`: the kernel may be scheduled before the
-// one ahead on the stream has finished; false right after launch_upload.
+// one ahead on the stream has finished; false right after launch_upload, whose
+// kernel lets it start before the descriptors are written.
 
 // Register kernel: warp tasks of 2^group_log2 chunks, 128-bit loads/stores.
 // `beside`: the launch just before it on the stream is the same call's
@@ -161,8 +162,8 @@ struct SmallArgs {
 };
 // host_plan: the descriptors (`bytes` of them, at most kSmallPlanMax, in
 // memory readable to kSmallPlanMax), sent with the launch; null: a.plan.
-cudaError_t launch_small(int mode, const uint8_t* host_plan, uint64_t bytes, const SmallArgs& a,
-                         int sm_count, int blocks_per_sm, cudaStream_t stream);
+cudaError_t launch_small(int mode, bool early, const uint8_t* host_plan, uint64_t bytes,
+                         const SmallArgs& a, int sm_count, int blocks_per_sm, cudaStream_t stream);
 
 // One level of the node reduction of stream i: count nodes at src, reduced
 // by aligned groups of 32 to ceil(count / 32) nodes at dst.

@@ -94,9 +94,12 @@ __device__ __forceinline__ void prefetch_l1(const void* p) {
 // before it on the stream is still finishing.  Each calls this before it
 // touches anything another kernel may write: wait until that kernel has
 // completed and its writes are visible, then let the next kernel be
-// scheduled.  Before this point a kernel reads only what the host wrote
-// before the launch (work lists and section, session and bank
-// descriptors), which no kernel writes.
+// scheduled.  Before this point a kernel reads only the call's descriptors
+// (work lists, sections, sessions and banks): kernel parameters, words that a
+// copy put into the workspace, or words that k_upload writes there.  k_upload
+// releases its dependents before it writes, so the call's first kernel after
+// it is launched without that attribute and starts when the words are there;
+// the later ones start no sooner than the first has.
 __device__ __forceinline__ void grid_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -1565,9 +1568,11 @@ __global__ void __launch_bounds__(kThreads)
 //
 // BYTES > 0: the call's descriptors travel as a kernel parameter of that size
 // (`blob`; launch_small picks the smallest that holds them), else they are at
-// a.plan in the workspace, where a copy engine put them ahead of the launch:
-// the copy, and the hand-over from copy engine to kernel, cost a call
-// more than its kernel.  Measured, checkpoint + verified restore + delete of
+// a.plan in the workspace: a plain call whose descriptors are too many for a
+// parameter sends them there ahead of the launch (then not an early one), a
+// prepared call keeps them there.  Sending them ahead, and the hand-over to
+// the kernel, cost a call more than its kernel.  Measured (sent by a copy
+// engine -> as a parameter), checkpoint + verified restore + delete of
 // one session of 196,608 bytes 31.4 -> 20.1 us, of 34 small ones 31.7 -> 25.8,
 // of 64 (27 KB of descriptors) 36.2 -> 31.5; fingerprints of 8 buffers 11.1 -> 5.8.
 template <int BYTES>
@@ -3770,7 +3775,7 @@ cudaError_t launch_bulk(int mode, bool shift, bool early, const SecDesc* secs, W
 }
 
 template <int MODE, int BYTES>
-static cudaError_t launch_small_mode(const uint8_t* host_plan, SmallArgs a, int blocks,
+static cudaError_t launch_small_mode(bool early, const uint8_t* host_plan, SmallArgs a, int blocks,
                                      cudaStream_t stream) {
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -3780,7 +3785,7 @@ static cudaError_t launch_small_mode(const uint8_t* host_plan, SmallArgs a, int 
   cfg.blockDim = dim3(kThreads);
   cfg.stream = stream;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   static const PlanBlob<0> none{};
   const void* blob = BYTES > 0 ? static_cast<const void*>(host_plan) : static_cast<const void*>(&none);
   void* args[] = {const_cast<void*>(blob), &a};
@@ -3788,25 +3793,26 @@ static cudaError_t launch_small_mode(const uint8_t* host_plan, SmallArgs a, int 
 }
 
 template <int MODE>
-static cudaError_t launch_small_size(const uint8_t* host_plan, uint64_t bytes, const SmallArgs& a,
-                                     int blocks, cudaStream_t stream) {
+static cudaError_t launch_small_size(bool early, const uint8_t* host_plan, uint64_t bytes,
+                                     const SmallArgs& a, int blocks, cudaStream_t stream) {
   static_assert(kSmallPlanMax == 31744, "the largest parameter below");
-  if (!host_plan) return launch_small_mode<MODE, 0>(host_plan, a, blocks, stream);
-  if (bytes <= 1008) return launch_small_mode<MODE, 1008>(host_plan, a, blocks, stream);
-  if (bytes <= 7936) return launch_small_mode<MODE, 7936>(host_plan, a, blocks, stream);
-  return launch_small_mode<MODE, 31744>(host_plan, a, blocks, stream);
+  if (!host_plan) return launch_small_mode<MODE, 0>(early, host_plan, a, blocks, stream);
+  if (bytes <= 1008) return launch_small_mode<MODE, 1008>(early, host_plan, a, blocks, stream);
+  if (bytes <= 7936) return launch_small_mode<MODE, 7936>(early, host_plan, a, blocks, stream);
+  return launch_small_mode<MODE, 31744>(early, host_plan, a, blocks, stream);
 }
 
-cudaError_t launch_small(int mode, const uint8_t* host_plan, uint64_t bytes, const SmallArgs& a,
-                         int sm_count, int blocks_per_sm, cudaStream_t stream) {
+cudaError_t launch_small(int mode, bool early, const uint8_t* host_plan, uint64_t bytes,
+                         const SmallArgs& a, int sm_count, int blocks_per_sm, cudaStream_t stream) {
   if (a.n_tasks == 0 || (host_plan && bytes > kSmallPlanMax)) return cudaErrorInvalidValue;
   const uint64_t want = (static_cast<uint64_t>(a.n_tasks) + kWarps - 1) / kWarps;
   const uint64_t cap = static_cast<uint64_t>(sm_count) * blocks_per_sm;
   const int blocks = static_cast<int>(want < cap ? want : cap);
   switch (mode) {
-    case kModeHash: return launch_small_size<kModeHash>(host_plan, bytes, a, blocks, stream);
-    case kModePack: return launch_small_size<kModePack>(host_plan, bytes, a, blocks, stream);
-    case kModeRestoreV: return launch_small_size<kModeRestoreV>(host_plan, bytes, a, blocks, stream);
+    case kModeHash: return launch_small_size<kModeHash>(early, host_plan, bytes, a, blocks, stream);
+    case kModePack: return launch_small_size<kModePack>(early, host_plan, bytes, a, blocks, stream);
+    case kModeRestoreV:
+      return launch_small_size<kModeRestoreV>(early, host_plan, bytes, a, blocks, stream);
     default: return cudaErrorInvalidValue;
   }
 }

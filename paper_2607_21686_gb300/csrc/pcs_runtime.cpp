@@ -606,10 +606,13 @@ uint8_t* plan_dst(pcs_ctx* c, uint64_t bytes, std::vector<uint8_t>& fallback) {
 
 // Send descriptors written where plan_dst said into the workspace: by a kernel
 // where they are in a pinned slot and at most kUploadMax, else by a copy.
-// c->uploaded says which, for the launch that follows.  One launch is not
-// worth a kernel ahead of it (`by_kernel` false): it costs the host about a
-// microsecond more than the copy, which bounds such calls (a log against 150
-// buffers 11.5 -> 12.2 us).
+// c->uploaded says which, for the launch that follows: it must not be early.
+// One launch that the host bounds is not worth a kernel ahead of it
+// (`by_kernel` false): it costs the host about a microsecond more than the copy
+// (a log against 150 buffers 11.5 -> 12.2 us).  A small call with more
+// descriptors than travel with its launch is not such a one (checkpoint +
+// verified restore + delete, copied / uploaded: 64 sessions of 3 sections 33.2 /
+// 32.8 us, of 8 48.7 / 47.3, of 32 123 / 120, one of 300 100.9 / 99.4).
 cudaError_t plan_send(pcs_ctx* c, uint8_t* ws, uint64_t bytes,
                       const std::vector<uint8_t>& fallback, cudaStream_t stream,
                       bool by_kernel = true) {
@@ -1207,6 +1210,7 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
   c->plan.resize(sent ? kSmallPlanMax : L.nodes);
   put(c->plan, L.secs, d);
   put_lists(c->plan, P, LL);
+  c->uploaded = false;
   if (!sent) PCS_CUDA(plan_copy(c, ws, L.nodes, stream));
   auto* dsecs = reinterpret_cast<const SecDesc*>(ws + L.secs);
   auto* nodes = reinterpret_cast<uint64_t*>(ws + L.nodes);
@@ -1216,8 +1220,8 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
     a.fp_before = fp_before;
     a.flags = flags;
     LaunchScope ls(c, kKStreamHash, stream);
-    PCS_CUDA(launch_small(kModeHash, sent ? c->plan.data() : nullptr, LL.end, a, c->sm_count,
-                          c->stream_bps, stream));
+    PCS_CUDA(launch_small(kModeHash, !c->uploaded, sent ? c->plan.data() : nullptr, LL.end, a,
+                          c->sm_count, c->stream_bps, stream));
     return ws_release(c, stream);
   }
   PCS_CUDA(launch_streams(c, kModeHash, dsecs, P, LL, ws, nodes, stream, !c->uploaded));
@@ -1354,7 +1358,8 @@ uint8_t* plan_ws(const pcs_plan* p) { return p->dev + kWsHeader; }
 uint32_t* plan_words(const pcs_plan* p) { return reinterpret_cast<uint32_t*>(p->dev); }
 
 // Launch a prepared call whose descriptors are at `ws` (nodes after them);
-// `words` are the call's header words (ticket of the fused kernel).
+// `words` are the call's header words (ticket of the fused kernel).  `early`:
+// its first kernel's, false after an upload (see launch_upload).
 cudaError_t launch_prepared(pcs_ctx* c, const Prepared& pr, uint8_t* ws, uint32_t* words,
                             cudaStream_t stream, bool early = true) {
   const auto* dsecs = reinterpret_cast<const SecDesc*>(ws + pr.L.secs);
@@ -1373,7 +1378,8 @@ cudaError_t launch_prepared(pcs_ctx* c, const Prepared& pr, uint8_t* ws, uint32_
     const auto* dent = reinterpret_cast<const Entry*>(ws + pr.L.entries);
     if (pr.fused) {
       LaunchScope ls(c, kKStreamPack, stream);
-      return launch_small(kModePack, sent, pr.LL.end, args(), c->sm_count, c->stream_bps, stream);
+      return launch_small(kModePack, early, sent, pr.LL.end, args(), c->sm_count, c->stream_bps,
+                          stream);
     }
     cudaError_t e = launch_streams(c, kModePack, dsecs, pr.P, pr.LL, ws, nodes, stream, early);
     if (e != cudaSuccess) return e;
@@ -1386,7 +1392,8 @@ cudaError_t launch_prepared(pcs_ctx* c, const Prepared& pr, uint8_t* ws, uint32_
     LaunchScope ls(c, kKStreamRestoreV, stream);
     SmallArgs a = args();
     a.bad = bad;
-    return launch_small(kModeRestoreV, sent, pr.LL.end, a, c->sm_count, c->stream_bps, stream);
+    return launch_small(kModeRestoreV, early, sent, pr.LL.end, a, c->sm_count, c->stream_bps,
+                        stream);
   }
   cudaError_t e = launch_streams(c, pr.verify ? kModeRestoreV : kModeRestore, dsecs, pr.P, pr.LL,
                                  ws, pr.verify ? nodes : nullptr, stream, early);

@@ -4,8 +4,8 @@ chain.
 
 The library launches its kernels so that one may be scheduled while the
 kernel ahead of it on the stream drains, and lets a kernel read its own
-host-written descriptors before it waits for that kernel.  Every read of
-data a kernel wrote must still come after that kernel: the checkpoint of
+kernel ahead of it on the stream drains, and lets a kernel read the call's
+descriptors before it waits for that kernel.  Every read of
 buffers a restore has just written, the fork of records a checkpoint has just
 finalised, a prune whose queries a restore has just written, and the pack of
 bank rows gathered by the indices the top-k has just chosen.  The results are
@@ -83,3 +83,45 @@ def test_dependent_calls_on_one_stream(ctx, dev, it):
         eo += x
     for x in snaps_a + snaps_b + kids + snaps_k + [qsnap]:
         ctx.delete(x)
+
+
+# Small calls whose descriptors are more than a launch carries, of session sets
+# that differ in number, order and buffers, in turn with no host wait: each call
+# works on its own descriptors, not on those the call before left in the workspace.
+@pytest.mark.parametrize("shapes", [[(64, 3), (1, 300), (40, 8)], [(3, 100), (64, 32), (53, 5)]])
+def test_small_calls_of_different_sessions_in_turn(ctx, dev, shapes):
+    rnd = np.random.default_rng(len(shapes[0]) + shapes[0][0])
+    sets = []
+    for k, (n, secs) in enumerate(shapes):
+        size = rnd.integers(1, (1 << 20) // (n * secs), (n, secs)).reshape(-1)
+        at = np.cumsum(np.concatenate([[16], size + 7 + k])).tolist()  # guard bytes between them
+        spans = list(zip(at, size.tolist()))
+        src = torch.from_numpy(rnd.integers(0, 256, at[-1] + 16, dtype=np.uint8))
+        order = rnd.permutation(len(spans)).tolist()  # the sections of a session lie anywhere
+        mk = lambda t, n=n, secs=secs, spans=spans, order=order: [
+            pcs.Session(s, 9, [pcs.contig_section(1 + i, t[o:o + b]) for i, (o, b) in
+                               enumerate(spans[j] for j in order[s * secs:(s + 1) * secs])],
+                        keep=[t]) for s in range(n)]
+        used = torch.zeros(len(src), dtype=torch.bool)
+        for o, b in spans:
+            used[o:o + b] = True
+        fps = [oracle.fingerprint(src[o:o + b].numpy()) for o, b in (spans[j] for j in order)]
+        sets.append((mk, src, src.to(dev), torch.empty_like(src, device=dev), used, fps, secs))
+    busy = torch.randn(4096, 4096, device=dev)
+    for rep in range(4):
+        for s in sets:
+            s[3].fill_(0x5A)
+        torch.mm(busy, busy)  # the calls pile up behind it
+        snaps = []
+        for mk, _, src, dst, _, _, _ in sets + sets[::-1]:
+            snaps.append(ctx.checkpoint(mk(src)))
+            ctx.restore(snaps[-1], mk(dst), verify=2)
+        ctx.sync()
+        for _, host, _, dst, used, _, _ in sets:
+            got = dst.cpu()
+            assert torch.equal(got[used], host[used])
+            assert bool((got[~used] == 0x5A).all())
+        for (_, _, _, _, _, fps, secs), sn in zip(sets + sets[::-1], snaps):
+            assert [ctx.section(x, i).fp for x in sn for i in range(secs)] == fps
+            for x in sn:
+                ctx.delete(x)
