@@ -18,6 +18,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <unordered_map>
 #include <map>
 #include <memory>
@@ -149,6 +150,12 @@ struct Slab {
 // (one count per block, not per snapshot).
 using Tables = std::shared_ptr<const std::vector<Entry>>;
 
+struct TablesBefore {
+  bool operator()(const Tables& a, const std::vector<Entry>* b) const {
+    return std::less<const std::vector<Entry>*>()(a.get(), b);
+  }
+};
+
 struct Block {
   Slab* slab = nullptr;
   uint64_t off = 0;
@@ -156,7 +163,7 @@ struct Block {
   uint8_t* ptr = nullptr;
   uint32_t placement = PCS_PLACE_DEVICE;
   int refs = 0;
-  std::vector<Tables> tables;                 // section tables of its snapshots
+  std::vector<Tables> tables;                 // section tables of its snapshots, by address
   Ev written;                                 // completion of the write
   std::map<cudaStream_t, Ev> uses;            // latest use per stream
 };
@@ -342,6 +349,7 @@ struct pcs_snapshot {
   uint32_t kind = 0;
   // Host copy of the section table (fp = 0): n_sections entries, in an array
   // that the block keeps (shared by the snapshots of one call and their forks).
+  const std::vector<Entry>* tables = nullptr;
   const Entry* entries = nullptr;
   uint32_t n_sections = 0;
   const Entry* table() const { return entries; }
@@ -1450,6 +1458,7 @@ pcs_status build_checkpoint(pcs_ctx* c, const pcs_session* sessions, int32_t n, 
     h->payload_start = pstart[s];
     h->session_id = S.session_id;
     h->kind = S.kind;
+    h->tables = &ent;
     h->entries = ent.data() + ent.size();  // (reserved above: the array does not move)
     h->n_sections = static_cast<uint32_t>(S.n_sections);
     sd[s].record = rec;
@@ -2448,13 +2457,15 @@ pcs_status pcs_fork_many(pcs_ctx* c, pcs_snapshot* const* parents, int32_t n,
     if (!blk[pl]) continue;
     blk[pl]->written = done;
     blk[pl]->refs = 0;
-    // The children's tables are their parents'.
+    // The tables the children point into, not all that their parents' blocks
+    // hold: in a loop of forks those would add up.
     auto& t = blk[pl]->tables;
     for (int i = 0; i < n; ++i) {
       const Block* from = parents[i]->block;
       if (from->placement != static_cast<uint32_t>(pl)) continue;
-      if (i > 0 && from == parents[i - 1]->block) continue;
-      t.insert(t.end(), from->tables.begin(), from->tables.end());
+      if (!t.empty() && t.back().get() == parents[i]->tables) continue;
+      t.push_back(*std::lower_bound(from->tables.begin(), from->tables.end(), parents[i]->tables,
+                                    TablesBefore()));
     }
     std::sort(t.begin(), t.end());
     t.erase(std::unique(t.begin(), t.end()), t.end());
@@ -2868,7 +2879,8 @@ pcs_status pcs_snapshot_read_file(pcs_ctx* c, const char* path, uint32_t placeme
   for (auto& e : table) e.fp = 0;
   h->n_sections = static_cast<uint32_t>(table.size());
   blk->tables.push_back(std::make_shared<const std::vector<Entry>>(std::move(table)));
-  h->entries = blk->tables.back()->data();
+  h->tables = blk->tables.back().get();
+  h->entries = h->tables->data();
   *out = h.release();
   c->live.insert(*out);
   return PCS_OK;

@@ -251,8 +251,70 @@ static void check_upload_order() {
   NEED(pcs_destroy(c) == PCS_OK);
 }
 
+// A forked child keeps its own section table and no other: a block's tables are
+// those its snapshots point into, each once, however its parents were made.
+static void check_fork_tables() {
+  pcs_ctx* c = nullptr;
+  NEED(pcs_create(0, &c) == PCS_OK);
+  // One old session forked again and again together with a new one, the
+  // parents and the new one's child dropped: the number does not grow.
+  Sessions A(1, 3, 1000), B(1, 2, 500), M(40, 2, 300);
+  pcs_snapshot* old = nullptr;
+  NEED(pcs_checkpoint(c, A.s.data(), 1, PCS_PLACE_DEVICE, &old, nullptr) == PCS_OK);
+  for (int it = 0; it < 50; ++it) {
+    pcs_snapshot *fresh = nullptr, *kid[2];
+    NEED(pcs_checkpoint(c, B.s.data(), 1, PCS_PLACE_DEVICE, &fresh, nullptr) == PCS_OK);
+    pcs_snapshot* par[2] = {old, fresh};
+    NEED(pcs_fork_many(c, par, 2, kid, nullptr) == PCS_OK);
+    std::vector<pcs_snapshot*> gone = {old, fresh, kid[1]};
+    drop(c, gone);
+    old = kid[0];
+    NEED(old->block->tables.size() <= 2);
+  }
+  NEED(old->n_sections == 3 && old->table()[2].bytes == 1000);
+  // Parents of several calls and both placements, in any order and more than once.
+  std::vector<pcs_snapshot*> dev(40), host(40), one(40), par, kid(400);
+  NEED(pcs_checkpoint(c, M.s.data(), 40, PCS_PLACE_DEVICE, dev.data(), nullptr) == PCS_OK);
+  NEED(pcs_checkpoint(c, M.s.data(), 40, PCS_PLACE_PINNED_HOST, host.data(), nullptr) == PCS_OK);
+  for (int i = 0; i < 40; ++i)
+    NEED(pcs_checkpoint(c, &M.s[i], 1, PCS_PLACE_DEVICE, &one[i], nullptr) == PCS_OK);
+  uint64_t rnd = 1;
+  for (int i = 0; i < 400; ++i) {
+    rnd = rnd * 6364136223846793005ull + 1442695040888963407ull;
+    const uint32_t r = static_cast<uint32_t>(rnd >> 33);
+    par.push_back((r & 1 ? dev : r & 2 ? host : one)[(r >> 2) % 40]);
+  }
+  NEED(pcs_fork_many(c, par.data(), 400, kid.data(), nullptr) == PCS_OK);
+  std::vector<uint32_t> ids;
+  for (auto* p : par) ids.push_back(p->session_id);
+  drop(c, dev);
+  drop(c, host);
+  drop(c, one);
+  for (int i = 0; i < 400; ++i) {
+    std::set<const void*> have;
+    size_t holds = 0;
+    for (auto& t : kid[i]->block->tables) {
+      NEED(have.insert(t.get()).second);
+      const Entry* e = t->data();
+      holds += kid[i]->entries >= e && kid[i]->entries + 2 <= e + t->size();
+    }
+    NEED(holds == 1);
+    std::set<const void*> used;
+    for (auto* k : kid)
+      if (k->block == kid[i]->block)
+        for (auto& t : k->block->tables)
+          if (k->entries >= t->data() && k->entries < t->data() + t->size()) used.insert(t.get());
+    NEED(used == have);
+    NEED(kid[i]->session_id == ids[i] && kid[i]->table()[1].bytes == 300);
+  }
+  drop(c, kid);
+  NEED(pcs_delete(c, old) == PCS_OK);
+  NEED(pcs_destroy(c) == PCS_OK);
+}
+
 int main(int argc, char** argv) {
-  const std::map<std::string, void (*)()> checks = {{"upload_order", check_upload_order}};
+  const std::map<std::string, void (*)()> checks = {{"upload_order", check_upload_order},
+                                                    {"fork_tables", check_fork_tables}};
   auto it = checks.find(argc > 1 ? argv[1] : "");
   if (it == checks.end()) return 2;
   it->second();

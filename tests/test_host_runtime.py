@@ -5,6 +5,8 @@ built here with g++).
 upload_order  descriptors written by k_upload are complete before the first
               kernel of the call may read them, over calls of every kind and
               around the sizes where descriptors stop travelling with a launch
+fork_tables   a block made by forks keeps the section tables of its own
+              snapshots only, in a loop of forks too
 """
 import os
 import shutil
@@ -30,7 +32,7 @@ def checker(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("check", ["upload_order"])
+@pytest.mark.parametrize("check", ["upload_order", "fork_tables"])
 def test_runtime(checker, check):
     out = subprocess.run([checker, check], capture_output=True, text=True, timeout=120)
     assert out.returncode == 0 and out.stdout.strip() == "ok", out.stdout + out.stderr
