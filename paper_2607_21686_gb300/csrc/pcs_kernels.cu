@@ -4040,10 +4040,23 @@ static cudaError_t launch_reads(const ReadPlan& p, const uint64_t* addr, const u
                                 int64_t m, uint8_t* flags, unsigned threads, size_t smem,
                                 int sm_count, cudaStream_t stream) {
   if (smem > 48 * 1024) {  // long bitmaps or many staged buffers
-    cudaError_t e = cudaFuncSetAttribute(k_classify_reads<STAGED, TABLE, N>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
+    // The limit is the kernel's on its device, whichever context asks: set
+    // once, to all that a block can have, so that no other thread's call can
+    // lower it between here and the launch.  limit[d]: 0 not set yet.
+    static std::atomic<int> limit[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
+    int most = limit[dev & 63].load(std::memory_order_acquire);
+    if (most == 0) {
+      e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_classify_reads<STAGED, TABLE, N>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+      if (e != cudaSuccess) return e;
+      limit[dev & 63].store(most, std::memory_order_release);
+    }
+    if (smem > static_cast<size_t>(most)) return cudaErrorInvalidValue;
   }
   const uint64_t want = (static_cast<uint64_t>(m) + threads - 1) / threads;
   // One resident wave: 2,048 threads per SM (32 registers), fewer where the

@@ -155,3 +155,39 @@ def test_discovery_on_a_gpu_model(ctx, dev):
     assert dict(zip(_Model.names, state)) == {"obs": 1, "rng": 1, "cache": 0, "frame": 0,
                                                "a": 1, "b": 0}
     ctx.delete(snap)
+
+
+def test_classify_reads_on_two_threads(dev):
+    # Two threads, each with its own context and stream: a log against 4,096 and
+    # one against 3,300 buffers ask for different amounts of shared memory over
+    # 48 KiB, a limit that a kernel has once per device.
+    import threading
+    space = torch.zeros(1 << 20, dtype=torch.uint8, device=dev)
+    base, errs = space.data_ptr(), []
+    start = threading.Barrier(2)
+
+    def worker(n):
+        try:
+            with pcs.Context(0) as c:
+                s = torch.cuda.Stream(device=dev)
+                bufs = pcs.BufArray([space[200 * i:200 * i + 150] for i in range(n)])
+                hit = np.arange(0, n, 7)
+                addr = torch.from_numpy(base + 200 * hit + 149).to(dev)
+                nb = torch.full((len(hit),), 3, dtype=torch.int64, device=dev)
+                flags = torch.zeros(n, dtype=torch.uint8, device=dev)
+                torch.cuda.synchronize()
+                start.wait(60)
+                for _ in range(3000):
+                    c.classify_reads(bufs, addr, nb, flags, stream=s)
+                c.sync(s)
+                got = flags.cpu().numpy()
+                assert got.sum() == len(hit) and got[hit].all()
+        except BaseException as e:  # surfaced below
+            errs.append(e)
+
+    ts = [threading.Thread(target=worker, args=(n,)) for n in (4096, 3300)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join(300)
+    assert not errs, errs
