@@ -1219,6 +1219,7 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
   put(c->plan, L.secs, d);
   put_lists(c->plan, P, LL);
   c->uploaded = false;
+  c->plan_slot_used = -1;  // (it may be a failed call's)
   if (!sent) PCS_CUDA(plan_copy(c, ws, L.nodes, stream));
   auto* dsecs = reinterpret_cast<const SecDesc*>(ws + L.secs);
   auto* nodes = reinterpret_cast<uint64_t*>(ws + L.nodes);

@@ -312,9 +312,61 @@ static void check_fork_tables() {
   NEED(pcs_destroy(c) == PCS_OK);
 }
 
+// A call that fails after its descriptors were sent from a pinned slot leaves
+// that slot held, since what it enqueued may still read it.  No later call may
+// give it back, whichever way that call's own descriptors travel.
+static void check_failed_call() {
+  Sessions big(8, 1, 1 << 20), few(2, 2, 100);
+  std::vector<pcs_buf> bufs(200);
+  for (int j = 0; j < 200; ++j) bufs[j] = {mem(64 * j), 60};
+  auto* w = reinterpret_cast<uint64_t*>(mem(1 << 20));
+  auto* f = reinterpret_cast<float*>(mem(1 << 20));
+  auto* ix = reinterpret_cast<int32_t*>(mem(8 << 20));
+  std::vector<pcs_bank> b(2);
+  for (auto& x : b) {
+    x = pcs_bank{};
+    x.keys = x.query = mem(0);
+    x.n_entries = 9;
+    x.key_dim = 64;
+    x.key_dtype = PCS_DT_F16;
+    x.entry_bytes = 100;
+  }
+  pcs_prune_params p{};
+  p.rule = PCS_K_FIXED;
+  p.k_max = 2;
+  cudaStream_t s2 = reinterpret_cast<cudaStream_t>(8);
+  for (int after = 0; after < 8; ++after) {
+    pcs_ctx* c = nullptr;
+    NEED(pcs_create(0, &c) == PCS_OK);
+    std::vector<pcs_snapshot*> h(8), k(2);
+    g_fail_at = "finalize";
+    NEED(pcs_checkpoint(c, big.s.data(), 8, PCS_PLACE_DEVICE, h.data(), nullptr) == PCS_E_CUDA);
+    g_fail_at.clear();
+    NEED(c->plan_slot_busy[0] && !c->plan_slot_busy[0]->done());
+    switch (after) {
+      case 0: NEED(pcs_fingerprint(c, bufs.data(), 3, w, s2) == PCS_OK); break;
+      case 1: NEED(pcs_fingerprint(c, bufs.data(), 200, w, s2) == PCS_OK); break;
+      case 2: NEED(pcs_mismatch(c, bufs.data(), bufs.data(), 3, w, s2) == PCS_OK); break;
+      case 3: NEED(pcs_classify_reads(c, bufs.data(), 3, w, w, 5, mem(0), s2) == PCS_OK); break;
+      case 4: NEED(pcs_prune(c, b.data(), 2, &p, nullptr, ix, ix, s2) == PCS_OK); break;
+      case 5: NEED(pcs_prune_global(c, b.data(), 2, 500, nullptr, ix, ix, s2) == PCS_OK); break;
+      case 6: NEED(pcs_prune(c, b.data(), 2, &p, f, ix, ix, s2) == PCS_OK); break;
+      default:
+        NEED(pcs_checkpoint(c, few.s.data(), 2, PCS_PLACE_DEVICE, k.data(), s2) == PCS_OK);
+        NEED(pcs_restore(c, k.data(), 2, few.s.data(), 2, s2) == PCS_OK);
+    }
+    if (c->plan_slot_busy[0]->done()) {
+      std::printf("call %d gave back the slot of a failed one\n", after);
+      std::exit(1);
+    }
+    NEED(pcs_destroy(c) == PCS_OK);
+  }
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, void (*)()> checks = {{"upload_order", check_upload_order},
-                                                    {"fork_tables", check_fork_tables}};
+                                                    {"fork_tables", check_fork_tables},
+                                                    {"failed_call", check_failed_call}};
   auto it = checks.find(argc > 1 ? argv[1] : "");
   if (it == checks.end()) return 2;
   it->second();

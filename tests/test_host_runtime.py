@@ -7,6 +7,8 @@ upload_order  descriptors written by k_upload are complete before the first
               around the sizes where descriptors stop travelling with a launch
 fork_tables   a block made by forks keeps the section tables of its own
               snapshots only, in a loop of forks too
+failed_call   the pinned slot of a call that failed half-way is not given back
+              by a later call
 """
 import os
 import shutil
@@ -32,7 +34,7 @@ def checker(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("check", ["upload_order", "fork_tables"])
+@pytest.mark.parametrize("check", ["upload_order", "fork_tables", "failed_call"])
 def test_runtime(checker, check):
     out = subprocess.run([checker, check], capture_output=True, text=True, timeout=120)
     assert out.returncode == 0 and out.stdout.strip() == "ok", out.stdout + out.stderr
