@@ -2,12 +2,13 @@
 
 pcs_prune_global through the C ABI against the oracle on the same seeded
 banks: scores bit-equal to the oracle's fixed-order fp32 score, kept sets and
-bank offsets identical, across several 4096-entry tiles with a ragged tail,
-with uniform and mixed entry sizes (the two select paths), empty banks at
-either end and in the middle, exact ties across banks, mixed key types and
-keys wider than 1024 (the first digit binned after the score kernel), and
-budgets that keep nothing, one entry, a fraction, all but one, and all.  The same population
-split into two parts (two threads, two contexts, the histograms summed on the
+bank offsets identical, with uniform and mixed entry sizes (the two select
+paths), empty banks at either end and in the middle, exact ties across banks,
+mixed key types and keys wider than 1024, and budgets that keep nothing, one
+entry, a fraction, all but one, and all.  Populations of at most 16,384 entries
+take one block after a plain score pass; the tests at the end have more, which
+the score kernel's histogram and the cooperative select take, over several
+4096-entry tiles with a ragged tail.  The same population split into two parts (two threads, two contexts, the histograms summed on the
 host each pass, as ranks would all-reduce them) gives each part its share of
 the one-population answer.
 """
@@ -60,7 +61,7 @@ def _views(b, dev):
 
 
 def test_global_threshold_uniform_bytes(ctx, dev):
-    # ~6,000 entries: two 4096-entry tiles, the second ragged.
+    # ~6,000 entries in 40 banks.
     b = synth.banks(301, 40, 1, 300, 256, torch.float16, (8,), torch.uint8)
     keys, qs = _views(b, dev)
     E = 512 + 8
@@ -116,8 +117,7 @@ def test_global_threshold_scores_optional_and_no_entries(ctx, dev):
 
 
 def test_global_threshold_unaligned_scores(ctx, dev):
-    # A scores buffer that starts 4 bytes past a 16-byte boundary: the scans
-    # read it one float at a time.
+    # A scores buffer that starts 4 bytes past a 16-byte boundary.
     b = synth.banks(304, 9, 100, 900, 64, torch.float16, (8,), torch.uint8)
     keys, qs = _views(b, dev)
     total = sum(b.n)
@@ -152,8 +152,7 @@ def test_global_threshold_keeps_relevant_sessions(ctx, dev):
 
 @pytest.mark.parametrize("mixed_bytes", [False, True])
 def test_global_threshold_mixed_key_types(ctx, dev, mixed_bytes):
-    # fp16 and bf16 banks together (and, below, keys wider than 1024): the
-    # score kernel takes no digit pass, so the first is binned after it.
+    # fp16 and bf16 banks together (and, below, keys wider than 1024).
     g = torch.Generator().manual_seed(21)
     D = 96
     keys, qs = [], []
@@ -251,3 +250,92 @@ def test_global_threshold_one_part_equals_whole(ctx, dev):
     want, woff = oracle.prune_global(_oracle_scores(keys, qs), b.n, 300, B)
     assert koff.cpu().tolist() == woff.tolist()
     assert kept.cpu().tolist()[:woff[-1]] == want.tolist()
+
+
+# --- populations past 16,384 entries: the cooperative select ---
+
+def _large(dev, dims, dtypes, sizes, seed):
+    """Banks of `sizes` entries, key widths and types in turn, a run of zero keys
+    (score 0) and of equal ones in some of them."""
+    g = torch.Generator().manual_seed(seed)
+    keys, qs = [], []
+    for i, n in enumerate(sizes):
+        d, dt = dims[i % len(dims)], dtypes[i % len(dtypes)]
+        k = torch.randn(n, d, generator=g)
+        k[100:140] = 0
+        k[n // 2:n // 2 + 90] = k[n // 2:n // 2 + 1]
+        keys.append(k.to(dt).to(dev))
+        qs.append(torch.randn(d, generator=g).to(dt).to(dev))
+    return keys, qs
+
+
+def _bytes(kind, n):
+    return [700] * n if kind == "uniform" else np.random.default_rng(n).integers(0, 3000, n).tolist()
+
+
+H, B16 = torch.float16, torch.bfloat16
+
+
+# Every build of the score kernel that histograms (key widths at the top of each
+# shape and just past it, both types, uniform and mixed entry bytes), and the
+# calls whose first digit is binned after it (both types together, wider keys).
+@pytest.mark.parametrize("dims,dtypes", [((64,), [H]), ((64, 8), [B16]), ((72, 128), [H]), ((128,), [B16]),
+                                         ((136, 256), [H]), ((256,), [B16]), ((264, 512), [H]),
+                                         ((512,), [B16]), ((520, 768), [H]), ((768,), [B16]),
+                                         ((776, 1024), [H]), ((1024,), [B16]), ((96,), [H, B16]),
+                                         ((1032, 40), [H]), ((1536,), [B16])])
+@pytest.mark.parametrize("kind", ["uniform", "mixed"])
+def test_global_threshold_of_larger_populations(ctx, dev, dims, dtypes, kind):
+    sizes = [5000, 0, 1, 7000, 333, 4096, 640]  # 17,070: five tiles, the last ragged
+    keys, qs = _large(dev, dims, dtypes, sizes, dims[0])
+    E = _bytes(kind, len(sizes))
+    T = sum(n * e for n, e in zip(sizes, E))
+    _check(ctx, dev, keys, qs, E, [0, T // 9, T // 2, T - 1, T])
+
+
+@pytest.mark.parametrize("kind", ["uniform", "mixed"])
+@pytest.mark.parametrize("off", [1, 2, 3])
+def test_global_threshold_of_larger_populations_unaligned_scores(ctx, dev, kind, off):
+    # Scores 4, 8 and 12 bytes past a 16-byte boundary: read one float at a time.
+    sizes = [9000, 11, 8500]
+    keys, qs = _large(dev, (64,), [H], sizes, 5)
+    E, total = _bytes(kind, 3), sum(sizes)
+    banks = ctx.banks_array(keys, qs, E)
+    scores = torch.zeros(total + 4, device=dev)[off:off + total]
+    kept = torch.empty(total, dtype=torch.int32, device=dev)
+    koff = torch.empty(4, dtype=torch.int32, device=dev)
+    B = sum(n * e for n, e in zip(sizes, E)) * 2 // 5
+    ctx.prune_global(banks, 3, B, kept, koff, scores)
+    s32 = _oracle_scores(keys, qs)
+    assert np.array_equal(scores.cpu().numpy().view(np.uint32), s32.view(np.uint32))
+    want, woff = oracle.prune_global(s32, sizes, E, B)
+    assert koff.cpu().tolist() == woff.tolist()
+    assert kept.cpu().tolist()[:woff[-1]] == want.tolist()
+
+
+# Equal scores at the threshold, as many as are gathered for the last choice (512)
+# and one more, which further digit passes settle; budgets that end before, inside
+# and after them.
+@pytest.mark.parametrize("ties", [2, 511, 512, 513, 3000])
+@pytest.mark.parametrize("kind", ["uniform", "mixed"])
+def test_global_threshold_of_larger_populations_ties(ctx, dev, ties, kind):
+    sizes = [6000, 4096, 7001, 20]
+    total = sum(sizes)
+    g = torch.Generator().manual_seed(ties)
+    k = torch.randn(total, 16, generator=g).half()
+    at = torch.randperm(total, generator=g)[:ties]
+    q = torch.randn(16, generator=g).half()
+    k[at] = (0.3 * q.float() + 0.7 * torch.randn(16, generator=g)).half()
+    cuts = np.cumsum([0] + sizes)
+    keys = [k[a:b].to(dev) for a, b in zip(cuts[:-1], cuts[1:])]
+    qs = [q.to(dev)] * 4
+    E = _bytes(kind, 4)
+    s32 = _oracle_scores(keys, qs)
+    order = np.lexsort((np.arange(total), -s32))
+    cost = np.cumsum(np.repeat(E, sizes)[order])
+    tied = np.flatnonzero(s32[order] == s32[at[0]])
+    assert len(tied) == ties
+    lo, hi = int(tied[0]), int(tied[-1])
+    assert lo > 0
+    _check(ctx, dev, keys, qs, E, sorted({int(cost[i]) + d for i in (lo - 1, lo, (lo + hi) // 2, hi)
+                                          for d in (-1, 0, 1)}))
