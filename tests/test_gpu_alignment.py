@@ -42,6 +42,31 @@ def test_mismatch_of_offset_pairs(ctx, dev, oa):
     assert ctx.mismatch(a, b).cpu().tolist() == want  # the scratch sums start over
 
 
+# Calls of few pairs have their plan with the launch, in two sizes; more pairs
+# have it in the workspace.
+@pytest.mark.parametrize("n", [1, 64, 65, 512, 513, 1500])
+def test_mismatch_of_many_pairs(ctx, dev, n):
+    rnd = np.random.default_rng(n)
+    ha, da = _arena(200000, 11, dev)
+    hb = ha.clone()
+    hb[torch.from_numpy(rnd.integers(0, 200000, 20000))] ^= 0x40
+    db = hb.to(dev)
+    for _ in range(2):  # the scratch sums start over
+        a, b, want = [], [], []
+        for i in range(n):
+            m = 0 if i % 7 == 3 else int(np.exp(rnd.uniform(0, 9.5)))
+            o, extra = int(rnd.integers(0, 150000)), (i % 3) * 5
+            a.append(da[o:o + m])
+            b.append(db[o:o + m + extra])
+            want.append(int((ha[o:o + m] != hb[o:o + m]).sum()) + extra)
+        assert ctx.mismatch(a, b).cpu().tolist() == want
+        shift = [int(x) for x in rnd.integers(0, 16, n)]  # and other offsets of b
+        b = [db[s:s + len(x)] for s, x in zip(shift, a)]
+        want = [int((ha[x.storage_offset():x.storage_offset() + len(x)] != hb[s:s + len(x)]).sum())
+                for s, x in zip(shift, a)]
+        assert ctx.mismatch(a, b).cpu().tolist() == want
+
+
 def _read_flags(spans, ro, rn):
     """1 for each (start, bytes) some read [ro, ro + rn) of at least one byte overlaps."""
     ro, rn = ro[rn > 0], rn[rn > 0]

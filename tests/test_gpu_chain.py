@@ -5,10 +5,11 @@ chain.
 The library launches its kernels so that one may be scheduled while the
 kernel ahead of it on the stream drains, and lets a kernel read its call's
 descriptors before it waits for that kernel.  Every read of data a kernel
-wrote must still come after that kernel: the checkpoint of buffers a restore has just written, the fork of records a checkpoint has just
-finalised, a prune whose queries a restore has just written, and the pack of
-bank rows gathered by the indices the top-k has just chosen.  The results are
-compared with the sources and with the oracle once the chain has finished."""
+wrote must still come after that kernel: the checkpoint of buffers a restore
+has just written, the fork of records a checkpoint has just finalised, a prune
+whose queries a restore has just written, and the pack of bank rows gathered by
+the indices the top-k has just chosen.  The results are compared with the
+sources and with the oracle once the chain has finished."""
 import numpy as np
 import pytest
 import torch
