@@ -3453,7 +3453,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 
 constexpr int kReadStage = 4096;         // buffers staged in shared memory
 constexpr int kReadSlices = 4096;        // slices of the address range at most
-constexpr int kReadThreads = 1024;       // threads of a block, long logs
+constexpr int kReadThreads = 1024;       // threads of a block, long logs or many buffers
 constexpr int kReadIlp = 4;              // reads a thread has in flight
 
 // A block marks the buffers it saw in a shared bitmap, adds it to the call's
@@ -3566,9 +3566,26 @@ __global__ void __launch_bounds__(kReadThreads, 2)
   __syncthreads();
   if (!seen[0]) return;
   __threadfence();
-  for (int i = threadIdx.x; i < P.n_all; i += blockDim.x)
-    flags[fetch<N == 0>(b_orig + i)] =
-        i < P.n ? static_cast<uint8_t>((__ldcg(P.bitmap + (i >> 5)) >> (i & 31)) & 1u) : 0;
+  // Several flags a thread in flight, and 1,024 threads where there are many
+  // (see the launcher): one after the other on 256, 100,000 flags took 107 us.
+  // Kernel time, 1,000 reads of 10,000 / 30,000 / 100,000 buffers 24.4 / 49.9 /
+  // 126 -> 15.3 / 19.7 / 30.3 us.  (All blocks setting the flags of what they
+  // saw instead took 4M reads of 6,000 buffers from 75 to 275 us, now 68.)
+  constexpr int kPer = N > 0 ? 1 : STAGED ? 4 : 8;
+  for (int i0 = threadIdx.x; i0 < P.n_all; i0 += kPer * blockDim.x) {
+    uint32_t to[kPer], word[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int i = i0 + q * static_cast<int>(blockDim.x);
+      to[q] = i < P.n_all ? fetch<N == 0>(b_orig + i) : 0;
+      word[q] = i < P.n ? __ldcg(P.bitmap + (i >> 5)) : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int i = i0 + q * static_cast<int>(blockDim.x);
+      if (i < P.n_all) flags[to[q]] = static_cast<uint8_t>((word[q] >> (i & 31)) & 1u);
+    }
+  }
   if (N > 0) {
     __syncthreads();
     for (int w = threadIdx.x; w < words; w += blockDim.x) P.bitmap[w] = 0;
@@ -4085,7 +4102,7 @@ cudaError_t launch_classify_reads(bool host, ReadPlan p, const uint64_t* addr,
   // block more than it saves (200 buffers, without / with: 500,000 reads 13.8 /
   // 17.6 us, 2M 23.8 / 23.3, 4M 35.3 / 30.9, 16M 106 / 76).
   const bool table = staged && m >= static_cast<int64_t>(sm_count) * 2048 * 8;
-  unsigned threads = 256;
+  unsigned threads = staged ? 256 : kReadThreads;  // (many buffers: one block writes their flags)
   if (table) {
     // Slices of the smallest power of two that cover the buffers' span.
     const uint64_t span = p.top - p.base;

@@ -74,9 +74,9 @@ def _read_flags(spans, ro, rn):
 
 
 # Buffers: one; few and many staged in shared memory; the most staged and one
-# more.  Reads: below and above the line where the address table is used.
+# more; more flags than one round of the block that writes them.  Reads: below and above the line where the address table is used.
 @pytest.mark.parametrize("n,m", [(1, 40), (33, 3_000_001), (600, 2_600_000), (4096, 2_500_000),
-                                 (4096, 5000), (4097, 5000)])
+                                 (4096, 5000), (4097, 5000), (8192, 900), (8193, 5000), (20011, 3000)])
 def test_classify_reads_paths(ctx, dev, n, m):
     rnd = np.random.default_rng(n + m)
     size = 1 << 26
