@@ -3421,9 +3421,20 @@ __global__ void __launch_bounds__(kThreads, 4)
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  for (int i = threadIdx.x; i < n; i += kThreads) {
-    counts[i] = __ldcg(sums + i) + blob.more(i);
-    if (N > 0) sums[i] = 0;
+  // Eight sums a thread in flight (one after the other, 20,000 took 21 us).
+  constexpr int kPer = N > 0 ? 2 : 8;
+  for (int i0 = threadIdx.x; i0 < n; i0 += kPer * kThreads) {
+    unsigned long long v[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) v[q] = i0 + q * kThreads < n ? __ldcg(sums + i0 + q * kThreads) : 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int i = i0 + q * kThreads;
+      if (i < n) {
+        counts[i] = v[q] + blob.more(i);
+        if (N > 0) sums[i] = 0;
+      }
+    }
   }
   if (threadIdx.x == 0) *ticket = 0;
 }

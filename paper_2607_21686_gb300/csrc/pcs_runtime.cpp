@@ -3065,11 +3065,11 @@ pcs_status pcs_mismatch(pcs_ctx* c, const pcs_buf* a, const pcs_buf* b, int32_t 
   if (st) return st;
   c->plan_slot_used = -1;
   if (!sent) {
-    c->plan.assign(total, 0);
-    put(c->plan, 0, pairs);
-    put(c->plan, o_tb, tb);
-    put(c->plan, o_ex, extra);
-    PCS_CUDA(plan_copy(c, ws, total, stream, false));
+    uint8_t* plan = plan_dst(c, total, c->plan);  // straight into a pinned slot
+    put(plan, 0, pairs);
+    put(plan, o_tb, tb);
+    put(plan, o_ex, extra);
+    PCS_CUDA(plan_send(c, ws, total, c->plan, stream, false));
   }
   // Counts start at the bytes only one buffer has.
   if (tiles == 0) {
