@@ -615,12 +615,13 @@ uint8_t* plan_dst(pcs_ctx* c, uint64_t bytes, std::vector<uint8_t>& fallback) {
 // Send descriptors written where plan_dst said into the workspace: by a kernel
 // where they are in a pinned slot and at most kUploadMax, else by a copy.
 // c->uploaded says which, for the launch that follows: it must not be early.
-// One launch that the host bounds is not worth a kernel ahead of it
-// (`by_kernel` false): it costs the host about a microsecond more than the copy
-// (a log against 150 buffers 11.5 -> 12.2 us).  A small call with more
-// descriptors than travel with its launch is not such a one (checkpoint +
-// verified restore + delete, copied / uploaded: 64 sessions of 3 sections 33.2 /
-// 32.8 us, of 8 48.7 / 47.3, of 32 123 / 120, one of 300 100.9 / 99.4).
+// One launch that the host bounds is not worth a kernel ahead of it, nor is a
+// call that waits for its end (`by_kernel` false): the first costs the host about
+// a microsecond more than the copy (a log against 150 buffers 11.5 -> 12.2 us).  A
+// small call with more descriptors than travel with its launch is not such a one
+// (checkpoint + verified restore + delete, copied / uploaded: 64 sessions of 3
+// sections 33.2 / 32.8 us, of 8 48.7 / 47.3, of 32 123 / 120, one of 300 100.9 /
+// 99.4).
 cudaError_t plan_send(pcs_ctx* c, uint8_t* ws, uint64_t bytes,
                       const std::vector<uint8_t>& fallback, cudaStream_t stream,
                       bool by_kernel = true) {
@@ -2514,13 +2515,16 @@ pcs_status pcs_restore(pcs_ctx* c, pcs_snapshot* const* snaps, int32_t n, const 
   st = ws_acquire(c, pr.L.total, stream, &ws);
   if (st) return st;
   c->uploaded = false;
-  if (!pr.in_launch) PCS_CUDA(plan_send(c, ws, pr.L.nodes, pr.plan, stream));
   // verify == 1: count failures of this call in words[1] and wait for them;
-  // verify == 2: accumulate them in words[2] for the next pcs_sync.
+  // verify == 2: accumulate them in words[2] for the next pcs_sync.  A call that
+  // waits has nothing ahead of it for an upload to run beside, and a memset
+  // between its descriptors and its kernels: there a copy is quicker (uploaded /
+  // copied: four contexts of 2 MB 48.7 / 40.1 us, four buffers of 32 MB 90.3 /
+  // 81.8, 300 sessions of 40 kB 57.9 / 55.7).
   uint32_t* words = c->call_words;
-  const bool early = !c->uploaded || verify == 1;  // (after a memset the launch waits anyway)
+  if (!pr.in_launch) PCS_CUDA(plan_send(c, ws, pr.L.nodes, pr.plan, stream, verify != 1));
   if (verify == 1) PCS_CUDA(cudaMemsetAsync(words + 1, 0, 4, stream));
-  PCS_CUDA(launch_prepared(c, pr, ws, words, stream, early));
+  PCS_CUDA(launch_prepared(c, pr, ws, words, stream, !c->uploaded));
   for (int s = 0; s < n; ++s) {
     if (s > 0 && snaps[s]->block == snaps[s - 1]->block) continue;
     st = note_use(c, snaps[s]->block, stream);

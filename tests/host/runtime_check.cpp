@@ -196,7 +196,10 @@ static void check_upload_order() {
         g_ops.clear();
         std::vector<pcs_snapshot*> h(sh.n), k(sh.n);
         NEED(pcs_checkpoint(c, S.s.data(), sh.n, place, h.data(), nullptr) == PCS_OK);
+        const size_t at = g_ops[nullptr].size();
         NEED(pcs_restore(c, h.data(), sh.n, S.s.data(), verify, nullptr) == PCS_OK);
+        for (size_t i = at; i < g_ops[nullptr].size(); ++i)
+          NEED(!(verify == 1 && g_ops[nullptr][i].upload));  // (copied: it waits for its end)
         NEED(pcs_fork_many(c, h.data(), sh.n, k.data(), nullptr) == PCS_OK);
         for (auto& o : g_ops[nullptr]) in_ws |= o.what == "small(ws)";
         const std::string e = upload_order(&uploads);
