@@ -408,6 +408,7 @@ struct pcs_ctx {
   };
   std::unordered_map<cudaStream_t, Workspace> ws;
   Workspace* ws_cur = nullptr;    // of the call in progress (calls hold mu)
+  bool ws_behind = false;         // its last call had not finished when this one began
   uint32_t* call_words = nullptr;  // its header words
   // Context-wide device words: [0] kernel error bits, [2] verify = 2
   // failures until the next pcs_sync, [4] a flag nothing writes (self-test).
@@ -539,6 +540,7 @@ uint32_t* header_words(uint8_t* ws) { return reinterpret_cast<uint32_t*>(ws - kW
 pcs_status ws_acquire(pcs_ctx* c, uint64_t bytes, cudaStream_t stream, uint8_t** out) {
   bytes = round_up(std::max<uint64_t>(bytes, 1), kRecordAlign) + kWsHeader;
   pcs_ctx::Workspace& W = c->ws[stream];
+  c->ws_behind = false;
   if (bytes > W.bytes) {
     if (W.busy) PCS_CUDA(cudaEventSynchronize(W.busy->ev));
     W.busy.reset();
@@ -555,6 +557,7 @@ pcs_status ws_acquire(pcs_ctx* c, uint64_t bytes, cudaStream_t stream, uint8_t**
     PCS_CUDA(cudaMemset(W.buf, 0, kWsHeader));
     W.bytes = want;
   } else if (W.busy && !W.busy->done()) {
+    c->ws_behind = true;
     PCS_CUDA(cudaStreamWaitEvent(stream, W.busy->ev, 0));
   }
   c->ws_cur = &W;
@@ -612,8 +615,16 @@ uint8_t* plan_dst(pcs_ctx* c, uint64_t bytes, std::vector<uint8_t>& fallback) {
   return fallback.data();
 }
 
-// Send descriptors written where plan_dst said into the workspace: by a kernel
-// where they are in a pinned slot and at most kUploadMax, else by a copy.
+// Send descriptors written where plan_dst said into the workspace.  By a kernel
+// where they are in a pinned slot and at most kUploadMax, and the stream's last
+// call has not finished: the kernel is scheduled beside that call's end and
+// spares the stream the two hand-overs to a copy engine and back.  On an idle
+// stream it has nothing to run beside, and the launch after it starts later than
+// after a copy.  Measured over 138 forms of calls of several kernels, geometric
+// means of their times (always copied / always uploaded / by this rule): back to
+// back 0.923 / 0.909 / 0.908 of what they took with copies before descriptors
+// travelled otherwise, each alone 0.934 / 0.983 / 0.937; one context of 2 MB,
+// verified restore: 15.3 / 12.6 / 12.6 and 24.1 / 26.1 / 24.4 us.
 // c->uploaded says which, for the launch that follows: it must not be early.
 // One launch that the host bounds is not worth a kernel ahead of it, nor is a
 // call that waits for its end (`by_kernel` false): the first costs the host about
@@ -625,7 +636,7 @@ uint8_t* plan_dst(pcs_ctx* c, uint64_t bytes, std::vector<uint8_t>& fallback) {
 cudaError_t plan_send(pcs_ctx* c, uint8_t* ws, uint64_t bytes,
                       const std::vector<uint8_t>& fallback, cudaStream_t stream,
                       bool by_kernel = true) {
-  c->uploaded = by_kernel && c->plan_slot_used >= 0 && bytes <= kUploadMax;
+  c->uploaded = by_kernel && c->ws_behind && c->plan_slot_used >= 0 && bytes <= kUploadMax;
   if (c->uploaded) {
     LaunchScope ls(c, kKUpload, stream);
     return launch_upload(ws, c->plan_slot_buf[c->plan_slot_used], bytes, stream);

@@ -1,6 +1,6 @@
 // Checks of the host runtime without a GPU: pcs_runtime.cpp is compiled into
 // this program over a stand-in CUDA runtime (device memory is host memory,
-// nothing runs, every event is done at once) and stand-in kernel launchers,
+// nothing runs, events are done at once or on demand one call late) and stand-in kernel launchers,
 // which keep the order and the arguments of what a call enqueues.
 // Usage: runtime_check <check>; prints "ok" or the first failure.
 #include <cstdlib>
@@ -20,6 +20,8 @@ struct Op {
 };
 static std::map<cudaStream_t, std::vector<Op>> g_ops;
 static std::string g_fail_at;  // a launcher that returns an error
+static bool g_behind = false;  // the event recorded last is not done yet
+static cudaEvent_t g_last_event = nullptr;
 
 static cudaError_t op(cudaStream_t s, const char* what, bool early = false) {
   g_ops[s].push_back({what, false, early});
@@ -43,8 +45,8 @@ cudaError_t cudaHostGetDevicePointer(void** d, void* h, unsigned) { *d = h; retu
 cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = reinterpret_cast<cudaEvent_t>(new int); return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { delete reinterpret_cast<int*>(e); return cudaSuccess; }
-cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) { g_last_event = e; return cudaSuccess; }
+cudaError_t cudaEventQuery(cudaEvent_t e) { return g_behind && e == g_last_event ? cudaErrorNotReady : cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 0; return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
@@ -178,7 +180,9 @@ static std::string upload_order(size_t* uploads) {
   return {};
 }
 
-static void check_upload_order() {
+// Uploads are for calls that find the stream's last one unfinished.
+static void upload_order_of_calls(bool behind) {
+  g_behind = behind;
   pcs_ctx* c = nullptr;
   NEED(pcs_create(0, &c) == PCS_OK);
   size_t uploads = 0;
@@ -250,8 +254,14 @@ static void check_upload_order() {
       }
     }
   }
-  NEED(uploads > 0);
+  NEED((uploads > 0) == behind);
   NEED(pcs_destroy(c) == PCS_OK);
+}
+
+static void check_upload_order() {
+  upload_order_of_calls(true);
+  g_ops.clear();
+  upload_order_of_calls(false);
 }
 
 // A forked child keeps its own section table and no other: a block's tables are

@@ -4,7 +4,8 @@ built here with g++).
 
 upload_order  descriptors written by k_upload are complete before the first
               kernel of the call may read them, over calls of every kind and
-              around the sizes where descriptors stop travelling with a launch
+              around the sizes where descriptors stop travelling with a launch;
+              calls on an idle stream, or that wait for their end, copy them
 fork_tables   a block made by forks keeps the section tables of its own
               snapshots only, in a loop of forks too
 failed_call   the pinned slot of a call that failed half-way is not given back
