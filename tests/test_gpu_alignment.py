@@ -315,3 +315,27 @@ def test_global_threshold_at_launch_shape_edges(ctx, dev, entries, kind):
         assert off.cpu().tolist() == woff.tolist(), budget
         assert np.array_equal(kept.cpu().numpy()[:woff[-1]], want), budget
     ctx.sync()
+
+
+# Top-k with and without the lists' offsets, by banks that travel with the launch
+# and banks in the workspace: empty banks, nothing kept, all kept, ties.
+@pytest.mark.parametrize("n_banks", [1, 60, 61, 300])
+def test_topk_with_and_without_offsets(ctx, dev, n_banks):
+    rnd = np.random.default_rng(n_banks)
+    n = [int(x) for x in rnd.integers(0, 70, n_banks)]
+    n[0] = 5000  # past what a block keeps in registers
+    k = [int(rnd.integers(0, x + 2)) if i % 4 else (0, x)[i % 8 == 0] for i, x in enumerate(n)]
+    k[0] = 1777
+    keys = (rnd.integers(0, 40, sum(n)) / 8).astype(np.float32)
+    dk = torch.from_numpy(keys).to(dev)
+    cuts, want = np.cumsum([0] + n), []
+    kept = [min(a, b) for a, b in zip(n, k)]
+    for a, b, x in zip(cuts[:-1], cuts[1:], kept):
+        want += oracle.topk(keys[a:b], x).tolist()
+    for with_off in (True, False):
+        out = torch.full((sum(kept) + 1,), -7, dtype=torch.int32, device=dev)
+        off = torch.full((n_banks + 1,), -7, dtype=torch.int32, device=dev) if with_off else None
+        ctx.topk(dk, n, k, out, off)
+        assert out.cpu().tolist() == want + [-7]
+        if with_off:
+            assert off.cpu().tolist() == np.cumsum([0] + kept).tolist()
