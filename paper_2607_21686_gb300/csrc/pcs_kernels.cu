@@ -577,8 +577,8 @@ __device__ __forceinline__ void run_stream_tasks(const SecDesc* secs, const Work
   const uint64_t nw = static_cast<uint64_t>(gridDim.x) * kWarps;
   const uint32_t t0 = static_cast<uint32_t>(wl.n_tasks * gw / nw);
   const uint32_t t1 = static_cast<uint32_t>(wl.n_tasks * (gw + 1) / nw);
-  // The work list and the descriptors are the host's: the first task's are
-  // read before waiting for the kernel ahead.
+  // The work list and the descriptors are there before the kernel starts: the
+  // first task's are read before waiting for the kernel ahead.
   const SecDesc& s = sdesc[wib];
   auto load_desc = [&](int j) {
     const SecDesc* src = &secs[fetch<GLOBAL>(wl.ids + j)];
@@ -1043,9 +1043,9 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1)
   const uint32_t t0 = static_cast<uint32_t>(T_all * gw / nw);
   const uint32_t t1 = static_cast<uint32_t>(T_all * (gw + 1) / nw);
   if (t0 >= t1) return;
-  // The work list and the descriptors are the host's, written before the
-  // launch: the first tile's item and section are found while the kernel
-  // ahead on the stream drains.
+  // The work list and the descriptors are there before the kernel starts: the
+  // first tile's item and section are found while the kernel ahead on the
+  // stream drains.
   int item = find_item(wl.begin, 0, wl.n_items, t0, lane);  // item of the next tile to stage
   stage_desc(secs, __ldg(wl.ids + item), sh.st[warp][0], lane);
   grid_dependency();
@@ -1118,8 +1118,8 @@ __global__ void __launch_bounds__(BulkShape<MODE>::kThreads, 1)
   const uint32_t t1 = static_cast<uint32_t>(T_static * (gw + 1) / nw);
   uint32_t next = t0, chunk_end = t1;  // tiles [next, chunk_end) are this warp's
   int item = find_item(wl.begin, 0, wl.n_items, t0, lane);  // item of the last tile taken
-  // The work list and the descriptors are the host's: the first static
-  // tile's section is read before waiting for the kernel ahead.  The
+  // The work list and the descriptors are there before the kernel starts: the
+  // first static tile's section is read before waiting for the kernel ahead.  The
   // counters in `sched` are touched only after the wait.
   if (t0 < t1) stage_desc(secs, __ldg(wl.ids + item), sh.st[warp][0], lane);
   grid_dependency();
@@ -1443,7 +1443,7 @@ __global__ void __launch_bounds__(512)
 
 // A session of at most 32 sections, finalised by one warp (lane j keeps
 // section j's fp): the same outputs as finalize_sessions_block.  Lane j's part
-// of the session's descriptors (the host's):
+// of the session's descriptors:
 struct SessLane {
   uint32_t fin_begin, fin_count;  // section j's nodes
   uint64_t bytes;                 // and its length
@@ -2967,7 +2967,7 @@ __global__ void __launch_bounds__(kGsThreads, 1)
   __shared__ uint32_t scan32[32];
   __shared__ uint32_t s_prefix;
   __shared__ uint64_t s_left;
-  // The bank descriptors are the host's.
+  // The bank descriptors are there before the kernel starts.
   for (int b = threadIdx.x; b < n_banks; b += kGsThreads) {
     s_beg[b] = static_cast<uint32_t>(banks[b].entry_begin);
     if (!UNIFORM) s_bytes[b] = banks[b].entry_bytes;

@@ -1195,7 +1195,6 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
   if (n < 0 || (n > 0 && !bufs)) return fail(PCS_E_INVAL, "bad buffer list");
   if (n == 0) return PCS_OK;
   SecVec& d = sec_array(c, n);
-  uint64_t chunks = 0;
   for (int i = 0; i < n; ++i) {
     if (bufs[i].bytes > 0 && !bufs[i].ptr) return fail(PCS_E_INVAL, "buffer %d: null pointer", i);
     pcs_section s{};
@@ -1203,9 +1202,7 @@ pcs_status fingerprint_impl(pcs_ctx* c, const pcs_buf* bufs, int32_t n, uint64_t
     s.base = const_cast<void*>(bufs[i].ptr);
     s.bytes = bufs[i].bytes;
     make_desc(d[i], s, nullptr, 0, 0);
-    chunks += d[i].n_chunks;
   }
-  (void)chunks;
   PtrCache cache;
   std::vector<char> bulk(n);
   const bool small = total_bytes(d) <= kSmallCallBytes;
