@@ -149,12 +149,9 @@ struct Slab {
 // A call's section tables, kept by every block whose snapshots point into them
 // (one count per block, not per snapshot).
 using Tables = std::shared_ptr<const std::vector<Entry>>;
-
-struct TablesBefore {
-  bool operator()(const Tables& a, const std::vector<Entry>* b) const {
-    return std::less<const std::vector<Entry>*>()(a.get(), b);
-  }
-};
+bool starts_before(const Tables& a, const Tables& b) {
+  return std::less<const Entry*>()(a->data(), b->data());
+}
 
 struct Block {
   Slab* slab = nullptr;
@@ -163,7 +160,7 @@ struct Block {
   uint8_t* ptr = nullptr;
   uint32_t placement = PCS_PLACE_DEVICE;
   int refs = 0;
-  std::vector<Tables> tables;                 // section tables of its snapshots, by address
+  std::vector<Tables> tables;                 // section tables of its snapshots (starts_before)
   Ev written;                                 // completion of the write
   std::map<cudaStream_t, Ev> uses;            // latest use per stream
 };
@@ -349,7 +346,6 @@ struct pcs_snapshot {
   uint32_t kind = 0;
   // Host copy of the section table (fp = 0): n_sections entries, in an array
   // that the block keeps (shared by the snapshots of one call and their forks).
-  const std::vector<Entry>* tables = nullptr;
   const Entry* entries = nullptr;
   uint32_t n_sections = 0;
   const Entry* table() const { return entries; }
@@ -1468,7 +1464,6 @@ pcs_status build_checkpoint(pcs_ctx* c, const pcs_session* sessions, int32_t n, 
     h->payload_start = pstart[s];
     h->session_id = S.session_id;
     h->kind = S.kind;
-    h->tables = &ent;
     h->entries = ent.data() + ent.size();  // (reserved above: the array does not move)
     h->n_sections = static_cast<uint32_t>(S.n_sections);
     sd[s].record = rec;
@@ -2470,14 +2465,18 @@ pcs_status pcs_fork_many(pcs_ctx* c, pcs_snapshot* const* parents, int32_t n,
     // The tables the children point into, not all that their parents' blocks
     // hold: in a loop of forks those would add up.
     auto& t = blk[pl]->tables;
+    const std::less<const Entry*> before;
     for (int i = 0; i < n; ++i) {
       const Block* from = parents[i]->block;
+      const Entry* e = parents[i]->entries;
       if (from->placement != static_cast<uint32_t>(pl)) continue;
-      if (!t.empty() && t.back().get() == parents[i]->tables) continue;
-      t.push_back(*std::lower_bound(from->tables.begin(), from->tables.end(), parents[i]->tables,
-                                    TablesBefore()));
+      if (!t.empty() && !before(e, t.back()->data()) && before(e, t.back()->data() + t.back()->size()))
+        continue;  // the parent before it has the same
+      t.push_back(*std::prev(std::upper_bound(
+          from->tables.begin(), from->tables.end(), e,
+          [&](const Entry* x, const Tables& y) { return before(x, y->data()); })));
     }
-    std::sort(t.begin(), t.end());
+    std::sort(t.begin(), t.end(), starts_before);
     t.erase(std::unique(t.begin(), t.end()), t.end());
   }
   c->live.reserve(n);
@@ -2892,8 +2891,7 @@ pcs_status pcs_snapshot_read_file(pcs_ctx* c, const char* path, uint32_t placeme
   for (auto& e : table) e.fp = 0;
   h->n_sections = static_cast<uint32_t>(table.size());
   blk->tables.push_back(std::make_shared<const std::vector<Entry>>(std::move(table)));
-  h->tables = blk->tables.back().get();
-  h->entries = h->tables->data();
+  h->entries = blk->tables.back()->data();
   *out = h.release();
   c->live.insert(*out);
   return PCS_OK;
