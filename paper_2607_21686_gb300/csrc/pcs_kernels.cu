@@ -3460,7 +3460,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 // none or one for most reads.  Each thread has four reads in flight.
 // Measured (calls back to back; two binary searches and a read at a time ->
 // this): 16M reads against 10 / 200 / 2,000 / 6,000 buffers 122 -> 62, 263 -> 76,
-// 332 -> 88, 665 -> 225 us (the last not staged); 100,000 reads against 200
+// 332 -> 88, 665 -> 206 us (the last not staged); 100,000 reads against 200
 // buffers 30 -> 11 us.  The log alone takes 40 us at 16M reads; address
 // arithmetic and the wavefronts of three to four lookups a read are the rest.
 // ---------------------------------------------------------------------------
